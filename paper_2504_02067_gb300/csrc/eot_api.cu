@@ -2,6 +2,7 @@
 // FP32 (mixed / plain) and FP64 solver instantiations, error capture.
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "plan_int.cuh"
 #include "solver.cuh"
@@ -171,21 +172,58 @@ void run_plan_int(eot_handle h, const eot_problem* P, const double* u, const dou
                   double log_tau, int64_t* idx_out, int64_t* counts, int64_t* total, cudaStream_t st) {
   unsigned long long* tot = reinterpret_cast<unsigned long long*>(total);
   if (tot) EOT_CUDA(cudaMemsetAsync(tot, 0, sizeof(unsigned long long), st));
+  // the FP32 screening kernels, unless the temperature leaves their bound's reach
   const dim3 grid((unsigned)((P->n + pint::kWarps - 1) / pint::kWarps));
+  auto in_reach = [](double g) { return g == 0.0 || (g >= 1e-30 && g <= 1e30); };
+  auto screen = [](double g, float c, int terms) {
+    return pint::Screen{(float)g, 3.0f * c, 1e-30f + (float)(g * terms * 1e-44)};
+  };
   if (P->kind == EOT_COST_SQEUCLID_POINTS) {
     double sC = P->cost_scale;
     if (!(sC > 0.0)) {
       Solver<double> S(h, P, st);  // computes s_C = 1 / max |x_i - y_j|^2 as the solver does
       sC = S.sC;
     }
-    launch_k(pint::plan_int_points_kernel<MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (int)P->d, P->X, P->Y,
-             sC, u, v, gamma, log_tau, idx_out, counts, tot);
-  } else if (P->kind == EOT_COST_DENSE_F64) {
-    launch_k(pint::plan_int_dense_kernel<double, MODE>, grid, dim3(pint::kThreads), st, P->n, P->m,
-             (const double*)P->C, P->ldc, u, v, gamma, log_tau, idx_out, counts, tot);
+    const double K = gamma * sC;
+    if (in_reach(K) && P->m < ((int64_t)1 << 31)) {
+      // Chunks of columns per cluster: the fewest waves x (tiles per CTA + 2, its fixed
+      // cost: the rows' coordinates, V, the contenders' FP64 exponents), two CTAs per SM.
+      // At n = m = 8192, d = 64, 2 chunks (one wave of 256 CTAs) against 3 (384 CTAs, the
+      // second wave a quarter full): 0.474 and 0.480 ms per call.
+      const int64_t B = (P->n + pint::kSR - 1) / pint::kSR, tiles = (P->m + pint::kSC - 1) / pint::kSC;
+      int64_t S = 1, chunk = 0, best = -1;
+      for (int64_t k = 1; k <= 8 && k <= tiles; ++k) {
+        const int64_t tk = (tiles + k - 1) / k, Sk = (tiles + tk - 1) / tk;
+        const int64_t waves = (B * Sk + 2 * h->sms - 1) / (2 * h->sms), cost = waves * (tk + 2);
+        if (best >= 0 && cost >= best) continue;
+        best = cost;
+        S = Sk;
+        chunk = tk * pint::kSC;
+      }
+      launch_kc(pint::plan_screen_points_kernel<MODE>, dim3((unsigned)B, (unsigned)S), dim3(pint::kThreads),
+                (unsigned)S, st, P->n, P->m, (int)P->d, P->X, P->Y, sC, u, v, gamma, log_tau,
+                screen(K, (float)(P->d + 12) * 5.9604645e-8f, (int)P->d), chunk, idx_out, counts, tot);
+    } else {
+      launch_k(pint::plan_int_points_kernel<MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (int)P->d, P->X, P->Y,
+               sC, u, v, gamma, log_tau, idx_out, counts, tot);
+    }
   } else {
-    launch_k(pint::plan_int_dense_kernel<float, MODE>, grid, dim3(pint::kThreads), st, P->n, P->m,
-             (const float*)P->C, P->ldc, u, v, gamma, log_tau, idx_out, counts, tot);
+    auto dense = [&](auto* C, float c) {
+      using T = std::remove_cv_t<std::remove_pointer_t<decltype(C)>>;
+      constexpr int VEC = 16 / (int)sizeof(T);
+      const bool vec = ((uintptr_t)C % 16) == 0 && P->m % VEC == 0 && P->ldc % VEC == 0;
+      if (!in_reach(gamma))
+        launch_k(pint::plan_int_dense_kernel<T, MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (const T*)C, P->ldc,
+                 u, v, gamma, log_tau, idx_out, counts, tot);
+      else if (vec)
+        launch_k(pint::plan_screen_dense_kernel<T, VEC, MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (const T*)C,
+                 P->ldc, u, v, gamma, log_tau, screen(gamma, c, 1), idx_out, counts, tot);
+      else
+        launch_k(pint::plan_screen_dense_kernel<T, 1, MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (const T*)C,
+                 P->ldc, u, v, gamma, log_tau, screen(gamma, c, 1), idx_out, counts, tot);
+    };
+    if (P->kind == EOT_COST_DENSE_F64) dense((const double*)P->C, 4.7683716e-7f);
+    else dense((const float*)P->C, 2.3841858e-7f);
   }
   EOT_LAUNCH_CHECK();
   h->launches++;
