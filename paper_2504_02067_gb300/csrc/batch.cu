@@ -99,6 +99,7 @@ struct Smem {
   int status;
   int fail;
   int prob;
+  __align__(16) ExpSmem<T> ex;
 };
 
 struct Grp {
@@ -419,7 +420,7 @@ struct Dev {
             T Dh, Dl;
             dist2<PRECISE, T, kDmax>(xr[r], [&](int k) { return yq[k]; }, Dh, Dl);
             if constexpr (!LSE) {
-              const T ex = expT(expo<PRECISE>(h[r] + hb, Kh, Kl, Dh, Dl));
+              const T ex = s.ex(expo<PRECISE>(h[r] + hb, Kh, Kl, Dh, Dl));
 #pragma unroll
               for (int k = 0; k < NR; ++k) {
                 if ((SQM >> k) & 1) acc[r][k] = fmaT(ex * ex, wq[k], acc[r][k]);
@@ -432,17 +433,17 @@ struct Dev {
                 mx_set[r] = true;
               }
               T t = expo<PRECISE>(hm[r] + hb, Kh, Kl, Dh, Dl);
-              for (int k = 0; k < 4 && t > T(kTheta); ++k) {  // raise the max, at most 4 steps
+              for (int k = 0; k < 4 && maybe_above(t, T(kTheta)) && t > T(kTheta); ++k) {  // raise the max, at most 4 steps
                 const T dlt = ceil_grid(t);
                 mx[r] += dlt;
                 hm[r] = h[r] - mx[r];
-                const T f = expT(-dlt);
+                const T f = s.ex(-dlt);
                 acc[r][0] *= f;
                 Sa[r][0] *= f;
                 Ca[r][0] *= f;
                 t = expo<PRECISE>(hm[r] + hb, Kh, Kl, Dh, Dl);
               }
-              acc[r][0] = fmaT(expT(t), wq[0], acc[r][0]);
+              acc[r][0] = fmaT(s.ex(t), wq[0], acc[r][0]);
             }
           }
         }
@@ -935,6 +936,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) batch_kernel
   gp.ipart = L.ipart + (size_t)gp.g * 2 * L.G;
   gp.rcount = 0;
   gp.abort = L.abort;
+  s.ex.fill();
   if (threadIdx.x == 0) {
     s.fail = 0;
     s.status = 0;

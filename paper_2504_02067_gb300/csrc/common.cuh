@@ -13,6 +13,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "exp64.cuh"
+
 namespace eot {
 
 constexpr int kWarps = 8;            // warps per CTA of every sweep kernel
@@ -53,9 +55,28 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// exp in the element type: FP32 via the MUFU ex2 unit, FP64 via the libm exp.
+// exp in the element type: FP32 via the MUFU ex2 unit, FP64 via exp64 and its table,
+// which a kernel that needs it keeps in shared memory (ExpSmem; fill() by all
+// threads, then a barrier before the first use).
 __device__ __forceinline__ float expT(float t) { return ex2_approx(t * kLog2e); }
-__device__ __forceinline__ double expT(double t) { return exp(t); }
+template <class T>
+struct ExpSmem {
+  __device__ __forceinline__ void fill() {}
+  __device__ __forceinline__ T operator()(T t) const { return expT(t); }
+};
+template <>
+struct ExpSmem<double> {
+  ExpTable tab;
+  __device__ __forceinline__ void fill() { exp_fill(tab); }
+  __device__ __forceinline__ double operator()(double t) const { return exp64(t, tab); }
+};
+
+// t > kTheta as a screen on the integer pipes for FP64 (a comparison would take the
+// FP64 pipe): false only if t <= kTheta; the caller compares again before acting.
+__device__ __forceinline__ bool maybe_above(float t, float theta) { return t > theta; }
+__device__ __forceinline__ bool maybe_above(double t, double theta) {
+  return __double2hiint(t) >= __double2hiint(theta);  // theta > 0
+}
 
 __device__ __forceinline__ float fmaT(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fmaT(double a, double b, double c) { return fma(a, b, c); }
@@ -248,21 +269,23 @@ struct LsePair {
 // Combine two pairs. The scaling factor exp(m - M) is formed in the element type
 // T: one FP32 rounding is far below the FP32 path's own error, and it keeps the
 // FP64 pipe free; the FP64 path scales in FP64.
-template <class T = double>
-__device__ __forceinline__ LsePair lse_combine(LsePair a, LsePair b) {
+template <class T>
+__device__ __forceinline__ LsePair lse_combine(LsePair a, LsePair b, const ExpSmem<T>& ex) {
   if (b.s == 0.0) return a;
   if (a.s == 0.0) return b;
   const double M = fmax(a.m, b.m);
-  return {M, a.s * (double)expT((T)(a.m - M)) + b.s * (double)expT((T)(b.m - M))};
+  return {M, a.s * (double)ex((T)(a.m - M)) + b.s * (double)ex((T)(b.m - M))};
 }
-template <class T = double>
-__device__ __forceinline__ LsePair warp_lse(LsePair p) {
+// FP64 pairs of a warp: their common maximum first, then one scaled sum (a pairwise
+// tree would take ten exponentials per lane instead of one).
+__device__ __forceinline__ LsePair warp_lse(LsePair p, const ExpSmem<double>& ex) {
+  double M = p.s != 0.0 ? p.m : -INFINITY;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    LsePair q{__shfl_xor_sync(0xffffffffu, p.m, o), __shfl_xor_sync(0xffffffffu, p.s, o)};
-    p = lse_combine<T>(p, q);
-  }
-  return p;
+  for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
+  double s = p.s != 0.0 ? p.s * ex(p.m - M) : 0.0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return {M == -INFINITY ? 0.0 : M, s};
 }
 
 __device__ __forceinline__ float warp_sum_f(float x) {

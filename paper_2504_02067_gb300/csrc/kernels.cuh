@@ -1049,6 +1049,9 @@ template <class T>
 __global__ void plan_dense_kernel(int64_t n, int64_t m, const T* C, int64_t ldc, const T* Ah,
                                   const T* Bh, const double* gamma_dev, const double* rowfac,
                                   const double* colfac, double scale, float* out, int64_t ldo) {
+  __shared__ __align__(16) ExpSmem<T> ex;
+  ex.fill();
+  if constexpr (sizeof(T) == 8) __syncthreads();
   pdl_wait();
   const T g = (T)*gamma_dev;
   const int64_t total = n * m;
@@ -1056,7 +1059,7 @@ __global__ void plan_dense_kernel(int64_t n, int64_t m, const T* C, int64_t ldc,
        k += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = k / m, j = k - i * m;
     const T t = fmaT(-g, C[i * ldc + j], Ah[i] + Bh[j]);
-    out[i * ldo + j] = (float)(scale * rowfac[i] * colfac[j] * (double)expT(t));
+    out[i * ldo + j] = (float)(scale * rowfac[i] * colfac[j] * (double)ex(t));
   }
 }
 

@@ -178,13 +178,6 @@ __device__ __forceinline__ float max_nan(float a, float b) {
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
-// (double)x on the integer pipes (exact; zeros, subnormals and non-finite values
-// take the conversion instruction)
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
-  if (e - 0x00800000u >= 0x7f000000u) return (double)x;
-  return __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
-}
 // |v_j| as it enters V: -inf (a column without mass, or below FP32's range: never
 // the answer) counts 0; NaN, +inf and what is above FP32's range make V infinite
 __device__ __forceinline__ float bound_of(float vf) {

@@ -238,7 +238,8 @@ __device__ __forceinline__ void row_load(const T* crow, int j0, int tw, T (&c)[U
 
 template <class T, int V, int U, int NR, int SQM, int NV, int TW>
 __device__ __forceinline__ void row_reduce_sum(const T (&c)[U][V], int j0, int tw, T ah, T g,
-                                               const T (&sv)[NV][TW], T (&S)[NR], T (&Cc)[NR]) {
+                                               const T (&sv)[NV][TW], T (&S)[NR], T (&Cc)[NR],
+                                               const ExpSmem<T>& ex) {
   T acc[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) acc[k] = T(0);
@@ -252,7 +253,7 @@ __device__ __forceinline__ void row_reduce_sum(const T (&c)[U][V], int j0, int t
     for (int k = 0; k < NR; ++k) ld_vec_smem<V>(&sv[1 + k][jl], w[k]);
 #pragma unroll
     for (int e = 0; e < V; ++e) {
-      const T x = expT(fmaT(-g, c[u][e], ah + b[e]));
+      const T x = ex(fmaT(-g, c[u][e], ah + b[e]));
 #pragma unroll
       for (int k = 0; k < NR; ++k) {
         if ((SQM >> k) & 1) acc[k] = fmaT(x * x, w[k][e], acc[k]);
@@ -271,7 +272,8 @@ __device__ __forceinline__ void row_reduce_sum(const T (&c)[U][V], int j0, int t
 // non-finite sum).
 template <class T, int V, int U, int NV, int TW>
 __device__ __forceinline__ void row_reduce_lse(const T (&c)[U][V], int j0, int tw, T ah, T g,
-                                               const T (&sv)[NV][TW], T& mx, T& am, T& S, T& Cc) {
+                                               const T (&sv)[NV][TW], T& mx, T& am, T& S, T& Cc,
+                                               const ExpSmem<T>& ex) {
   T acc = T(0);
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -281,16 +283,24 @@ __device__ __forceinline__ void row_reduce_lse(const T (&c)[U][V], int j0, int t
     ld_vec_smem<V>(&sv[0][jl], b);
     ld_vec_smem<V>(&sv[1][jl], w);
     T tmax = T(-3.0e38);
+    bool over = sizeof(T) == 4;  // FP64: the maximum is formed only if a t may exceed theta
 #pragma unroll
     for (int e = 0; e < V; ++e) {
       t[e] = fmaT(-g, c[u][e], am + b[e]);
-      tmax = fmax(tmax, t[e]);
+      if constexpr (sizeof(T) == 4) tmax = fmax(tmax, t[e]);
+      else over |= maybe_above(t[e], T(kTheta));
+    }
+    if constexpr (sizeof(T) == 8) {
+      if (over) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) tmax = fmax(tmax, t[e]);
+      }
     }
     for (int k = 0; k < 4 && tmax > T(kTheta); ++k) {
       const T dlt = ceil_grid(tmax);
       mx += dlt;
       am = ah - mx;
-      const T f = expT(-dlt);
+      const T f = ex(-dlt);
       acc *= f;
       S *= f;
       Cc *= f;
@@ -302,21 +312,24 @@ __device__ __forceinline__ void row_reduce_lse(const T (&c)[U][V], int j0, int t
       }
     }
 #pragma unroll
-    for (int e = 0; e < V; ++e) acc = fmaT(expT(t[e]), w[e], acc);
+    for (int e = 0; e < V; ++e) acc = fmaT(ex(t[e]), w[e], acc);
   }
   kadd(S, Cc, acc);
 }
 
 template <class T, int V, int NR, bool LSE, int SQM, class Epi>
-__global__ void __launch_bounds__(kThreads, 4) row_sweep_kernel(SweepArgs<T> a, Epi epi) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) row_sweep_kernel(SweepArgs<T> a, Epi epi) {
   constexpr int U = 4;                               // chunks per batch (two batches in flight)
   constexpr int NV = 1 + (LSE ? 1 : NR);             // staged column vectors
-  // tile width (<= 32 KB smem), a multiple of 128 so that tiles and rows of sv stay 16-byte aligned
-  constexpr int TW = ((sizeof(T) == 4 ? 8192 : 4096) / NV) / 128 * 128;
+  // tile width (<= 32 KB smem; FP64: 24 KB beside the exponential's table), a multiple of
+  // 128 so that tiles and rows of sv stay 16-byte aligned
+  constexpr int TW = ((sizeof(T) == 4 ? 8192 : 3072) / NV) / 128 * 128;
   constexpr int ND = Epi::kDot;
   constexpr int NA = LSE ? 1 : NR;
   constexpr int STEP = 32 * V * U;
   __shared__ __align__(16) T sv[NV][TW];
+  __shared__ __align__(16) ExpSmem<T> ex;
+  ex.fill();  // (visible after the first tile's barrier)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * kWarps + warp;
   const bool rv = i < a.n;
@@ -389,13 +402,13 @@ __global__ void __launch_bounds__(kThreads, 4) row_sweep_kernel(SweepArgs<T> a, 
     for (;;) {
       const int j1 = j0 + STEP;
       if (j1 < tw) row_load<T, V, U>(ct, j1, tw, cB, pol);
-      if constexpr (!LSE) row_reduce_sum<T, V, U, NR, SQM, NV, TW>(cA, j0, tw, ah, g, sv, S, Cc);
-      else row_reduce_lse<T, V, U, NV, TW>(cA, j0, tw, ah, g, sv, mx, am, S[0], Cc[0]);
+      if constexpr (!LSE) row_reduce_sum<T, V, U, NR, SQM, NV, TW>(cA, j0, tw, ah, g, sv, S, Cc, ex);
+      else row_reduce_lse<T, V, U, NV, TW>(cA, j0, tw, ah, g, sv, mx, am, S[0], Cc[0], ex);
       if (j1 >= tw) break;
       const int j2 = j1 + STEP;
       if (j2 < tw) row_load<T, V, U>(ct, j2, tw, cA, pol);
-      if constexpr (!LSE) row_reduce_sum<T, V, U, NR, SQM, NV, TW>(cB, j1, tw, ah, g, sv, S, Cc);
-      else row_reduce_lse<T, V, U, NV, TW>(cB, j1, tw, ah, g, sv, mx, am, S[0], Cc[0]);
+      if constexpr (!LSE) row_reduce_sum<T, V, U, NR, SQM, NV, TW>(cB, j1, tw, ah, g, sv, S, Cc, ex);
+      else row_reduce_lse<T, V, U, NV, TW>(cB, j1, tw, ah, g, sv, mx, am, S[0], Cc[0], ex);
       if (j2 >= tw) break;
       j0 = j2;
     }
@@ -417,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, 4) row_sweep_kernel(SweepArgs<T> a, 
         }
       } else {
         LsePair p{mx_set ? (double)mx : 0.0, (double)S[0] + (double)Cc[0]};
-        p = warp_lse<T>(p);
+        p = warp_lse(p, ex);
         if (lane == 0) {
           DotArr<ND> d;
           epi.row_lse(i, p.m, p.s, d.v);
@@ -462,15 +475,18 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
   const int64_t r1 = min(a.n, r0 + (int64_t)a.rows_per_block);
   // the first batch of (immutable) cost rows is in flight before the wait
   const uint64_t pol = cost_policy(a.keep_l2);
+  __shared__ __align__(16) ExpSmem<T> ex;
   T cA[U][V], cB[U][V];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int64_t i = r0 + warp + (int64_t)u * kWarps;
     if (i < r1 && jv) ld_stream(a.C + i * a.ldc + j, cA[u], pol);
   }
+  ex.fill();
   pdl_wait();
   if (a.active && *a.active == 0.0) return;
   if constexpr (HasPrefetch<Epi>::value) epi.begin(strip * SW, SW, a.m);
+  if constexpr (sizeof(T) == 8) __syncthreads();  // the exponential's table is complete
   const T g = a.gamma_dev ? (T)*a.gamma_dev : a.gamma;
 
   T b[V], wcv[2][V];
@@ -526,16 +542,28 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
         for (int e = 0; e < V; ++e) {
           T t[U];
           T tmax = T(-3.0e38);
+          bool over = false;
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             t[u] = fmaT(-g, c[u][e], hh[u] + bm[e]);
-            if (i0 + (int64_t)u * kWarps < r1) tmax = fmax(tmax, t[u]);
+            if constexpr (sizeof(T) == 4) {
+              if (i0 + (int64_t)u * kWarps < r1) tmax = fmax(tmax, t[u]);
+            } else {
+              over |= i0 + (int64_t)u * kWarps < r1 && maybe_above(t[u], T(kTheta));
+            }
+          }
+          if constexpr (sizeof(T) == 8) {
+            if (over) {
+#pragma unroll
+              for (int u = 0; u < U; ++u)
+                if (i0 + (int64_t)u * kWarps < r1) tmax = fmax(tmax, t[u]);
+            }
           }
           for (int k = 0; k < 4 && tmax > T(kTheta); ++k) {
             const T dlt = ceil_grid(tmax);
             mx[e] += dlt;
             bm[e] = b[e] - mx[e];
-            const T f = expT(-dlt);
+            const T f = ex(-dlt);
             tot[1][e] *= f;
             cmp[1][e] *= f;
             tmax = T(-3.0e38);
@@ -547,7 +575,7 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
           }
 #pragma unroll
           for (int u = 0; u < U; ++u)
-            if (i0 + (int64_t)u * kWarps < r1) acc[1][e] = fmaT(expT(t[u]), xx[0][u], acc[1][e]);
+            if (i0 + (int64_t)u * kWarps < r1) acc[1][e] = fmaT(ex(t[u]), xx[0][u], acc[1][e]);
         }
       }
     } else {
@@ -559,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
       for (int e = 0; e < V; ++e) {
         if constexpr (!LSE) {
           const T t = fmaT(-g, c[u][e], hh[u] + b[e]);
-          const T x = jv ? expT(t) : T(0);
+          const T x = jv ? ex(t) : T(0);
           acc[0][e] = fmaT(x, xx[0][u], acc[0][e]);
           if constexpr (NC > 1) acc[1][e] = fmaT(x, xx[1][u], acc[1][e]);
           if constexpr (NR > 0) racc0 = fmaT(x, wcv[0][e], racc0);
@@ -691,7 +719,7 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
         }
       } else {
         LsePair p{0.0, 0.0};
-        for (int w = 0; w < kWarps; ++w) p = lse_combine<T>(p, LsePair{smax[w][cc], sred[1][w][cc]});
+        for (int w = 0; w < kWarps; ++w) p = lse_combine<T>(p, LsePair{smax[w][cc], sred[1][w][cc]}, ex);
         a.colpart[((int64_t)0 * R + rb) * a.m + jj] = p.m;
         a.colpart[((int64_t)1 * R + rb) * a.m + jj] = p.s;
       }
@@ -758,7 +786,7 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
       } else {
         LsePair p{0.0, 0.0};
         ordered_loads2(a.colpart + jj, a.colpart + (int64_t)R * a.m + jj, a.m, R,
-                       [&](double qm, double qs) { p = lse_combine<T>(p, LsePair{qm, qs}); });
+                       [&](double qm, double qs) { p = lse_combine<T>(p, LsePair{qm, qs}, ex); });
         epi.col_lse(jj, p.m, p.s, d.v);
       }
 #pragma unroll

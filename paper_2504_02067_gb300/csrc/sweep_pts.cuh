@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(kThreads, 2) pts_sweep_kernel(SweepArgs<T> a, 
   __shared__ T sy[DMAX][TO];
   __shared__ T sh[TO];
   __shared__ T sw[NW][TO];
+  __shared__ __align__(16) ExpSmem<T> ex_;
   __shared__ int last_blk;
+  ex_.fill();  // (visible after the first tile's barrier)
 
   const int64_t n_own = ROWS ? a.n : a.m, n_oth = ROWS ? a.m : a.n;
   const float* xo = ROWS ? a.X : a.Y;
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(kThreads, 2) pts_sweep_kernel(SweepArgs<T> a, 
         dist2<PRECISE, T, DMAX>(x[r], [&](int k) { if constexpr (YREG) return y[k]; else return sy[k][q]; },
                                 Dh, Dl);
         if constexpr (!LSE) {
-          const T ex = expT(expo<PRECISE>(h[r] + hb, Kh, Kl, Dh, Dl));
+          const T ex = ex_(expo<PRECISE>(h[r] + hb, Kh, Kl, Dh, Dl));
 #pragma unroll
           for (int k = 0; k < NR; ++k) {
             if ((SQM >> k) & 1) acc[r][k] = fmaT(ex * ex, w[k], acc[r][k]);
@@ -179,17 +181,17 @@ __global__ void __launch_bounds__(kThreads, 2) pts_sweep_kernel(SweepArgs<T> a, 
             mx_set[r] = true;
           }
           T t = expo<PRECISE>(hm[r] + hb, Kh, Kl, Dh, Dl);
-          for (int k = 0; k < 4 && t > T(kTheta); ++k) {  // raise the max, at most 4 steps
+          for (int k = 0; k < 4 && maybe_above(t, T(kTheta)) && t > T(kTheta); ++k) {  // raise the max, at most 4 steps
             const T dlt = ceil_grid(t);
             mx[r] += dlt;
             hm[r] = h[r] - mx[r];
-            const T f = expT(-dlt);
+            const T f = ex_(-dlt);
             acc[r][0] *= f;
             Sa[r][0] *= f;
             Ca[r][0] *= f;
             t = expo<PRECISE>(hm[r] + hb, Kh, Kl, Dh, Dl);
           }
-          acc[r][0] = fmaT(expT(t), w[0], acc[r][0]);
+          acc[r][0] = fmaT(ex_(t), w[0], acc[r][0]);
         }
       }
     }
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 2) pts_sweep_kernel(SweepArgs<T> a, 
     } else {
       LsePair p{0.0, 0.0};
       ordered_loads2(a.rowpart + e[r], a.rowpart + S * n_own + e[r], n_own, S,
-                     [&](double qm, double qs) { p = lse_combine<T>(p, LsePair{qm, qs}); });
+                     [&](double qm, double qs) { p = lse_combine<T>(p, LsePair{qm, qs}, ex_); });
       if constexpr (ROWS) epi.row_lse(e[r], p.m, p.s, dd.v);
       else epi.col_lse(e[r], p.m, p.s, dd.v);
     }
@@ -273,7 +275,9 @@ __global__ void __launch_bounds__(kThreads, DMAX > 16 ? 1 : 2)
   __shared__ T sy[DMAX][TO];
   __shared__ T sh[TO];
   __shared__ T sw[TO];
+  __shared__ __align__(16) ExpSmem<T> ex_;
   __shared__ int last_blk;
+  ex_.fill();  // (visible after the first tile's barrier)
 
   const int64_t n_own = ROWS ? a.n : a.m, n_oth = ROWS ? a.m : a.n;
   const float* xo = ROWS ? a.X : a.Y;
@@ -320,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, DMAX > 16 ? 1 : 2)
       for (int q = q0; q < q1; ++q) {
         T Dh, Dl;
         dist2<PRECISE, T, DMAX>(x, [&](int k) { return sy[k][q]; }, Dh, Dl);
-        const T pw = expT(expo<PRECISE>(h + sh[q], Kh, Kl, Dh, Dl)) * sw[q];
+        const T pw = ex_(expo<PRECISE>(h + sh[q], Kh, Kl, Dh, Dl)) * sw[q];
 #pragma unroll
         for (int k = 0; k < DG; ++k) acc[k] = fmaT(pw, xg[k] - sy[k0 + k][q], acc[k]);
       }
