@@ -11,9 +11,11 @@
 // table-driven scheme of P. T. P. Tang, ACM TOMS 15, 1989, with the Taylor
 // polynomial of 2^x). About 55 integer instructions, 14 of them multiplies.
 // Against 200-bit arithmetic: largest error 0.81 ulp for |t| < 40 and 1.27 ulp up
-// to |t| = 708, rms 0.30 ulp (perfect rounding: 0.289).
-// Measured (FP64, before -> after): solve of the 28 x 28 grid 76.3 -> 50.9 ms, its
-// marginals 264 -> 190 us, the Hessian-vector product at 1501 x 1999 755 -> 570 us.
+// to |t| = 708.39, rms 0.30 ulp (perfect rounding: 0.289).
+// Measured (FP64, CUDA's exp -> this one): solve of the 28 x 28 grid 75.1 -> 29.9 ms,
+// its marginals 267 -> 153 us, the Hessian-vector product at 1501 x 1999 763 -> 379 us,
+// Round of the 64 x 64 grid 2.54 -> 0.71 ms. (With subnormal results left to CUDA's
+// exp, which most warps of a wide cost then call: 50.9 ms, 190, 570 us and 1.21 ms.)
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -67,17 +69,22 @@ __device__ __forceinline__ uint64_t mulhi_approx(uint32_t ah, uint32_t al, uint3
 __device__ __forceinline__ double exp64(double t, const ExpTable& tab) {
   const uint32_t hi = (uint32_t)__double2hiint(t), lo = (uint32_t)__double2loint(t);
   const uint32_t ax = hi & 0x7fffffffu;
-  // 2^-20 <= |t| < 708; the rest (tiny, overflowing, subnormal results, NaN) is rare
-  if (ax - 0x3eb00000u >= 0x40862000u - 0x3eb00000u) {
+  // 2^-20 <= |t| < 708.39 (normal results). Below, results are subnormal down to -745.5:
+  // they take the same way with 2^-64 put aside, since a sweep over a wide cost meets
+  // them in most warps; the rest (tiny, overflowing, NaN) is rare.
+  bool sub = false;
+  if (ax - 0x3eb00000u >= 0x4086232bu - 0x3eb00000u) {
     if (hi >= 0xc0874c00u && hi < 0xfff00000u) return 0.0;  // t < -745.5
-    return exp_rare(t);
+    if (ax < 0x3c900000u) return 1.0;                       // |t| < 2^-54
+    sub = hi >= 0xc086232bu && hi < 0xc0874c00u;
+    if (!sub) return exp_rare(t);
   }
   // H = |t| log2(e) as mantissa x 2^-63 / 2^64, then W = t log2(e) 2^85 (96 bits, two's complement)
   const uint32_t mh = __funnelshift_l(lo, ax, 11) | 0x80000000u, ml = lo << 11;
   const uint64_t H = mulhi_approx(mh, ml, 0xb8aa3b29u, 0x5c17f0bcu);
   const uint32_t sh = 1032u - (ax >> 20);  // 0 .. 29
   const uint32_t sgn = (uint32_t)((int32_t)hi >> 31);
-  const uint32_t w2 = ((uint32_t)(H >> 32) >> sh) ^ sgn;
+  const uint32_t w2 = (((uint32_t)(H >> 32) >> sh) - (sub ? 64u << 21 : 0u)) ^ sgn;
   const uint32_t w1 = __funnelshift_r((uint32_t)H, (uint32_t)(H >> 32), sh) ^ sgn;
   const uint32_t w0 = __funnelshift_r(0u, (uint32_t)H, sh) ^ sgn;
   // 11 bits of exponent, 11 of table index, 64 of x2 = 2048 x (x < 2^-11)
@@ -92,7 +99,8 @@ __device__ __forceinline__ double exp64(double t, const ExpTable& tab) {
   const uint64_t m = T + (tp >> 11);  // 2^(j / 2048 + x) in Q2.62
   const uint32_t rlo = __funnelshift_r((uint32_t)m, (uint32_t)(m >> 32), 10);
   const uint32_t rhi = ((uint32_t)(m >> 32) >> 10) + ((uint32_t)((int32_t)w2 >> 1) & 0xfff00000u) + (1022u << 20);
-  return __hiloint2double((int)rhi, (int)rlo);
+  const double r = __hiloint2double((int)rhi, (int)rlo);
+  return sub ? r * 5.42101086242752217e-20 : r;
 }
 
 // (double)x on the integer pipes (exact; zeros, subnormals and non-finite values
