@@ -51,7 +51,7 @@ enum ScCtl : int {
                                      // while a column half runs)
   SC_CTL_END
 };
-static_assert((int)SC_CTL_END <= (int)SC_TOTAL, "device scalar array too small for the stage control");
+static_assert((int)SC_CTL_END <= (int)SC_DMAX, "device scalar array too small for the stage control");
 
 enum Err : int { E_NONE = 0, E_MAXNEWTON, E_CHISK, E_CGMAX, E_RHO, E_LS, E_TIME };
 

@@ -55,7 +55,10 @@ void ensure_capacity(eot_handle h, int64_t n, int64_t m) {
   EOT_CUDA(cudaMemset(h->cnt_rowblk, 0, h->rowblk_slots * sizeof(int)));
   EOT_CUDA(cudaMemset(h->cnt_dot, 0, sizeof(int)));
   h->colpart = (double*)dev_alloc(h, 2 * h->max_rowblk * Mm * sizeof(double));
-  h->dotpart = (double*)dev_alloc(h, 2 * h->dot_slots * sizeof(double));
+  // dot partials: one pair per CTA of a sweep or O(n) kernel (the split-coordinate point
+  // sweeps: up to 8 CTAs per 32 points)
+  h->dot_cap = std::max<int64_t>(h->dot_slots, 8 * (L / 32 + 1));
+  h->dotpart = (double*)dev_alloc(h, 2 * h->dot_cap * sizeof(double));
   h->cgpart = (double*)dev_alloc(h, 2 * (4 * (int64_t)h->sms + 8) * sizeof(double));
   double** nv[] = {&h->Al, &h->rowfac, &h->rP, &h->logrP, &h->rowmax, &h->rt, &h->logrt,
                    &h->du, &h->x, &h->res, &h->z, &h->p, &h->q, &h->y, &h->Yx, &h->M,

@@ -63,7 +63,7 @@ struct eot_handle_s {
   // sweep scratch
   int *cnt_strip = nullptr, *cnt_rowblk = nullptr, *cnt_dot = nullptr;
   double *colpart = nullptr, *rowpart = nullptr, *dotpart = nullptr;
-  int64_t max_strips = 0, max_rowblk = 64, dot_slots = 0, rowblk_slots = 0;
+  int64_t max_strips = 0, max_rowblk = 64, dot_slots = 0, dot_cap = 0, rowblk_slots = 0;
   double* maxbuf = nullptr;  // per-CTA candidates of the point-cost maximum
   int64_t maxbuf_len = 0;
   // FP64 n-vectors

@@ -18,7 +18,8 @@ enum Sc : int {
   SC_RZPREV,         // <res, z> of the previous CG iteration (dense CG: beta's denominator)
   SC_CTL_BEGIN,      // the stage control's slots follow (control.cuh)
   SC_COUNT = 32,     // the slots the sweeps and O(n) kernels use (eot_marginals_noalloc keeps these)
-  SC_TOTAL = 64      // with the stage control's slots (control.cuh): the handle's array
+  SC_DMAX = 64,      // point clouds: a bound on max |x_i - y_j|^2 (after the stage control's slots, control.cuh)
+  SC_TOTAL = 68      // the handle's array
 };
 
 // ----------------------------------------------------------------------------
@@ -1127,5 +1128,10 @@ static __global__ void dual_value_kernel(const double* sc, int s_ru, int s_cv, i
 
 static __global__ void set_scalar_kernel(double* sc, int slot, double v) {
   pdl_wait(); sc[slot] = v; }
+static __global__ void set_scalars_kernel(double* sc, int s0, double v0, int s1, double v1) {
+  pdl_wait();
+  sc[s0] = v0;
+  sc[s1] = v1;
+}
 
 }  // namespace eot

@@ -16,6 +16,7 @@
 
 #include "control.cuh"
 #include "handle.cuh"
+#include "sweep_pgrid.cuh"
 #include "sweep_pts.cuh"
 #include "sweep_tc.cuh"
 
@@ -130,6 +131,7 @@ struct Solver {
   const float *X = nullptr, *Y = nullptr;
   int d = 0;
   double sC = 0.0;
+  bool sc_given = false;  // s_C is the caller's
 
   Solver(eot_handle h_, const eot_problem* P, cudaStream_t s)
       : h(h_), st(s), n(P->n), m(P->m), ldc(P->ldc), C((const T*)P->C) {
@@ -147,7 +149,8 @@ struct Solver {
       // set-up row sweep reduces three sums)
       ensure_rowpart_elems(h, kPtsMaxPartials * pts_geo(true).S * n);
       ensure_rowpart_elems(h, kPtsMaxPartials * pts_geo(false).S * m);
-      sC = P->cost_scale > 0.0 ? P->cost_scale : max_cost_scale();
+      sc_given = P->cost_scale > 0.0;
+      sC = sc_given ? P->cost_scale : max_cost_scale();
       if constexpr (sizeof(T) == 4) {
         if (!plain && d >= tc::kMinD && tc_enabled()) setup_tc();
       }
@@ -180,6 +183,73 @@ struct Solver {
 
   // ---- point-cloud geometry (pts_geo_of / tc_geo_of above the class) ----
   PtsGeo pts_geo(bool rows) const { return pts_geo_of(h, rows ? n : m, rows ? m : n, d); }
+  // ---- split-coordinate point sweeps (mixed precision, d <= pg::kMaxD) ----
+  bool pg_on = false;
+  static bool pg_enabled() {
+    const char* e = std::getenv("EOT_PGRID");
+    return !(e && e[0] == '0');
+  }
+  // Sets gamma for the sweeps of this call (the largest it will use) and decides
+  // whether its point sweeps take split coordinates: their accuracy holds up to
+  // pg::kMaxBound base-2 exponent units, gamma s_C log2(e) max |x - y|^2. A library-
+  // computed s_C gives the maximum itself; for a caller's s_C the clouds' extent
+  // bounds it, which takes a read back (not possible when the call must stay
+  // asynchronous).
+  void begin(double gamma, bool may_sync = true) {
+    gamma_host = gamma;
+    double dmax = 0.0;
+    pg_on = false;
+    if (sizeof(T) == 4 && points && !plain && d <= pg::kMaxD && pg_enabled()) {
+      if (!sc_given) dmax = 1.00001 / sC;
+      else if (may_sync) dmax = extent_bound();
+      pg_on = dmax > 0.0 && gamma * sC * pg::kLog2eD * dmax <= pg::kMaxBound;
+    }
+    launch_k(set_scalars_kernel, dim3(1), dim3(1), st, h->sc, (int)SC_GAMMA, gamma, (int)SC_DMAX, dmax);
+    EOT_LAUNCH_CHECK();
+    h->launches++;
+  }
+  // (max |x - x_0| + max |y - x_0|)^2 >= max |x_i - y_j|^2, from one pass over the points
+  double extent_bound() {
+    int* r2 = (int*)h->maxbuf;
+    EOT_CUDA(cudaMemsetAsync(r2, 0, 2 * sizeof(int), st));
+    const int64_t blocks = std::min<int64_t>((n + m + kThreads - 1) / kThreads, 2 * (int64_t)h->sms);
+    launch_k(pg::extent_kernel, dim3((unsigned)blocks), dim3(kThreads), st, X, Y, n, m, d, r2);
+    EOT_LAUNCH_CHECK();
+    h->launches++;
+    EOT_CUDA(cudaMemcpyAsync(h->h_sc, r2, sizeof(double), cudaMemcpyDeviceToHost, st));
+    EOT_CUDA(cudaStreamSynchronize(st));
+    float f[2];
+    std::memcpy(f, h->h_sc, sizeof(f));
+    const double rx = std::sqrt((double)f[0]), ry = std::sqrt((double)f[1]);
+    return (rx + ry) * (rx + ry);
+  }
+  template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
+  void launch_pg_at(cudaStream_t s, const SweepArgs<T>& a, const pg::Geo& g, const Epi& e) {
+    launch_kc(pg::sweep_kernel<D, RO, NR, LSE, SQM, ROWS, GRAD, Epi>, dim3((unsigned)g.B, (unsigned)g.S),
+              dim3(kThreads), (unsigned)g.S, s, a, pg::Args{h->sc + SC_DMAX, g.ws}, e);
+  }
+  template <int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
+  void launch_pg(cudaStream_t s, SweepArgs<T> a, const Epi& e) {
+    const pg::Geo g = pg::geo_of(h->sms, ROWS ? n : m, ROWS ? m : n, d, GRAD);
+    a.chunk = g.chunk;
+    if (Epi::kDot > 0 && g.B * g.S > h->dot_cap)
+      throw EotError{EOT_ERR_INVALID_ARG, "point sweep scratch smaller than the launch needs"};
+    constexpr int R4 = GRAD ? 2 : 4, R2 = GRAD ? 1 : 2;  // own elements per thread at small d, at d > 4
+    if (d <= 2) {
+      if (g.ro == 1) launch_pg_at<2, 1, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      else launch_pg_at<2, R4, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+    } else if (d == 3) {
+      if (g.ro == 1) launch_pg_at<3, 1, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      else launch_pg_at<3, R4, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+    } else if (d == 4) {
+      if (g.ro == 1) launch_pg_at<4, 1, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      else launch_pg_at<4, R4, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+    } else if (d <= 8) {
+      launch_pg_at<8, R2, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+    } else {
+      launch_pg_at<16, R2, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+    }
+  }
   // ---- tensor-core point path (mixed precision, d >= tc::kMinD) ----
   bool tc_on = false;
   tc::TcArgs targs{};
@@ -416,6 +486,10 @@ struct Solver {
         launch_tc<NR, LSE, SQM, ROWS>(s, a, e);
         return;
       }
+      if (pg_on) {
+        launch_pg<NR, LSE, SQM, ROWS, false>(s, a, e);
+        return;
+      }
     }
     const PtsGeo g = pts_geo(ROWS);
     a.chunk = g.chunk;
@@ -515,6 +589,17 @@ struct Solver {
   // components in groups of DG (one launch per group); ROWS: own = rows.
   template <bool ROWS>
   void grad_pts(double scale, const double* ownfac, float* out) {
+    if constexpr (sizeof(T) == 4) {
+      if (pg_on) {
+        SweepArgs<T> a = args();
+        a.wc[0] = ewc();
+        a.wr[0] = ewr();
+        launch_pg<1, false, 0, ROWS, true>(st, a, pg::GradEpi{scale, ownfac, out, d});
+        EOT_LAUNCH_CHECK();
+        h->launches++;
+        return;
+      }
+    }
     const int64_t n_own = ROWS ? n : m, n_oth = ROWS ? m : n;
     const int64_t B = (n_own + kThreads - 1) / kThreads;
     int64_t S = (2 * (int64_t)h->sms + B - 1) / B;
@@ -686,7 +771,7 @@ struct Solver {
     const uintptr_t src = points ? ((uintptr_t)X ^ ((uintptr_t)Y << 1) ^ (uintptr_t)sbits) : (uintptr_t)C;
     const ProgKey key{tag | ((int)sizeof(T) << 4) | ((plain ? 1 : 0) << 8) | ((points ? 1 : 0) << 9) | (d << 10) |
                           ((full_system ? 1 : 0) << 20),
-                      V | ((tc_on ? 1 : 0) << 4) | ((keep_l2 ? 1 : 0) << 5), 0, n, m, ldc, src};
+                      V | ((tc_on ? 1 : 0) << 4) | ((keep_l2 ? 1 : 0) << 5) | ((pg_on ? 1 : 0) << 6), 0, n, m, ldc, src};
     auto it = h->graphs.find(key);
     if (it == h->graphs.end()) {
       if (h->graphs.size() >= 32) free_graphs(h);

@@ -26,7 +26,7 @@ void run_marginals(eot_handle h, const eot_problem* P, const double* u, const do
                    double* total_out, cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.set_scalar(SC_GAMMA, round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma));
   double* lr = lr_out ? lr_out : h->logrP;
   double* lc = lc_out ? lc_out : h->logcP;
   S.row_lse(u, v, nullptr, lr, nullptr, nullptr, SC_MASS, SC_AUX1);
@@ -52,7 +52,7 @@ void run_value(eot_handle h, const eot_problem* P, const double* u, const double
                double* value_out, cudaStream_t st) {
   Solver<T> S(h, P, st);
   const double g = round_gamma<T>(gamma);
-  S.set_scalar(SC_GAMMA, g);
+  S.begin(g, P->cost_scale <= 0.0);  // (asynchronous with a given s_C)
   S.row_lse(u, v, nullptr, nullptr, nullptr, nullptr, SC_MASS, SC_AUX1);
   launch_k(dot_kernel, dim3(S.vg_n), dim3(kOnThreads), st, P->n, P->r, u, h->sc, (int)SC_AUX0, h->dotpart,
            h->cnt_dot);
@@ -70,7 +70,7 @@ void run_hvp(eot_handle h, const eot_problem* P, const double* u, const double* 
              double* c_out, cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.set_scalar(SC_GAMMA, round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma));
   // row maxima for the factorisation P = rowfac * colfac * E
   S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
   S.split_rows(u, nullptr, 0.0, h->rowmax, h->Al, nullptr, h->rowfac, h->rowmax);
@@ -120,7 +120,7 @@ void run_newton(eot_handle h, const eot_problem* P, const double* u, const doubl
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
   if (max_cg <= 0) max_cg = (int)std::min<int64_t>(4 * (full ? P->n + P->m : P->n), 2000);
   S.init_control(1, 1, max_cg);
-  S.set_scalar(SC_GAMMA, round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma));
   // the program runs on the handle's buffers (a captured graph keeps their addresses)
   S.copy(h->U, u, P->n);
   S.copy(h->V, v, P->m);
@@ -154,6 +154,7 @@ void run_solve(eot_handle h, const eot_problem* P, const eot_params* prm_in, dou
   const int max_cg = prm.max_cg > 0 ? prm.max_cg : (int)std::min<int64_t>(4 * (S.full_system ? n + m : n), 2000);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
   S.init_control(prm.max_newton, prm.max_ls, max_cg);
+  S.begin(round_gamma<T>(prm.gamma_f));  // the largest temperature of the call
   if (capped) {
     launch_k(set_deadline_kernel, dim3(1), dim3(1), st, h->sc, prm.max_seconds);
     EOT_LAUNCH_CHECK();
@@ -331,7 +332,7 @@ double run_sweep_bench(eot_handle h, const eot_problem* P, const double* u, cons
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
   S.retain_cost();
-  S.set_scalar(SC_GAMMA, round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma));
   // untimed set-up: the Newton-step factorisation and a CG start at rho = 1/2
   S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
   launch_k(exp_kernel, dim3(S.vg_n), dim3(kOnThreads), st, P->n, h->logrP, h->rt);  // r~ := r(P) (any finite target)
@@ -428,7 +429,7 @@ void run_backward_dense(eot_handle h, const eot_problem* P, const double* u, con
                         double gamma, double scale, const double* scale_dev, float* dC, cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.set_scalar(SC_GAMMA, round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma));
   S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
   S.split_rows(u, nullptr, 0.0, h->rowmax, h->Al, nullptr, h->rowfac, h->rowmax);
   S.split_cols(v, nullptr, 0.0, nullptr, h->Bl, nullptr, h->colfac, nullptr);
@@ -456,7 +457,7 @@ void run_backward_points(eot_handle h, const eot_problem* P, const double* u, co
                          cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.set_scalar(SC_GAMMA, round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma));
   const double f = scale * 2.0 * S.sC;
   if (dX) {
     S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);

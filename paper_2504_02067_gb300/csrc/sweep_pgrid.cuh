@@ -1,0 +1,452 @@
+// Mixed-precision sweeps of low-dimensional point clouds (d <= 16) from split
+// coordinates. As pts_sweep_kernel (sweep_pts.cuh) they form the cost
+// C_ij = s_C |x_i - y_j|^2 on the fly; the exponent is kept in base 2,
+//     t2_ij = (Ah_i + Bh_j) log2 e - |x'_i - y'_j|^2,   x' = sqrt(gamma s_C log2 e) (x - x_0),
+// so that no scaling is left per entry and ex2 takes t2 as it is. Every scaled
+// coordinate is split once per point, x' = xh + xl with xh on a grid of step s (a
+// power of two) and |xl| <= s / 2, and
+//     |x' - y'|^2 = sum dh^2 + sum dl (2 dh + dl),   dh = xh - yh, dl = xl - yl.
+// s = 2^ceil(log2(sqrt(D') 2^-11)) for D' >= max |x' - y'|^2 makes dh and dh^2 exact
+// in FP32 and keeps the running sum of Ah + Bh (on the 1/8 grid, s^2 <= 1/8) and the
+// -dh^2 exact while below 4 D'; dl is rounded at 2^-25 s. The pairs that carry the
+// plan's mass have D' of a few tens, so the second sum is of order 10 s and its
+// rounding below 1e-7 of an exponent unit up to D' = 2^15: less than the rounding of
+// t2 itself, and t2 is rounded once where the scheme of sweep_pts.cuh (TwoSum
+// differences, compensated squares, a two-term gamma s_C) rounds four times.
+// Five FP32 instructions per coordinate against eighteen.
+//
+// Work split: FP32-issue-bound for large clouds (each thread owns RO elements, the
+// other side's records are broadcast from shared memory), latency-bound for small
+// ones, where a CTA's warps split the other side `ws` ways for the same own
+// elements and a cluster of up to 8 CTAs splits it further. All partial sums meet in
+// shared memory, then through distributed shared memory in rank order: no global
+// partials, no ticket, a fixed order. Measured (general sweeps -> these): gradients of
+// n = m = 65536, d = 3 (four sweeps) 62.4 -> 18.5 ms; training step of n = 1000,
+// m = 700, d = 2 36.8 -> 13.3 ms.
+#pragma once
+#include "sweep_pts.cuh"
+
+namespace eot {
+namespace pg {
+
+constexpr int kMaxD = 16;
+constexpr double kMaxBound = 32768.0;  // largest gamma s_C log2(e) max |x - y|^2 (base-2 exponent units)
+// The online max of an LSE moves in whole units of the base-2 exponent, so that every
+// rescaling (here and where partial sums meet) is by an exact power of two.
+constexpr float kThetaB2 = 12.0f;      // lazy-rescale threshold
+constexpr float kLowest = -2097152.0f; // an LSE's start: below every exponent of the split range
+constexpr double kLog2eD = 1.4426950408889634074;
+constexpr double kLn2D = 0.69314718055994530942;
+
+struct Args {
+  const double* dmax;  // device: >= max |x_i - y_j|^2
+  int ws;              // warps of a CTA that share own elements (1, 2, 4 or 8)
+};
+
+struct Geo {
+  int64_t B, S, chunk;
+  int ro, ws;
+};
+// Fewest waves x per-thread entries. A CTA's fixed cost (prologue, combine, epilogue:
+// about 2 us) is worth about 48 entries per thread at two CTAs per SM; staging an
+// other-side record costs a thread about 3.5 entries.
+// grad: the gradient sweeps, with a sum per coordinate in registers.
+inline Geo geo_of(int sms, int64_t n_own, int64_t n_oth, int d, bool grad) {
+  Geo best{};
+  double bc = -1.0;
+  for (int ro : {1, 2, 4}) {
+    const bool built = grad ? (ro == 1 || (d <= 4 && ro == 2)) : (d <= 4 ? ro != 2 : ro == 2);
+    if (!built) continue;
+    for (int ws : {1, 2, 4, 8}) {
+      const int64_t own = (int64_t)(kThreads / ws) * ro, B = (n_own + own - 1) / own;
+      for (int64_t S = 1; S <= 8; ++S) {
+        const int64_t chunk = ((n_oth + S - 1) / S + 7) / 8 * 8, Sr = (n_oth + chunk - 1) / chunk;
+        if (Sr != S) continue;
+        const int64_t waves = (B * S + 2 * sms - 1) / (2 * sms);
+        const double c = (double)waves * (48.0 + (double)((chunk + ws - 1) / ws) * ro + 3.5 * (double)((chunk + kThreads - 1) / kThreads));
+        if (bc < 0.0 || c < bc) {
+          bc = c;
+          best = Geo{B, S, chunk, ro, ws};
+        }
+      }
+    }
+  }
+  return best;
+}
+
+// dX, dY: out_e,k = scale ownfac_e sum_o P-weights (x_e - x_o)_k, the sum in scaled
+// coordinates (1 / sigma undoes the scaling)
+struct GradEpi {
+  static constexpr int kDot = 0;
+  double scale;
+  const double* ownfac;
+  float* out;
+  int d;
+  template <int D>
+  __device__ void grad(int64_t e, const double (&v)[D], double inv_sigma) {
+    const double f = scale * ownfac[e] * inv_sigma;
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      if (k < d) out[e * d + k] = (float)(f * v[k]);
+  }
+  __device__ void finish(const double*) {}
+};
+
+struct Scale {
+  float sh, sl;   // sigma = sqrt(gamma s_C log2 e) as an FP32 pair
+  float magic;    // 1.5 x 2^23 s: adding and subtracting it rounds to the grid
+  double sigma;
+};
+
+// (x - c) sigma as a grid part and a remainder
+__device__ __forceinline__ void split_coord(float x, float c, const Scale& sc, float& xh, float& xl) {
+  const float t = sub_rn(x, c);  // TwoSum: x - c = t + e
+  const float bv = sub_rn(t, x);
+  const float e = sub_rn(sub_rn(x, sub_rn(t, bv)), add_rn(c, bv));
+  const float p = mul_rn(t, sc.sh);
+  const float pe = fmaf(t, sc.sh, -p) + fmaf(t, sc.sl, e * sc.sh);
+  xh = sub_rn(add_rn(p, sc.magic), sc.magic);
+  xl = add_rn(sub_rn(p, xh), pe);
+}
+// A log2 e (A on the 1/8 grid, |A| < 2^19) as a part on the 1/8 grid and a remainder
+__device__ __forceinline__ void split_offset(float A, float& ph, float& pr) {
+  constexpr float L = 1.44269502f, Ll = 1.92596299e-8f;  // log2 e = L + Ll
+  const float p = mul_rn(A, L);
+  const float pe = fmaf(A, L, -p) + A * Ll;
+  ph = rintf(p * 8.0f) * 0.125f;
+  pr = sub_rn(p, ph) + pe;
+}
+
+template <class V>
+__device__ __forceinline__ float ld_cluster_f(const V* p, uint32_t rank) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  uint32_t ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
+  return v;
+}
+
+// What one thread does with its RO own elements and a tile of the other side's
+// records; shared by the sweep kernel below and the batched solver's sweeps.
+template <int D, int RO, int NR, bool LSE, int SQM, bool GRAD>
+struct Core {
+  static constexpr int NA = GRAD ? D : (LSE ? 1 : NR);  // sums per own element
+  static constexpr int NW = GRAD || LSE ? 1 : NR;       // weights per other element
+  static constexpr int REC = (2 * D + 2 + NW + 3) / 4 * 4;
+  float xh[RO][D], xl[RO][D], ph[RO], pr[RO];
+  float S[RO][NA], Cc[RO][NA], mx[RO], hm[RO];
+
+  __device__ __forceinline__ void own(int r, bool ev, const float* x, int d, const float (&ctr)[D], const Scale& sc,
+                                      float A) {
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      if (ev && k < d) split_coord(__ldg(x + k), ctr[k], sc, xh[r][k], xl[r][k]);
+      else xh[r][k] = xl[r][k] = 0.f;
+    }
+    split_offset(ev ? A : 0.f, ph[r], pr[r]);
+    mx[r] = kLowest;
+    hm[r] = LSE ? ph[r] - kLowest : ph[r];
+#pragma unroll
+    for (int k = 0; k < NA; ++k) S[r][k] = Cc[r][k] = 0.f;
+  }
+  // one record: [yh (D), yl (D), high offset, low offset, weights]
+  static __device__ __forceinline__ void stage(float (&rec)[REC], const float* y, int d, const float (&ctr)[D],
+                                               const Scale& sc, float B, const float (&w)[NW]) {
+    float v[REC];
+#pragma unroll
+    for (int k = 0; k < REC; ++k) v[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      if (k < d) split_coord(__ldg(y + k), ctr[k], sc, v[k], v[D + k]);
+    split_offset(B, v[2 * D], v[2 * D + 1]);
+#pragma unroll
+    for (int k = 0; k < NW; ++k) v[2 * D + 2 + k] = w[k];
+#pragma unroll
+    for (int k = 0; k < REC; k += 4)
+      *reinterpret_cast<float4*>(&rec[k]) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+  }
+  static __device__ __forceinline__ void load(const float (&rec)[REC], float (&v)[REC]) {
+#pragma unroll
+    for (int k = 0; k < REC; k += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(&rec[k]);
+      v[k] = x.x;
+      v[k + 1] = x.y;
+      v[k + 2] = x.z;
+      v[k + 3] = x.w;
+    }
+  }
+  // t2 of own element r and the record v (h: the own side's high offset)
+  __device__ __forceinline__ float expo2(int r, float h, const float (&v)[REC]) const {
+    float acc = h + v[2 * D];
+    float lo = pr[r] + v[2 * D + 1];
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      const float dh = xh[r][k] - v[k], dl = xl[r][k] - v[D + k];
+      acc = fmaf(-dh, dh, acc);
+      lo = fmaf(-dl, fmaf(2.0f, dh, dl), lo);
+    }
+    return acc + lo;
+  }
+  // the records q0 <= q < q1 of a tile
+  __device__ __forceinline__ void tile(const float (*rec)[REC], int q0, int q1) {
+    for (int qb = q0; qb < q1; qb += kPtsFlush) {
+      const int qe = min(q1, qb + kPtsFlush);
+      float acc[RO][NA];
+#pragma unroll
+      for (int r = 0; r < RO; ++r)
+#pragma unroll
+        for (int k = 0; k < NA; ++k) acc[r][k] = 0.f;
+      if constexpr (LSE) {
+        constexpr int G = RO == 1 ? 4 : (D <= 4 ? 2 : 1);  // entries per test of the running max
+        for (int q = qb; q < qe; q += G) {
+          float t[RO][G], w[G], tm[RO];
+          bool up = false;
+#pragma unroll
+          for (int u = 0; u < G; ++u) {
+            float v[REC];
+            load(rec[min(q + u, qe - 1)], v);
+            w[u] = q + u < qe ? v[2 * D + 2] : 0.f;
+#pragma unroll
+            for (int r = 0; r < RO; ++r) t[r][u] = expo2(r, hm[r], v);
+          }
+#pragma unroll
+          for (int r = 0; r < RO; ++r) {
+            tm[r] = t[r][0];
+#pragma unroll
+            for (int u = 1; u < G; ++u) tm[r] = fmaxf(tm[r], t[r][u]);
+            up |= tm[r] > kThetaB2;
+          }
+          for (int k = 0; k < 4 && up; ++k) {  // raise the max, form the group again
+            up = false;
+#pragma unroll
+            for (int r = 0; r < RO; ++r) {
+              if (!(tm[r] > kThetaB2)) continue;
+              const float dlt = ceilf(tm[r]);
+              mx[r] += dlt;
+              hm[r] = ph[r] - mx[r];
+              const float f = ex2_approx(-dlt);
+              acc[r][0] *= f;
+              S[r][0] *= f;
+              Cc[r][0] *= f;
+#pragma unroll
+              for (int u = 0; u < G; ++u) {
+                float v[REC];
+                load(rec[min(q + u, qe - 1)], v);
+                t[r][u] = expo2(r, hm[r], v);
+                tm[r] = u == 0 ? t[r][0] : fmaxf(tm[r], t[r][u]);
+              }
+              up |= tm[r] > kThetaB2;
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < RO; ++r)
+#pragma unroll
+            for (int u = 0; u < G; ++u) acc[r][0] = fmaf(ex2_approx(t[r][u]), w[u], acc[r][0]);
+        }
+      } else {
+#pragma unroll 2
+        for (int q = qb; q < qe; ++q) {
+          float v[REC];
+          load(rec[q], v);
+#pragma unroll
+          for (int r = 0; r < RO; ++r) {
+            const float ex = ex2_approx(expo2(r, ph[r], v));
+            if constexpr (GRAD) {
+              const float pw = ex * v[2 * D + 2];
+#pragma unroll
+              for (int k = 0; k < D; ++k)
+                acc[r][k] = fmaf(pw, (xh[r][k] - v[k]) + (xl[r][k] - v[D + k]), acc[r][k]);
+            } else {
+#pragma unroll
+              for (int k = 0; k < NR; ++k) {
+                if ((SQM >> k) & 1) acc[r][k] = fmaf(ex * ex, v[2 * D + 2 + k], acc[r][k]);
+                else acc[r][k] = fmaf(ex, v[2 * D + 2 + k], acc[r][k]);
+              }
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < RO; ++r)
+#pragma unroll
+        for (int k = 0; k < NA; ++k) kadd(S[r][k], Cc[r][k], acc[r][k]);
+    }
+  }
+};
+
+// sigma and the grid of one temperature: kap = gamma s_C log2 e, dmax >= max |x - y|^2
+__device__ __forceinline__ Scale make_scale(double gamma, double sC, double dmax) {
+  const double kap = gamma * sC * kLog2eD;
+  Scale s;
+  s.sigma = sqrt(kap);
+  s.sh = (float)s.sigma;
+  s.sl = (float)(s.sigma - (double)s.sh);
+  // s = 2^ceil(log2(sqrt(kap dmax) 2^-11)), at least 2^-30
+  const int ex = max(ilogb(sqrt(kap * dmax)) + 1 - 11, -30);
+  s.magic = 1.5f * __int_as_float((127 + 23 + ex) << 23);
+  return s;
+}
+
+// Adds the sums of the `ws` warp groups that share own elements (slots w * OWN + o of
+// red and rmx, o < OWN) into slot o, in order; all threads, between barriers.
+template <int NA, bool LSE, int L>
+__device__ __forceinline__ void combine_groups(float2 (*red)[L], float* rmx, int OWN, int ws) {
+  for (int o = threadIdx.x; o < OWN; o += kThreads) {
+    float M = kLowest;
+    if constexpr (LSE) {
+      for (int w = 0; w < ws; ++w) M = fmaxf(M, rmx[w * OWN + o]);
+    }
+#pragma unroll
+    for (int k = 0; k < NA; ++k) {
+      float s0 = 0.f, c0 = 0.f;
+      for (int w = 0; w < ws; ++w) {
+        const float2 q = red[k][w * OWN + o];
+        const float f = LSE ? ex2_approx(rmx[w * OWN + o] - M) : 1.0f;
+        kadd(s0, c0, q.x * f);
+        c0 += q.y * f;
+      }
+      red[k][o] = make_float2(s0, c0);
+    }
+    if constexpr (LSE) rmx[o] = M;
+  }
+}
+
+template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
+__global__ void __launch_bounds__(kThreads, 2) sweep_kernel(SweepArgs<float> a, Args g, Epi epi) {
+  using C = Core<D, RO, NR, LSE, SQM, GRAD>;
+  constexpr int NA = C::NA, NW = C::NW, REC = C::REC;
+  constexpr int TO = D <= 4 ? 256 : 128;
+  constexpr int ND = Epi::kDot;
+  constexpr int kRec = REC * TO * 4, kRed = NA * kThreads * RO * 8;
+  __shared__ __align__(16) unsigned char buf[kRec > kRed ? kRec : kRed];
+  __shared__ float rmx[LSE ? kThreads * RO : 1];
+  __shared__ Scale sc_s;
+  float(*rec)[REC] = reinterpret_cast<float(*)[REC]>(buf);
+  float2(*red)[kThreads * RO] = reinterpret_cast<float2(*)[kThreads * RO]>(buf);  // (after the sweep)
+
+  const int64_t n_own = ROWS ? a.n : a.m, n_oth = ROWS ? a.m : a.n;
+  const float* xo = ROWS ? a.X : a.Y;
+  const float* xt = ROWS ? a.Y : a.X;
+  const float* ho = ROWS ? a.Ah : a.Bh;
+  const float* ht = ROWS ? a.Bh : a.Ah;
+  const int d = a.d;
+  const int64_t blk = blockIdx.x;
+  const int64_t j0 = (int64_t)blockIdx.y * a.chunk, j1 = min(n_oth, j0 + a.chunk);
+  float ctr[D];  // the common centre: the first point of X
+#pragma unroll
+  for (int k = 0; k < D; ++k) ctr[k] = k < d ? __ldg(a.X + k) : 0.f;
+  pdl_wait();
+  if (a.active && *a.active == 0.0) return;  // (no CTA changes it before all have read it: the cluster stays whole)
+  if (threadIdx.x == 0) sc_s = make_scale(a.gamma_dev ? *a.gamma_dev : (double)a.gamma, a.sC, *g.dmax);
+  __syncthreads();
+  const Scale sc = sc_s;
+
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ow = kWarps / g.ws, grp = warp / ow;  // warps across own elements; this warp's share of the others
+  const int OWN = ow * 32 * RO, ol = (warp - grp * ow) * 32 + lane;
+  C c;
+#pragma unroll
+  for (int r = 0; r < RO; ++r) {
+    const int64_t e = blk * OWN + r * (ow * 32) + ol;
+    const bool ev = e < n_own;
+    c.own(r, ev, xo + e * d, d, ctr, sc, ev ? ho[e] : 0.f);
+  }
+  for (int64_t jt = j0; jt < j1; jt += TO) {
+    const int tn = (int)min((int64_t)TO, j1 - jt);
+    __syncthreads();
+    for (int q = threadIdx.x; q < tn; q += kThreads) {
+      const int64_t j = jt + q;
+      float w[NW];
+#pragma unroll
+      for (int k = 0; k < NW; ++k) w[k] = ROWS ? a.wc[k][j] : a.wr[k][j];
+      C::stage(rec[q], xt + j * d, d, ctr, sc, ht[j], w);
+    }
+    __syncthreads();
+    const int seg = (tn + g.ws - 1) / g.ws;
+    c.tile(rec, grp * seg, min(tn, (grp + 1) * seg));
+  }
+  pdl_trigger();
+
+  // ---- the CTA's warp groups, then the cluster's CTAs, in order ----
+  __syncthreads();  // (the records are done with)
+#pragma unroll
+  for (int r = 0; r < RO; ++r) {
+    const int at = grp * OWN + r * (ow * 32) + ol;
+#pragma unroll
+    for (int k = 0; k < NA; ++k) red[k][at] = make_float2(c.S[r][k], c.Cc[r][k]);
+    if constexpr (LSE) rmx[at] = c.mx[r];
+  }
+  __syncthreads();
+  if (g.ws > 1) combine_groups<NA, LSE>(red, rmx, OWN, g.ws);
+  cluster_sync();  // every CTA's sums are visible to the cluster
+  const uint32_t rank = cluster_rank(), ranks = gridDim.y;
+  const int per = (OWN + (int)ranks - 1) / (int)ranks;
+  const int o0 = (int)rank * per, o1 = min(OWN, o0 + per);
+  double wd[ND > 0 ? ND : 1];
+#pragma unroll
+  for (int k = 0; k < (ND > 0 ? ND : 1); ++k) wd[k] = 0.0;
+  for (int o = o0 + threadIdx.x; o < o1; o += kThreads) {
+    const int64_t e = blk * OWN + o;
+    if (e >= n_own) continue;
+    float M = kLowest;
+    if constexpr (LSE) {
+      for (uint32_t q = 0; q < ranks; ++q) M = fmaxf(M, ld_cluster_f(&rmx[o], q));
+    }
+    double tot[NA];
+#pragma unroll
+    for (int k = 0; k < NA; ++k) {
+      float s0 = 0.f, c0 = 0.f;
+      for (uint32_t q = 0; q < ranks; ++q) {
+        const float2 x = ld_cluster_f2(&red[k][o], q);
+        const float f = LSE ? ex2_approx(ld_cluster_f(&rmx[o], q) - M) : 1.0f;
+        kadd(s0, c0, x.x * f);
+        c0 += x.y * f;
+      }
+      tot[k] = (double)s0 + (double)c0;
+    }
+    DotArr<ND> dd;
+    if constexpr (GRAD) epi.template grad<D>(e, tot, 1.0 / sc.sigma);
+    else if constexpr (LSE && ROWS) epi.row_lse(e, (double)M * kLn2D, tot[0], dd.v);
+    else if constexpr (LSE) epi.col_lse(e, (double)M * kLn2D, tot[0], dd.v);
+    else if constexpr (ROWS) epi.row(e, tot, dd.v);
+    else epi.col(e, tot, dd.v);
+#pragma unroll
+    for (int k = 0; k < ND; ++k) wd[k] += dd.v[k];
+  }
+  if constexpr (ND > 0) {
+#pragma unroll
+    for (int k = 0; k < ND; ++k) wd[k] = warp_sum(wd[k]);
+    cta_dot_finish<ND>(wd, blk * ranks + rank, (int64_t)gridDim.x * ranks, a.dotpart, a.cnt_dot, epi);
+  }
+  cluster_sync();  // no CTA leaves while another reads its shared memory
+}
+
+// max over both clouds of |x - x_0|^2 (FP32, rounded up by a part in 10^5) as a bound
+// on their extent: |x_i - y_j| <= |x_i - x_0| + |y_j - x_0|. r2[0]: X, r2[1]: Y (zeroed;
+// a NaN or overflow gives an infinite bound).
+static __global__ void __launch_bounds__(kThreads) extent_kernel(const float* X, const float* Y, int64_t n, int64_t m,
+                                                                 int d, int* r2) {
+  pdl_wait();
+  float bx = 0.f, by = 0.f;
+  for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < n + m; q += (int64_t)gridDim.x * kThreads) {
+    const float* p = q < n ? X + q * d : Y + (q - n) * d;
+    float s = 0.f;
+    for (int k = 0; k < d; ++k) {
+      const float t = __ldg(p + k) - __ldg(X + k);
+      s = fmaf(t, t, s);
+    }
+    s = s == s ? s * 1.00001f : INFINITY;
+    if (q < n) bx = fmaxf(bx, s);
+    else by = fmaxf(by, s);
+  }
+  bx = warp_max_f(bx);
+  by = warp_max_f(by);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(r2, __float_as_int(bx));
+    atomicMax(r2 + 1, __float_as_int(by));
+  }
+}
+
+}  // namespace pg
+}  // namespace eot
