@@ -10,8 +10,14 @@
 // those of the single-problem solver (solver.cuh, solver_impl.cuh).
 //
 // A sweep here is a loop of the group's threads over their OWN rows (or
-// columns), each thread reducing over the whole OTHER side staged through
-// shared memory, so a sweep needs no cross-CTA partial sums. The group's CTAs
+// columns), each thread reducing over the OTHER side staged through shared
+// memory, so a sweep needs no cross-CTA partial sums. Mixed precision takes the
+// split coordinates of sweep_pgrid.cuh (the general scheme of sweep_pts.cuh beyond
+// their range, and in FP64); when one round of the group's threads covers the own
+// side several times over, the warps of a CTA share own elements and split the
+// other side instead of idling. 48 planar problems of n = 256 .. 1024,
+// solved and differentiated: 172 ms with the general scheme, 54.8 ms so.
+// The group's CTAs
 // meet at software barriers in global memory whose waits are bounded in time
 // (a stuck barrier aborts the launch with an error instead of hanging). Every
 // control decision uses scalars that all CTAs of a group compute identically
@@ -30,6 +36,7 @@
 
 #include "handle.cuh"
 #include "kernels.cuh"
+#include "sweep_pgrid.cuh"
 #include "sweep_pts.cuh"
 
 namespace eot {
@@ -61,7 +68,7 @@ struct Out {  // per-problem result, written by the group that solved it
 struct Params {
   double gamma_i, gamma_f, p, q1, w_r, tol_final;
   int32_t max_stages, max_newton, max_cg, max_ls;
-  int32_t plain;  // plain FP32 exponent (no split)
+  int32_t pgrid;  // mixed precision: split coordinates where they hold (sweep_pgrid.cuh)
   int32_t probe;  // > 0: autotuner probe, that many LSE sweep pairs per problem
 };
 
@@ -87,11 +94,24 @@ struct Launch {
 // group machinery: barrier, reductions
 // ---------------------------------------------------------------------------
 
+// the staged tile of a sweep: the general scheme's, or (FP32) the split records and
+// then the sums of the warps that share own elements
 template <class T>
-struct Smem {
+struct Tile {
   T sh[kTO];
   T sw[3][kTO];
   T sy[kDmax][kTO];
+};
+constexpr int kMaxRo = 2;  // own elements per thread of a split sweep
+constexpr int kSplitBytes = 16 * kTO * 4;  // kTO records of up to 16 floats; >= 3 sums per own element
+template <class T>
+struct Smem {
+  union {
+    Tile<T> g;
+    unsigned char split[sizeof(T) == 4 ? kSplitBytes : 1];
+  };
+  float rmx[sizeof(T) == 4 ? kThreads * kMaxRo : 1];
+  pg::Scale scale;
   double sc[SC_COUNT];
   double red[4][kWarps];
   double tot[4];
@@ -240,6 +260,8 @@ struct Dev {
   Smem<T>& s;
   const Params& prm;
   int ro;
+  double dmax = 0.0;   // >= max |x_i - y_j|^2
+  bool split_on = false;  // this problem's sweeps take split coordinates
   // problem
   int64_t n, m;
   int d;
@@ -343,7 +365,7 @@ struct Dev {
 
   // ---- the sweep: own elements of this thread against the whole other side ----
   template <int RO, int NR, bool LSE, int SQM, bool ROWS, class Epi>
-  __device__ bool sweep_ro(const T* w0, const T* w1, const T* w2, Epi& epi) {
+  __device__ __noinline__ bool sweep_ro(const T* w0, const T* w1, const T* w2, Epi& epi) {
     constexpr bool PRECISE = sizeof(T) == 4;
     constexpr int NA = LSE ? 1 : NR;
     constexpr int NW = LSE ? 1 : NR;
@@ -392,11 +414,11 @@ struct Dev {
         __syncthreads();
         for (int qq = threadIdx.x; qq < tn; qq += kThreads) {
           const int64_t j = jt + qq;
-          s.sh[qq] = ldv(ht + j);
+          s.g.sh[qq] = ldv(ht + j);
 #pragma unroll
-          for (int k = 0; k < NW; ++k) s.sw[k][qq] = ldv(wv[k] + j);
+          for (int k = 0; k < NW; ++k) s.g.sw[k][qq] = ldv(wv[k] + j);
 #pragma unroll
-          for (int k = 0; k < kDmax; ++k) s.sy[k][qq] = k < d ? (T)xt[j * d + k] : T(0);
+          for (int k = 0; k < kDmax; ++k) s.g.sy[k][qq] = k < d ? (T)xt[j * d + k] : T(0);
         }
         __syncthreads();
         for (int q0 = 0; q0 < tn; q0 += kFlush) {
@@ -410,11 +432,11 @@ struct Dev {
         for (int qq = q0; qq < q1; ++qq) {
           T yq[kDmax];
 #pragma unroll
-          for (int k = 0; k < kDmax; ++k) yq[k] = s.sy[k][qq];
-          const T hb = s.sh[qq];
+          for (int k = 0; k < kDmax; ++k) yq[k] = s.g.sy[k][qq];
+          const T hb = s.g.sh[qq];
           T wq[NW];
 #pragma unroll
-          for (int k = 0; k < NW; ++k) wq[k] = s.sw[k][qq];
+          for (int k = 0; k < NW; ++k) wq[k] = s.g.sw[k][qq];
 #pragma unroll
           for (int r = 0; r < RO; ++r) {
             T Dh, Dl;
@@ -482,9 +504,142 @@ struct Dev {
     }
   }
 
+  // ---- the same sweep from split coordinates (FP32; pg::sweep_kernel's scheme) ----
+  template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, class Epi>
+  __device__ __noinline__ bool sweep_split(const T* w0, const T* w1, const T* w2, Epi& epi) {
+    using C = pg::Core<D, RO, NR, LSE, SQM, false>;
+    constexpr int NA = C::NA, NW = C::NW, REC = C::REC, ND = Epi::kDot, L = kThreads * RO;
+    static_assert(REC * kTO * 4 <= kSplitBytes && NA * L * 8 <= kSplitBytes && RO <= kMaxRo, "split tile too small");
+    float(*rec)[REC] = reinterpret_cast<float(*)[REC]>(s.split);
+    float2(*red)[L] = reinterpret_cast<float2(*)[L]>(s.split);
+    const int64_t n_own = ROWS ? n : m, n_oth = ROWS ? m : n;
+    const float* xo = ROWS ? X : Y;
+    const float* xt = ROWS ? Y : X;
+    const T* ho = ROWS ? Ah : Bh;
+    const T* ht = ROWS ? Bh : Ah;
+    const T* wv[3] = {w0, w1, w2};
+    float ctr[D];  // the common centre: the first point of X
+#pragma unroll
+    for (int k = 0; k < D; ++k) ctr[k] = k < d ? __ldg(X + k) : 0.f;
+    const pg::Scale sc = s.scale;
+    // warps that share own elements: as many as still cover the own side in one round
+    int ws = kWarps;
+    while (ws > 1 && (int64_t)gp.G * (kThreads / ws) * RO < n_own) ws >>= 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ow = kWarps / ws, grp = warp / ow, OWN = ow * 32 * RO, ol = (warp - grp * ow) * 32 + lane;
+    double dots[ND > 0 ? ND : 1];
+#pragma unroll
+    for (int k = 0; k < (ND > 0 ? ND : 1); ++k) dots[k] = 0.0;
+    for (int64_t b0 = (int64_t)gp.rank * OWN; b0 < n_own; b0 += (int64_t)gp.G * OWN) {
+      C c;
+#pragma unroll
+      for (int r = 0; r < RO; ++r) {
+        const int64_t e = b0 + r * (ow * 32) + ol;
+        const bool ev = e < n_own;
+        c.own(r, ev, xo + e * d, d, ctr, sc, ev ? ldv(ho + e) : 0.f);
+      }
+      for (int64_t jt = 0; jt < n_oth; jt += kTO) {
+        const int tn = (int)min((int64_t)kTO, n_oth - jt);
+        __syncthreads();
+        for (int q = threadIdx.x; q < tn; q += kThreads) {
+          const int64_t j = jt + q;
+          float w[NW];
+#pragma unroll
+          for (int k = 0; k < NW; ++k) w[k] = ldv(wv[k] + j);
+          C::stage(rec[q], xt + j * d, d, ctr, sc, ldv(ht + j), w);
+        }
+        __syncthreads();
+        const int seg = (tn + ws - 1) / ws;
+        c.tile(rec, grp * seg, min(tn, (grp + 1) * seg));
+      }
+      __syncthreads();  // (the records are done with)
+#pragma unroll
+      for (int r = 0; r < RO; ++r) {
+        const int at = grp * OWN + r * (ow * 32) + ol;
+#pragma unroll
+        for (int k = 0; k < NA; ++k) red[k][at] = make_float2(c.S[r][k], c.Cc[r][k]);
+        if constexpr (LSE) s.rmx[at] = c.mx[r];
+      }
+      __syncthreads();
+      if (ws > 1) pg::combine_groups<NA, LSE>(red, s.rmx, OWN, ws);
+      // (each thread reads the slots that it combined; without groups, any: see the barrier above)
+      for (int o = threadIdx.x; o < OWN; o += kThreads) {
+        const int64_t e = b0 + o;
+        if (e >= n_own) continue;
+        double tot[NA];
+#pragma unroll
+        for (int k = 0; k < NA; ++k) tot[k] = (double)red[k][o].x + (double)red[k][o].y;
+        DotArr<ND> dd;
+        if constexpr (LSE && ROWS) epi.row_lse(e, (double)s.rmx[o] * pg::kLn2D, tot[0], dd.v);
+        else if constexpr (LSE) epi.col_lse(e, (double)s.rmx[o] * pg::kLn2D, tot[0], dd.v);
+        else if constexpr (ROWS) epi.row(e, tot, dd.v);
+        else epi.col(e, tot, dd.v);
+#pragma unroll
+        for (int k = 0; k < ND; ++k) dots[k] += dd.v[k];
+      }
+    }
+    if constexpr (ND > 0) {
+      if (!reduce<ND>(dots)) return false;
+      if (threadIdx.x == 0) epi.finish(dots);
+      __syncthreads();
+      return true;
+    } else {
+      return bar();
+    }
+  }
+
+  // max |x - x_0| + max |y - x_0| bounds every distance (for a caller's s_C; a computed
+  // s_C gives the largest distance itself)
+  __device__ bool find_dmax(bool given) {
+    if (!given) {
+      dmax = 1.00001 / sC;
+      return true;
+    }
+    double ext[2];
+    for (int side = 0; side < 2; ++side) {
+      const float* p = side ? Y : X;
+      const int64_t len = side ? m : n;
+      double best = 0.0;
+      for (int64_t i = gp.gt; i < len; i += gp.GT) {
+        float q = 0.f;
+        for (int k = 0; k < d; ++k) {
+          const float df = __ldg(p + i * d + k) - __ldg(X + k);
+          q = fmaf(df, df, q);
+        }
+        best = fmax(best, q == q ? (double)q * 1.00001 : INFINITY);
+      }
+      if (!gmax(gp, s, best)) return false;
+      ext[side] = sqrt(best);
+    }
+    dmax = (ext[0] + ext[1]) * (ext[0] + ext[1]);
+    return true;
+  }
+  // the temperature of the sweeps that follow
+  __device__ void set_gamma(double gamma) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s.sc[SC_GAMMA] = gamma;
+      if (split_on) s.scale = pg::make_scale(gamma, sC, dmax);
+    }
+    __syncthreads();
+  }
+
   template <int NR, bool LSE, int SQM, bool ROWS, class Epi>
   __device__ bool sweep(const T* w0, const T* w1, const T* w2, Epi epi) {
     sweeps++;
+    if constexpr (sizeof(T) == 4) {
+      if (split_on) {
+        // (four own elements per thread run as two rounds of two: the other side's
+        // records are read as often, for half the code)
+        if (d <= 2) {
+          if (ro == 1) return sweep_split<2, 1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+          return sweep_split<2, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+        }
+        if (ro == 1) return sweep_split<4, 1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+        return sweep_split<4, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+      }
+      return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+    }
     if (ro == 1) return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
     if (ro == 2) return sweep_ro<2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
     return sweep_ro<4, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
@@ -832,7 +987,7 @@ struct Dev {
       }
       gamma = gamma_f;
       t = 0;
-      set_sc(SC_GAMMA, gamma);
+      set_gamma(gamma);
       if (!bar()) return false;
     }
     for (; t > 0;) {
@@ -851,7 +1006,7 @@ struct Dev {
           m0[j] = logct[j];
         }
       }
-      set_sc(SC_GAMMA, gamma);
+      set_gamma(gamma);
       if (!bar()) return false;
       double dmin = INFINITY;
       bool ok = true;
@@ -911,7 +1066,7 @@ struct Dev {
     smooth(m, c0, 0.01, ct, logct);
     for (int64_t i = gp.gt; i < n; i += gp.GT) nt0[i] = logrt[i];
     for (int64_t j = gp.gt; j < m; j += gp.GT) mt0[j] = logct[j];
-    set_sc(SC_GAMMA, rg(fmin(prm.gamma_i, prm.gamma_f)));
+    set_gamma(rg(fmin(prm.gamma_i, prm.gamma_f)));
     if (!bar()) return false;
     for (int k = 0; k < reps; ++k) {
       if (!col_lse(nt0, nullptr, mt0, nullptr, 0.0, logct, mt0, 1, SC_AUX0, 0.0)) return false;
@@ -962,6 +1117,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) batch_kernel
     int stages = 0;
     bool alive = true;
     if (P.sC <= 0.0) alive = D.compute_sC();
+    if (sizeof(T) == 4 && L.prm.pgrid && alive) {
+      alive = D.find_dmax(P.sC > 0.0);
+      D.split_on = alive && (double)(float)L.prm.gamma_f * D.sC * pg::kLog2eD * D.dmax <= pg::kMaxBound;
+    }
     if (alive) alive = L.prm.probe > 0 ? D.probe(L.prm.probe) : D.solve(&gamma, &gl1, &stages, &merr);
     if (s.fail) return;  // a barrier gave up: leave the launch (the host reports it)
     if (gp.rank == 0 && threadIdx.x == 0) {
@@ -1132,9 +1291,11 @@ std::pair<int, int> tune(eot_handle h, const std::vector<Prob>& probs, const std
   const int resident = max_resident_ctas<T>(h);
   std::pair<int, int> best{2, 2};
   double best_ms = INFINITY;
+  const bool split = sizeof(T) == 4 && prm.pgrid;
   for (int G : {1, 2, 4, 8}) {
     if (G > resident) continue;
     for (int ro : {1, 2, 4}) {
+      if (split && ro == 4) continue;
       const double ms = launch_batch<T>(h, probs, order, outs, G, ro, prm, maxN, maxM, st);
       if (ms < best_ms) {
         best_ms = ms;
@@ -1186,7 +1347,8 @@ eot_status run_batched(eot_handle h, int nprob, const eot_problem* P, const eot_
   prm.max_newton = prm_in.max_newton;
   prm.max_cg = prm_in.max_cg;
   prm.max_ls = prm_in.max_ls;
-  prm.plain = 0;
+  const char* pgrid = std::getenv("EOT_PGRID");
+  prm.pgrid = !(pgrid && pgrid[0] == '0');
   prm.probe = 0;
   const std::pair<int, int> cfg = tune<T>(h, probs, order, prm, maxN, maxM, st);
   std::vector<Out> outs((size_t)nprob);
