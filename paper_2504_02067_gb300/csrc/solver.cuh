@@ -281,7 +281,7 @@ struct Solver {
       return p;
     };
     auto carve = [&](tc::Side& sd, int64_t np) {
-      sd.slices = (const __nv_bfloat16*)take((size_t)np * tc::kSlices * 64 * 2);
+      sd.slices = (const __half*)take((size_t)np * tc::kSlices * 64 * 2);
       sd.nx = (const double*)take((size_t)np * sizeof(double));
       sd.rec = (float*)take((size_t)np * sizeof(float4));
       sd.own = (tc::OwnRec*)take((size_t)np * sizeof(tc::OwnRec));
@@ -301,7 +301,7 @@ struct Solver {
     auto digits = [&](const tc::Side& sd, const float* P, int64_t len, const unsigned long long* em) {
       const int64_t threads = sd.npad * 32;
       launch_k(tc::tc_prep_kernel, dim3((unsigned)((threads + kThreads - 1) / kThreads)), dim3(kThreads), st, P,
-               len, d, sd.npad, X, em, (__nv_bfloat16*)sd.slices, (double*)sd.nx);
+               len, d, sd.npad, X, em, (__half*)sd.slices, (double*)sd.nx);
       EOT_LAUNCH_CHECK();
       h->launches++;
     };

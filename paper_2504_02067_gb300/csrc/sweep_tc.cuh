@@ -1,25 +1,29 @@
 // Point-cloud sweeps whose cross term x_i . y_j runs on the tensor cores
-// (tcgen05, kind::f16 on BF16, FP32 accumulation in TMEM), for the mixed path at
+// (tcgen05, kind::f16 on FP16, FP32 accumulation in TMEM), for the mixed path at
 // larger d (up to 64 coordinates).
 //
 // Exactness (an exact-slice / Ozaki-style splitting). Both point sets are moved
 // by one common centre c (the first point of X; exact in FP64, distances do not
 // change). Each cloud gets one exponent E (every centred coordinate |x_k| < 2^E)
-// and every coordinate is cut into five signed 8-bit digits
-//     x_k = 2^E sum_s d_sk 2^-8(s+1)      (to 2^(E-40)).
-// A digit is an integer of magnitude <= 255, exact in BF16; a digit product is an
-// integer below 2^16 and a dot product over 64 coordinates stays below 2^22, so
-// every MMA of two digit slices is exact in the FP32 accumulator. The 15 slice
-// pairs (s, t) with s + t <= 4 are added into five "level" accumulators
-// S_L = sum_{s+t=L} D_s D_t^T (levels 0-3 hold at most four pairs, below 2^24,
-// and stay exact; level 4 may round by one unit, 2^-32 of a level-0 unit), and
-//     x . y = 2^(Ex + Ey - 16) G,   G = S_0 + 2^-8 S_1 + 2^-16 S_2 + 2^-24 S_3 + 2^-32 S_4
-// to about 2^-38 of the largest |x||y| (the dropped pairs s + t >= 5 and the
-// digit truncation).
+// and every coordinate is rounded to 2^(E-37) and cut into four balanced digits of
+// radix 1024,
+//     x_k = 2^(E-7) sum_s d_sk 2^-10s,   |d_0| <= 128, -512 <= d_s < 512,
+// integers that FP16 holds exactly. The 10 slice pairs (s, t) with s + t <= 3 are
+// added into four "level" accumulators S_L = sum_{s+t=L} D_s D_t^T: over 64
+// coordinates |S_0| <= 2^20 and |S_1| <= 2^23 are exact in the FP32 accumulator
+// whatever the data, S_2 and S_3 while below 2^24 (one unit off, 2^-20 and less of a
+// level-0 unit, beyond), and
+//     x . y = 2^(Ex + Ey - 14) G,   G = S_0 + 2^-10 S_1 + 2^-20 S_2 + 2^-30 S_3
+// to about 2^-36 of the largest |x||y| (the dropped pairs s + t >= 4 and the
+// coordinates' rounding): at gamma = 2^10 about 1e-9 of an exponent unit, a hundredth
+// of the exponent's own FP32 rounding. (Five signed 8-bit digits in BF16 take 15
+// pairs for 2^-38: a training step of n = m = 16384, d = 64 took 384 ms, with ten
+// pairs 339 ms.) Coordinates beyond d are zero: only ceil(d / 16) of the four K = 16 steps
+// of a pair are issued.
 //
 // Exponent algebra. In base-2 units (t2 = t log2 e) the exponent of the plan is
 //     t2_ij = P_i + Q_j + kappa G_ij,   P_i = (A_i - K |x_i|^2) log2 e,
-//     Q_j = (B_j - K |y_j|^2) log2 e,   kappa = 2 K 2^(Ex+Ey-16) log2 e,
+//     Q_j = (B_j - K |y_j|^2) log2 e,   kappa = 2 K 2^(Ex+Ey-14) log2 e,
 // with K = gamma s_C and A, B the high parts of the potentials. A small kernel
 // before each sweep (tc_sweep_prep_kernel) forms P and Q in FP64 and splits each
 // into a high part on the 1/8 grid and a low part below 1/16: the other side's
@@ -33,12 +37,12 @@
 //
 // Tile width. A tcgen05.mma of M = 128, K = 16 costs about 50 cycles whatever
 // its N up to ~96 (measured on GB300: 55 cycles at N = 32, 48 and 96; 96 at
-// N = 192), so the tile is 96 points wide: the five level accumulators then
-// fill 480 of the 512 TMEM columns, one buffer, handed over level by level.
+// N = 192), so the tile is 96 points wide: the four level accumulators take 384 of
+// the 512 TMEM columns, one buffer, handed over level pair by level pair.
 //
 // CTA roles (480 threads, one CTA per SM: about 215 KB of shared memory):
-//   warp 0, lane 0 and warp 14, lane 0: the 60 MMAs of each tile, level by
-//     level (levels 0, 1, 4 and levels 2, 3), with a commit per level group. A
+//   warp 0, lane 0 and warp 14, lane 0: the (up to) 40 MMAs of each tile, twenty
+//     each (levels 0, 3 and levels 1, 2), with a commit per level. A
 //     tcgen05.mma blocks its thread while the tensor unit's short queue is
 //     full, so these threads do nothing else: any other work in them, or a
 //     lost issue slot, leaves the tensor unit idle;
@@ -49,12 +53,11 @@
 //     point per thread) and a third (32) of the tile's 96 columns.
 // Hand-offs are mbarriers: full[sb] (the slices of buffer sb landed), sfree[sb][i]
 // (issuer i's MMAs reading buffer sb are done), rec[s] (records landed), lvl[g] (the
-// MMAs of level group g = {0,1}, {2,3}, {4} are done: accumulators readable),
-// lfree[0] / lfree[1] (the 12 epilogue warps have loaded levels 0-3 / level 4
-// into registers; the next tile's MMAs may overwrite them). Every wait is
-// bounded (tc.cuh).
+// MMAs of levels {0,1}, {2,3} are done, one arrival per issuer: accumulators readable),
+// lfree[g] (the 12 epilogue warps have loaded those levels into registers; the next
+// tile's MMAs may overwrite them). Every wait is bounded (tc.cuh).
 #pragma once
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "sweep_pts.cuh"
 #include "tc.cuh"
@@ -64,8 +67,9 @@ namespace tc {
 
 constexpr int kM = 128;     // own points per CTA = TMEM lanes = MMA M
 constexpr int kN = 96;      // other-side points per tile = MMA N
-constexpr int kSlices = 5;  // 8-bit digits per coordinate
-constexpr int kLevels = 5;  // s + t = 0 .. 4
+constexpr int kSlices = 4;  // radix-1024 digits per coordinate
+constexpr int kLevels = 4;  // s + t = 0 .. 3
+constexpr int kCoordBits = 37;  // |x_k| 2^-E in units of 2^-37
 constexpr int kEpiWarps = 12;                  // 3 per TMEM lane quarter
 constexpr int kParts = kEpiWarps / 4;          // column parts of a tile
 constexpr int kPartCols = kN / kParts;         // 32 columns per epilogue warp and tile
@@ -73,19 +77,19 @@ constexpr int kGroups = kPartCols / 8;         // groups of 8 columns in the ari
 constexpr int kMmaWarpB = 2 + kEpiWarps;      // the second MMA-issuing warp (after the epilogue warps)
 constexpr int kTcThreads = 32 * (3 + kEpiWarps);
 constexpr int kTcWarps = kTcThreads / 32;
-constexpr uint32_t kRowB = 128;    // bytes per point and slice: 64 BF16 coordinates
+constexpr uint32_t kRowB = 128;    // bytes per point and slice: 64 FP16 digits
 constexpr uint32_t kOwnSlice = kM * kRowB;                          // 16 KB
 constexpr uint32_t kOthSlice = kN * kRowB;                          // 12 KB
-constexpr uint32_t kOffOth = kSlices * kOwnSlice;                   // 80 KB
+constexpr uint32_t kOffOth = kSlices * kOwnSlice;                   // 64 KB
 constexpr int kSliceBufs = 2;                                       // tile tt: slice buffer tt % 2
 constexpr int kRecSlots = 4;                                        // tile tt: record slot tt % 4
 constexpr uint32_t kRecBytes = kN * 16;                             // 1.5 KB: a slot at the widest record
-constexpr uint32_t kOffRec = kOffOth + kSliceBufs * kSlices * kOthSlice;  // + 120 KB
+constexpr uint32_t kOffRec = kOffOth + kSliceBufs * kSlices * kOthSlice;  // + 96 KB
 constexpr uint32_t kOffBar = kOffRec + kRecSlots * kRecBytes;            // + 6 KB
 constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;               // barriers, TMEM slot; 1024-byte alignment slack
-constexpr uint32_t kTmemCols = 512;                                 // 5 levels x 96 columns used
+constexpr uint32_t kTmemCols = 512;                                 // 4 levels x 96 columns used
 constexpr int64_t kPadRows = 384;                                   // lcm(kM, kN)
-constexpr uint32_t kIdesc = idesc_bf16_f32(kM, kN);
+constexpr uint32_t kIdesc = idesc_f16_f32(kM, kN);
 static_assert(kLevels * kN <= (int)kTmemCols, "level accumulators exceed TMEM");
 constexpr int kMinD = 17;  // the tensor-core path serves d >= kMinD
 constexpr double kLog2eD = 1.4426950408889634;
@@ -106,7 +110,7 @@ struct OwnRec {
 // Per point set: the fixed digit slices and |x - c|^2 (per problem), and the
 // per-sweep records of the point set in either role.
 struct Side {
-  const __nv_bfloat16* slices;  // [kSlices][npad][64], 128-byte swizzle per 8-row atom
+  const __half* slices;  // [kSlices][npad][64], 128-byte swizzle per 8-row atom
   const double* nx;             // [npad] |x - c|^2 (0 for padding)
   float* rec;                   // [npad][rec_floats(NR)] as the other side: {Qh, w0 2^ql[, w1 2^ql, w2 2^ql]}
   OwnRec* own;                  // [npad] as the own side
@@ -146,13 +150,13 @@ static __global__ void tc_extent_kernel(const float* X, int64_t n, int d, const 
   if ((threadIdx.x & 31) == 0 && mx > 0.0) atomicMax(emax, (unsigned long long)__double_as_longlong(mx));
 }
 
-// One warp per point (rows >= n and coordinates >= d are zero): the five digit
+// One warp per point (rows >= n and coordinates >= d are zero): the four digit
 // slices in the swizzled K-major layout and |x - c|^2 in FP64. Centring keeps
 // |x|^2, |y|^2 and x.y bounded by the data's extent, so the expansion
 // |x|^2 + |y|^2 - 2 x.y keeps its accuracy however far the clouds lie from the
 // origin.
 static __global__ void tc_prep_kernel(const float* X, int64_t n, int d, int64_t npad, const float* centre,
-                                      const unsigned long long* emax, __nv_bfloat16* sl, double* nx) {
+                                      const unsigned long long* emax, __half* sl, double* nx) {
   pdl_wait();
   const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -170,16 +174,15 @@ static __global__ void tc_prep_kernel(const float* X, int64_t n, int d, int64_t 
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const int k = lane + 32 * c;
-    const double Qd = trunc(ldexp(xv[c], 40 - e));  // |Q| < 2^40
-    const long long Q = (long long)Qd;
-    const unsigned long long aQ = (unsigned long long)(Q < 0 ? -Q : Q);
-    const float sgn = Q < 0 ? -1.f : 1.f;
+    long long Q = (long long)rint(ldexp(xv[c], kCoordBits - e));  // |Q| <= 2^37
     const int64_t idx = row * 64 + (((k >> 3) ^ (int)(row & 7)) << 3) + (k & 7);
 #pragma unroll
-    for (int s = 0; s < kSlices; ++s) {
-      const unsigned dig = (unsigned)((aQ >> (8 * (kSlices - 1 - s))) & 255ull);
-      sl[(int64_t)s * npad * 64 + idx] = __float2bfloat16_rn(sgn * (float)dig);
+    for (int s = kSlices - 1; s > 0; --s) {  // balanced digits from the lowest up
+      const long long dig = ((Q + 512) & 1023) - 512;
+      sl[(int64_t)s * npad * 64 + idx] = __float2half_rn((float)dig);
+      Q = (Q - dig) >> 10;
     }
+    sl[idx] = __float2half_rn((float)Q);  // |Q| <= 128
   }
 }
 
@@ -197,7 +200,7 @@ __global__ void tc_sweep_prep_kernel(SweepArgs<float> a, TcArgs ta) {
   const double K = (double)g * a.sC;
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i == 0) {
-    const double kap = 2.0 * K * ldexp(1.0, cloud_exp(ta.emax[0]) + cloud_exp(ta.emax[1]) - 16) * kLog2eD;
+    const double kap = 2.0 * K * ldexp(1.0, cloud_exp(ta.emax[0]) + cloud_exp(ta.emax[1]) - 14) * kLog2eD;
     const float kh = (float)kap;
     ta.kappa[0] = kh;
     ta.kappa[1] = (float)(kap - (double)kh);
@@ -274,13 +277,13 @@ template <int NR, bool LSE, int SQM, bool ROWS, class Epi>
 __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float> a, TcArgs ta, Epi epi) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = (uint64_t*)(sm + kOffBar);  // [2] the five slices of the slice buffer landed
+  uint64_t* full = (uint64_t*)(sm + kOffBar);  // [2] the slices of the slice buffer landed
   uint64_t* sfree = full + 2;                  // [2][2] per issuer: its MMAs reading the slice buffer done
-  uint64_t* lvl = full + 6;                    // [3] MMAs of levels {0,1}, {2,3}, {4} done
-  uint64_t* lfree = full + 9;                  // [2] levels 0-3, level 4 loaded by all epilogue warps
-  uint64_t* recf = full + 11;                  // [4] records of the slot landed
-  uint64_t* ownf = full + 15;
-  uint32_t* tslot = (uint32_t*)(full + 16);
+  uint64_t* lvl = full + 6;                    // [2] MMAs of levels {0,1}, {2,3} done (one arrival per issuer)
+  uint64_t* lfree = full + 8;                  // [2] those levels loaded by all epilogue warps
+  uint64_t* recf = full + 10;                  // [4] records of the slot landed
+  uint64_t* ownf = full + 14;
+  uint32_t* tslot = (uint32_t*)(full + 15);
   constexpr int NA = LSE ? 1 : NR;
   constexpr int ND = Epi::kDot;
   constexpr int RW = rec_floats(NR);
@@ -302,7 +305,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
       mbar_init(&sfree[2 * k], 1);
       mbar_init(&sfree[2 * k + 1], 1);
     }
-    for (int g = 0; g < 3; ++g) mbar_init(&lvl[g], 1);
+    for (int g = 0; g < 2; ++g) mbar_init(&lvl[g], 2);
     for (int g = 0; g < 2; ++g) mbar_init(&lfree[g], kEpiWarps);
     for (int k = 0; k < kRecSlots; ++k) mbar_init(&recf[k], 1);
     mbar_init(ownf, 1);
@@ -335,7 +338,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
 
   if (warp == 1) {
     // ---------------- bulk copies (one thread) ----------------
-    // The own 128 points' slices once; tile tt's five slices into buffer tt % 2
+    // The own 128 points' slices once; tile tt's slices into buffer tt % 2
     // and its records into slot tt % 4. Tiles 0 and 1 go at once; tile tt >= 2 once the MMAs of tile
     // tt - 2 are done (sfree), by when the epilogue had loaded tile tt - 3 and
     // so finished tile tt - 4, the previous user of the record slot.
@@ -376,17 +379,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
     __syncwarp();
   } else if (warp == 0 || warp == kMmaWarpB) {
     // ---------------- MMAs (two threads) ----------------
-    // Issuer A (warp 0) owns levels 0, 1 and 4, issuer B (the last warp)
-    // levels 2 and 3: each level's accumulation chain stays in one thread, and
-    // with the issuers on two SM sub-partitions the tensor unit's short queue
-    // stays fed while the epilogue warps compete for issue slots (one issuer
-    // loses ~25 % of the MMA rate to them). Per tile each waits for the slices
-    // and for the epilogue to have loaded levels 0-3 of the previous tile; A
-    // commits levels {0,1}, waits for level 4 of the previous tile to be loaded,
-    // and commits level 4; B commits levels {2,3}; each commits its use of the
-    // slice buffer (sfree[buffer][issuer]).
+    // Issuer A (warp 0) owns levels 0 and 3, issuer B (the last warp) levels 1
+    // and 2 (five slice pairs each): each level's accumulation chain stays in one
+    // thread, and with the issuers on two SM sub-partitions the tensor unit's short
+    // queue stays fed while the epilogue warps compete for issue slots (one issuer
+    // loses ~25 % of the MMA rate to them). Per tile each waits for the slices, then
+    // for the epilogue to have loaded levels {0,1} and {2,3} of the previous tile,
+    // issues and commits its level of either pair, and commits its use of the slice
+    // buffer (sfree[buffer][issuer]).
     if (lane == 0) {
       const int who = warp == 0 ? 0 : 1;
+      const int ksteps = (a.d + 15) / 16;
       const bool own_ok = mbar_wait(ownf, 0, ta.err, kStatTimeout);
       // descriptors of the first own slice and of the first other-side slice;
       // every MMA adds a compile-time offset (all unrolled)
@@ -394,15 +397,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
       const uint64_t bdesc0 = desc_sw128(smem_u32(sm + kOffOth));
       auto level = [&](uint64_t bdesc, int L) {
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4)
+        for (int k4 = 0; k4 < 4; ++k4) {
+          if (k4 >= ksteps) break;  // coordinates beyond d are zero
 #pragma unroll
           for (int s = 0; s < kSlices; ++s) {
             const int t = L - s;
             if (t < 0 || t >= kSlices) continue;
-            mma_bf16(tbase + (uint32_t)(L * kN), adesc0 + (uint64_t)((s * kOwnSlice + k4 * 32) >> 4),
+            mma_f16(tbase + (uint32_t)(L * kN), adesc0 + (uint64_t)((s * kOwnSlice + k4 * 32) >> 4),
                      bdesc + (uint64_t)((t * kOthSlice + k4 * 32) >> 4), kIdesc,
-                     (k4 == 0 && s == (L > kSlices - 1 ? L - (kSlices - 1) : 0)) ? 0u : 1u);
+                     (k4 == 0 && s == 0) ? 0u : 1u);
           }
+        }
       };
       int committed = 0;
       bool ok = own_ok;
@@ -414,23 +419,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
         if (!mbar_wait(&full[sb], fpar, ta.err, kStatTimeout) ||
             (tt >= 1 && !mbar_wait(&lfree[0], ppar, ta.err, kStatTimeout))) {
           ok = false;
-        } else if (who == 0) {
+        } else {
           tc_fence_after();
-          level(bdesc, 0);
-          level(bdesc, 1);
+          if (who == 0) level(bdesc, 0);
+          else level(bdesc, 1);
           mma_commit(&lvl[0]);
           if (tt >= 1 && !mbar_wait(&lfree[1], ppar, ta.err, kStatTimeout)) {
             ok = false;
           } else {
             tc_fence_after();
-            level(bdesc, 4);
-            mma_commit(&lvl[2]);
+            if (who == 0) level(bdesc, 3);
+            else level(bdesc, 2);
+            mma_commit(&lvl[1]);
           }
-        } else {
-          tc_fence_after();
-          level(bdesc, 2);
-          level(bdesc, 3);
-          mma_commit(&lvl[1]);
         }
         uint64_t* sf = &sfree[2 * sb + who];
         mma_commit(sf);  // also after a partly issued tile: its MMAs end before the CTA does
@@ -468,43 +469,37 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
       tmem_ld32(tcol, gh);
       tmem_ld32(tcol + (uint32_t)kN, gl);
       tmem_ld_wait();
-      // G = S_0 + 2^-8 S_1 + ... as an FP32 pair (gh, gl). S_0 is an integer
-      // below 2^22 and 2^-8 S_1 a multiple of 2^-8 below 2^15: where
-      // |S_0| >= |2^-8 S_1| Fast2Sum is exact, and otherwise the sum lies below
-      // 2^16 on the 2^-8 grid and is exact already (z = 2^-8 S_1, error 0).
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&lfree[0]);
+      // G = S_0 + 2^-10 S_1 + ... as an FP32 pair (gh, gl). S_0 is an integer up to
+      // 2^20 and 2^-10 S_1 a multiple of 2^-10 up to 2^13: where
+      // |S_0| >= |2^-10 S_1| Fast2Sum is exact, and otherwise the sum stays within
+      // 2^14 on the 2^-10 grid and is exact already (z = 2^-10 S_1, error 0).
 #pragma unroll
       for (int c = 0; c < kPartCols; ++c) {
         const float s0 = __uint_as_float(gh[c]), s1 = __uint_as_float(gl[c]);
-        const float h = fmaf(s1, 0x1p-8f, s0);
+        const float h = fmaf(s1, 0x1p-10f, s0);
         const float z = __fsub_rn(h, s0);
         gh[c] = __float_as_uint(h);
-        gl[c] = __float_as_uint(fmaf(s1, 0x1p-8f, -z));
+        gl[c] = __float_as_uint(fmaf(s1, 0x1p-10f, -z));
       }
       if (!warp_wait(&lvl[1], par, ta.err)) break;  // levels 2 and 3
       tc_fence_after();
-      bool ok = true;
 #pragma unroll
       for (int L = 2; L < kLevels; ++L) {
-        if (L == 4) {
-          if (!warp_wait(&lvl[2], par, ta.err)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-        }
         tmem_ld32(tcol + (uint32_t)(L * kN), u);
         tmem_ld_wait();
-        if (L >= 3) {  // levels 0-3, then level 4, go back to the MMAs
+        if (L == 3) {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&lfree[L - 3]);
+          if (lane == 0) mbar_arrive(&lfree[1]);
         }
-        const float sc = L == 2 ? 0x1p-16f : (L == 3 ? 0x1p-24f : 0x1p-32f);
+        const float sc = L == 2 ? 0x1p-20f : 0x1p-30f;
 #pragma unroll
         for (int c = 0; c < kPartCols; ++c)
           gl[c] = __float_as_uint(fmaf(__uint_as_float(u[c]), sc, __uint_as_float(gl[c])));
       }
-      if (!ok) break;
       const int rs = tt % kRecSlots;
       if (!warp_wait(&recf[rs], (uint32_t)(tt / kRecSlots) & 1u, ta.err)) break;
       const float* rt = recs + rs * (kRecBytes / 4) + part * kPartCols * RW;

@@ -1,6 +1,6 @@
 // Blackwell (sm_103a) tensor-core plumbing in inline PTX: mbarriers, 1-D bulk
 // copies (the TMA engine), TMEM allocation, tcgen05.mma / commit / ld, and the
-// shared-memory and instruction descriptors of kind::f16 MMAs on BF16 operands
+// shared-memory and instruction descriptors of kind::f16 MMAs on FP16 operands
 // in the 128-byte-swizzled K-major layout.
 //
 // Every wait here is bounded: mbar_wait gives up (after enough polls and time,
@@ -128,11 +128,11 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] x B[smem]^T, kind::f16 (BF16 in, FP32 accumulate), issued
+// D[tmem] (+)= A[smem] x B[smem]^T, kind::f16 (FP16 in, FP32 accumulate), issued
 // by one thread; accumulate = 0 overwrites D. A descriptor's start-address field
 // is linear in the address: desc(addr + off) = desc(addr) + off / 16 while the
 // address stays below 256 KB.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -178,13 +178,13 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor (64 bits) for a K-major operand whose rows are
-// 128 bytes (64 BF16) in the 128-byte swizzle: 8-row atoms of 1024 bytes.
+// 128 bytes (64 FP16) in the 128-byte swizzle: 8-row atoms of 1024 bytes.
 //   [0,14)  start address >> 4      [16,30) leading-dimension byte offset >> 4
 //   [32,46) stride byte offset >> 4 (1024: next 8-row atom)
 //   [46,49) fixed 0b001             [49,52) base offset (0: atoms 1024-aligned)
 //   [61,64) swizzle mode: 2 = 128-byte swizzle
 // The K step inside the 128-byte row advances the start address by 32 bytes per
-// 16 BF16; the hardware applies the swizzle to the resulting addresses.
+// 16 FP16; the hardware applies the swizzle to the resulting addresses.
 __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
@@ -195,11 +195,11 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   return d;
 }
 
-// Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits
-// 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22,
+// Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B FP16 (bits
+// 7-9 = 0, 10-12 = 0), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22,
 // M >> 4 at bits 24-28.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 }  // namespace tc
