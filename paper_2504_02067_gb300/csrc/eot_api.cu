@@ -204,7 +204,7 @@ void run_plan_int(eot_handle h, const eot_problem* P, const double* u, const dou
         chunk = tk * pint::kSC;
       }
       launch_kc(pint::plan_screen_points_kernel<MODE>, dim3((unsigned)B, (unsigned)S), dim3(pint::kThreads),
-                (unsigned)S, st, P->n, P->m, (int)P->d, P->X, P->Y, sC, u, v, gamma, log_tau,
+                (unsigned)S, 0, st, P->n, P->m, (int)P->d, P->X, P->Y, sC, u, v, gamma, log_tau,
                 screen(K, (float)(P->d + 12) * 5.9604645e-8f, (int)P->d), chunk, idx_out, counts, tot);
     } else {
       launch_k(pint::plan_int_points_kernel<MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (int)P->d, P->X, P->Y,

@@ -139,14 +139,14 @@ inline void launch_kd(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
   if (e != cudaSuccess)
     throw EotError{EOT_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e)};
 }
-// launch_k in thread-block clusters of (1, cy, 1) CTAs
+// launch_k in thread-block clusters of (1, cy, 1) CTAs, with dynamic shared memory
 template <typename... KArgs, typename... Args>
-inline void launch_kc(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned cy, cudaStream_t st,
+inline void launch_kc(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned cy, size_t smem, cudaStream_t st,
                       Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;

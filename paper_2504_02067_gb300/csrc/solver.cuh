@@ -185,6 +185,7 @@ struct Solver {
   PtsGeo pts_geo(bool rows) const { return pts_geo_of(h, rows ? n : m, rows ? m : n, d); }
   // ---- split-coordinate point sweeps (mixed precision, d <= pg::kMaxD) ----
   bool pg_on = false;
+  bool pg_grad = false;  // the gradient sweeps (any d)
   static bool pg_enabled() {
     const char* e = std::getenv("EOT_PGRID");
     return !(e && e[0] == '0');
@@ -195,14 +196,15 @@ struct Solver {
   // computed s_C gives the maximum itself; for a caller's s_C the clouds' extent
   // bounds it, which takes a read back (not possible when the call must stay
   // asynchronous).
-  void begin(double gamma, bool may_sync = true) {
+  void begin(double gamma, bool may_sync = true, bool gradients = false) {
     gamma_host = gamma;
     double dmax = 0.0;
-    pg_on = false;
-    if (sizeof(T) == 4 && points && !plain && d <= pg::kMaxD && pg_enabled()) {
+    pg_on = pg_grad = false;
+    if (sizeof(T) == 4 && points && !plain && (d <= pg::kMaxD || gradients) && pg_enabled()) {
       if (!sc_given) dmax = 1.00001 / sC;
       else if (may_sync) dmax = extent_bound();
-      pg_on = dmax > 0.0 && gamma * sC * pg::kLog2eD * dmax <= pg::kMaxBound;
+      pg_grad = dmax > 0.0 && gamma * sC * pg::kLog2eD * dmax <= pg::kMaxBound;
+      pg_on = pg_grad && d <= pg::kMaxD;
     }
     launch_k(set_scalars_kernel, dim3(1), dim3(1), st, h->sc, (int)SC_GAMMA, gamma, (int)SC_DMAX, dmax);
     EOT_LAUNCH_CHECK();
@@ -226,7 +228,7 @@ struct Solver {
   template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
   void launch_pg_at(cudaStream_t s, const SweepArgs<T>& a, const pg::Geo& g, const Epi& e) {
     launch_kc(pg::sweep_kernel<D, RO, NR, LSE, SQM, ROWS, GRAD, Epi>, dim3((unsigned)g.B, (unsigned)g.S),
-              dim3(kThreads), (unsigned)g.S, s, a, pg::Args{h->sc + SC_DMAX, g.ws}, e);
+              dim3(kThreads), (unsigned)g.S, 0, s, a, pg::Args{h->sc + SC_DMAX, g.ws}, e);
   }
   template <int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
   void launch_pg(cudaStream_t s, SweepArgs<T> a, const Epi& e) {
@@ -562,7 +564,7 @@ struct Solver {
             done = true;
           }
         }
-        launch_kc(V == VEC ? kv : k1, grid, dim3(kThreads), (unsigned)cgeo.R, s, a, e);
+        launch_kc(V == VEC ? kv : k1, grid, dim3(kThreads), (unsigned)cgeo.R, 0, s, a, e);
         return;
       }
     }
@@ -590,11 +592,20 @@ struct Solver {
   template <bool ROWS>
   void grad_pts(double scale, const double* ownfac, float* out) {
     if constexpr (sizeof(T) == 4) {
-      if (pg_on) {
+      if (pg_grad) {
         SweepArgs<T> a = args();
         a.wc[0] = ewc();
         a.wr[0] = ewr();
-        launch_pg<1, false, 0, ROWS, true>(st, a, pg::GradEpi{scale, ownfac, out, d});
+        if (pg_on) {
+          launch_pg<1, false, 0, ROWS, true>(st, a, pg::GradEpi{scale, ownfac, out, d});
+        } else {
+          const pg::Geo g = pg::grad_geo(h->sms, ROWS ? n : m, ROWS ? m : n);
+          a.chunk = g.chunk;
+          EOT_CUDA(cudaFuncSetAttribute(pg::grad_tile_kernel<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)sizeof(pg::GradSmem)));
+          launch_kc(pg::grad_tile_kernel<ROWS>, dim3((unsigned)g.B, (unsigned)g.S), dim3(kThreads), (unsigned)g.S,
+                    sizeof(pg::GradSmem), st, a, pg::Args{h->sc + SC_DMAX, 1}, scale, ownfac, out);
+        }
         EOT_LAUNCH_CHECK();
         h->launches++;
         return;

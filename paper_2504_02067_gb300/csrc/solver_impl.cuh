@@ -457,7 +457,7 @@ void run_backward_points(eot_handle h, const eot_problem* P, const double* u, co
                          cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.begin(round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma), true, true);
   const double f = scale * 2.0 * S.sC;
   if (dX) {
     S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
