@@ -288,13 +288,26 @@ __device__ __forceinline__ LsePair warp_lse(LsePair p, const ExpSmem<double>& ex
   return {M == -INFINITY ? 0.0 : M, s};
 }
 
-__device__ __forceinline__ float warp_sum_f(float x) {
+// Warp sums of N values (a power of two up to 32) at once: each step halves the
+// values a lane carries, so eight sums take 9 shuffles instead of 40, with the
+// additions of a butterfly per value (lane distances 16, 8, 4, 2, 1: the same bits).
+// Lane l returns the sum of value l / (32 / N).
+template <int N, class T>
+__device__ __forceinline__ T warp_sum_many(T (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
+  for (int h = N / 2; h > 0; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;  // this lane keeps the upper half of the values
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const T mine = up ? v[k + h] : v[k], other = up ? v[k] : v[k + h];
+      v[k] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
 }
-// warp sum in the element type (FP32 path: FP32 shuffles and adds)
-__device__ __forceinline__ double warp_sum_t(float x) { return (double)warp_sum_f(x); }
-__device__ __forceinline__ double warp_sum_t(double x) { return warp_sum(x); }
 
 }  // namespace eot

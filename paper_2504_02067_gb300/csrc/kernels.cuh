@@ -421,18 +421,30 @@ inline int on_grid(int64_t n, int sms, int64_t slots) {
   return (int)(g < 1 ? 1 : g);
 }
 
-// Split A = x + alpha*y - z into a high part h (multiple of 1/8, exact in T)
-// and a low FP64 part l; optional ew = (T)exp(l), fac = exp(fshift + l).
-// plain != 0: round A to T directly and drop the remainder (plain FP32 path).
+// One side's exponent split: A = x + alpha y - z into a high part h (multiple of 1/8,
+// exact in T) and a low FP64 part l; optional ew = (T)exp(l), fac = exp(fshift + l)
+// and the sweep weights w0 = (T)fac, w1 = (T)(fac wx).
 template <class T>
-__device__ __forceinline__ void split_range(int64_t n, const double* x, const double* y, double alpha,
-                                            const double* z, int plain, T* h, double* l, T* ew, double* fac,
-                                            const double* fshift, int* status) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    double A = x[i];
-    if (y) A += alpha * y[i];
-    if (z) A -= z[i];
+struct SplitJob {
+  int64_t n = 0;
+  const double *x = nullptr, *y = nullptr, *z = nullptr;
+  double alpha = 0.0;
+  T* h = nullptr;
+  double* l = nullptr;
+  T* ew = nullptr;
+  double* fac = nullptr;
+  const double* fshift = nullptr;
+  T *w0 = nullptr, *w1 = nullptr;
+  const double* wx = nullptr;
+};
+// plain: round A to T directly and drop the remainder (plain FP32 path).
+template <class T>
+__device__ __forceinline__ void split_range(const SplitJob<T>& J, double alpha, int plain, int* status, int64_t block,
+                                            int64_t blocks) {
+  for (int64_t i = block * (int64_t)blockDim.x + threadIdx.x; i < J.n; i += blocks * blockDim.x) {
+    double A = J.x[i];
+    if (J.y) A += alpha * J.y[i];
+    if (J.z) A -= J.z[i];
     double hh, ll;
     if (!isfinite(A)) {
       atomicOr(status, kStatNonfinite);
@@ -449,26 +461,33 @@ __device__ __forceinline__ void split_range(int64_t n, const double* x, const do
       hh = rint(A * 8.0) * kGrid;
       ll = A - hh;
     }
-    h[i] = (T)hh;
-    if (l) l[i] = ll;
-    if (ew) ew[i] = (T)exp(ll);
-    if (fac) fac[i] = exp((fshift ? fshift[i] : 0.0) + ll);
+    J.h[i] = (T)hh;
+    if (J.l) J.l[i] = ll;
+    if (J.ew) J.ew[i] = (T)exp(ll);
+    if (J.fac) {
+      const double f = exp((J.fshift ? J.fshift[i] : 0.0) + ll);
+      J.fac[i] = f;
+      if (J.w0) J.w0[i] = (T)f;
+      if (J.w1) J.w1[i] = (T)(f * J.wx[i]);
+    }
   }
 }
+// Both sides in one launch: the first `ba` CTAs split the rows, the rest the columns
+// (each side's split alone takes about 4 us, nearly all of it launch and latency).
+// alpha_dev (nullable): alpha read on the device (a line-search step decided there).
+// sc (nullable): gamma and the points' bound are written here by the way.
 template <class T>
-__global__ void split_kernel(int64_t n, const double* x, const double* y, double alpha,
-                             const double* z, int plain, T* h, double* l, T* ew, double* fac,
-                             const double* fshift, int* status) {
+__global__ void split_pair_kernel(SplitJob<T> a, SplitJob<T> b, int ba, const double* alpha_dev, int plain, int* status,
+                                  double* sc, double gamma, double dmax) {
   pdl_wait();
-  split_range<T>(n, x, y, alpha, z, plain, h, l, ew, fac, fshift, status);
-}
-// The same split with alpha read on the device (a line-search step decided there).
-template <class T>
-__global__ void split_dev_kernel(int64_t n, const double* x, const double* y, const double* alpha,
-                                 const double* z, int plain, T* h, double* l, T* ew, double* fac,
-                                 const double* fshift, int* status) {
-  pdl_wait();
-  split_range<T>(n, x, y, *alpha, z, plain, h, l, ew, fac, fshift, status);
+  if (sc && blockIdx.x == 0 && threadIdx.x == 0) {
+    sc[SC_GAMMA] = gamma;
+    sc[SC_DMAX] = dmax;
+  }
+  const bool rows = (int)blockIdx.x < ba;
+  const SplitJob<T>& J = rows ? a : b;
+  split_range<T>(J, alpha_dev ? *alpha_dev : J.alpha, plain, status, rows ? blockIdx.x : blockIdx.x - ba,
+                 rows ? ba : (int)gridDim.x - ba);
 }
 
 // Deterministic grid reduction of up to two per-thread values: warp sums, then
@@ -1093,6 +1112,17 @@ static __global__ void exp_kernel(int64_t n, const double* x, double* y) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     y[i] = exp(x[i]);
+}
+
+// The same for two vectors in one launch: the first bx CTAs take (x, y), the rest (v, w).
+static __global__ void exp_pair_kernel(int64_t n, const double* x, double* y, int bx, int64_t m, const double* v,
+                                       double* w) {
+  pdl_wait();
+  const bool first = (int)blockIdx.x < bx;
+  const int64_t len = first ? n : m, b = first ? blockIdx.x : blockIdx.x - bx, nb = first ? bx : gridDim.x - bx;
+  const double* in = first ? x : v;
+  double* out = first ? y : w;
+  for (int64_t i = b * blockDim.x + threadIdx.x; i < len; i += nb * blockDim.x) out[i] = exp(in[i]);
 }
 
 // y *= *s (nullable s: no-op): applies a device-resident scale, e.g. the

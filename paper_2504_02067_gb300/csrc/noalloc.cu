@@ -126,13 +126,21 @@ void marginals_noalloc(const eot_problem* P, const double* u, const double* v, d
   a.active = nullptr;
   a.keep_l2 = 0;
 
-  // log r(P) = LSE_j(u_i + v_j - gamma C_ij): rows split, columns split with weights exp(Bl)
-  launch_k(split_kernel<T>, dim3(vg_n), dim3(kThreads), st, n, u, (const double*)nullptr, 0.0,
-           (const double*)nullptr, plain ? 1 : 0, Ah, Al, (T*)nullptr, (double*)nullptr,
-           (const double*)nullptr, status);
-  launch_k(split_kernel<T>, dim3(vg_m), dim3(kThreads), st, m, v, (const double*)nullptr, 0.0,
-           (const double*)nullptr, plain ? 1 : 0, Bh, Bl, ewc, (double*)nullptr,
-           (const double*)nullptr, status);
+  // one split serves both sweeps: log r(P) = LSE_j(u_i + v_j - gamma C_ij) with the column
+  // weights exp(Bl), log c(P) = LSE_i(...) with the row weights exp(Al)
+  SplitJob<T> jr, jc;
+  jr.n = n;
+  jr.x = u;
+  jr.h = Ah;
+  jr.l = Al;
+  jr.ew = ewr;
+  jc.n = m;
+  jc.x = v;
+  jc.h = Bh;
+  jc.l = Bl;
+  jc.ew = ewc;
+  launch_k(split_pair_kernel<T>, dim3(vg_n + vg_m), dim3(kThreads), st, jr, jc, vg_n, (const double*)nullptr,
+           plain ? 1 : 0, status, (double*)nullptr, 0.0, 0.0);
   {
     SweepArgs<T> ar = a;
     ar.wc[0] = ewc;
@@ -141,10 +149,6 @@ void marginals_noalloc(const eot_problem* P, const double* u, const double* v, d
     if (V == VEC) launch_k(row_sweep_kernel<T, VEC, 1, true, 0, RowLseEpi>, grid, dim3(kThreads), st, ar, e);
     else launch_k(row_sweep_kernel<T, 1, 1, true, 0, RowLseEpi>, grid, dim3(kThreads), st, ar, e);
   }
-  // log c(P) = LSE_i(u_i + v_j - gamma C_ij): rows split with weights exp(Al)
-  launch_k(split_kernel<T>, dim3(vg_n), dim3(kThreads), st, n, u, (const double*)nullptr, 0.0,
-           (const double*)nullptr, plain ? 1 : 0, Ah, Al, ewr, (double*)nullptr,
-           (const double*)nullptr, status);
   {
     SweepArgs<T> ac = a;
     ac.wr[0] = ewr;

@@ -196,7 +196,10 @@ struct Solver {
   // computed s_C gives the maximum itself; for a caller's s_C the clouds' extent
   // bounds it, which takes a read back (not possible when the call must stay
   // asynchronous).
-  void begin(double gamma, bool may_sync = true, bool gradients = false) {
+  // defer: the next split's launch writes gamma (the caller splits before any sweep).
+  bool pending = false;
+  double dmax_host = 0.0;
+  void begin(double gamma, bool defer, bool may_sync = true, bool gradients = false) {
     gamma_host = gamma;
     double dmax = 0.0;
     pg_on = pg_grad = false;
@@ -206,6 +209,9 @@ struct Solver {
       pg_grad = dmax > 0.0 && gamma * sC * pg::kLog2eD * dmax <= pg::kMaxBound;
       pg_on = pg_grad && d <= pg::kMaxD;
     }
+    dmax_host = dmax;
+    pending = defer;
+    if (defer) return;
     launch_k(set_scalars_kernel, dim3(1), dim3(1), st, h->sc, (int)SC_GAMMA, gamma, (int)SC_DMAX, dmax);
     EOT_LAUNCH_CHECK();
     h->launches++;
@@ -445,26 +451,19 @@ struct Solver {
   }
 
   // ---------------- O(n) helpers ----------------
-  // Split A = x + alpha y - z (alpha_dev: read alpha on the device instead).
-  void split_rows(const double* x, const double* y, double alpha, const double* z, double* l,
-                  T* ew, double* fac, const double* fshift, const double* alpha_dev = nullptr) {
-    if (alpha_dev)
-      launch_k(split_dev_kernel<T>, dim3(vg_n), dim3(kOnThreads), st, n, x, y, alpha_dev, z, plain ? 1 : 0, Ah(), l,
-               ew, fac, fshift, h->status);
-    else
-      launch_k(split_kernel<T>, dim3(vg_n), dim3(kOnThreads), st, n, x, y, alpha, z, plain ? 1 : 0, Ah(), l, ew, fac,
-               fshift, h->status);
-    EOT_LAUNCH_CHECK();
-    h->launches++;
-  }
-  void split_cols(const double* x, const double* y, double alpha, const double* z, double* l,
-                  T* ew, double* fac, const double* fshift, const double* alpha_dev = nullptr) {
-    if (alpha_dev)
-      launch_k(split_dev_kernel<T>, dim3(vg_m), dim3(kOnThreads), st, m, x, y, alpha_dev, z, plain ? 1 : 0, Bh(), l,
-               ew, fac, fshift, h->status);
-    else
-      launch_k(split_kernel<T>, dim3(vg_m), dim3(kOnThreads), st, m, x, y, alpha, z, plain ? 1 : 0, Bh(), l, ew, fac,
-               fshift, h->status);
+  // The exponent splits of both sides in one launch (jr.h, jc.h, sizes and low parts
+  // are filled in here).
+  using Job = SplitJob<T>;
+  void split(Job jr, Job jc, const double* alpha_dev = nullptr) {
+    jr.n = n;
+    jr.h = Ah();
+    jr.l = h->Al;
+    jc.n = m;
+    jc.h = Bh();
+    jc.l = h->Bl;
+    launch_k(split_pair_kernel<T>, dim3(vg_n + vg_m), dim3(kOnThreads), st, jr, jc, vg_n, alpha_dev, plain ? 1 : 0,
+             h->status, pending ? h->sc : nullptr, gamma_host, dmax_host);
+    pending = false;
     EOT_LAUNCH_CHECK();
     h->launches++;
   }
@@ -646,8 +645,15 @@ struct Solver {
 
   void row_lse(const double* u, const double* v, const double* rshift, double* out_lse,
                double* out_max, const double* rt, int s0 = SC_GL1, int s1 = SC_CHI2) {
-    split_rows(u, nullptr, 0.0, rshift, h->Al, nullptr, nullptr, nullptr);
-    split_cols(v, nullptr, 0.0, nullptr, h->Bl, ewc(), nullptr, nullptr);
+    Job jr, jc;
+    jr.x = u;
+    jr.z = rshift;
+    jc.x = v;
+    jc.ew = ewc();
+    split(jr, jc);
+    row_lse_sweep(rshift, out_lse, out_max, rt, s0, s1);
+  }
+  void row_lse_sweep(const double* rshift, double* out_lse, double* out_max, const double* rt, int s0, int s1) {
     SweepArgs<T> a = args();
     a.wc[0] = ewc();
     RowLseEpi e{rshift, h->Al, out_lse, out_max, rt, h->sc, s0, s1};
@@ -660,8 +666,19 @@ struct Solver {
   void col_lse(const double* u, const double* du, const double* v, const double* dv, double alpha,
                const double* cshift, double* out, int mode, int slot, double minus,
                const double* alpha_dev = nullptr) {
-    split_rows(u, du, alpha, nullptr, h->Al, ewr(), nullptr, nullptr, alpha_dev);
-    split_cols(v, dv, alpha, cshift, h->Bl, nullptr, nullptr, nullptr, alpha_dev);
+    Job jr, jc;
+    jr.x = u;
+    jr.y = du;
+    jr.alpha = alpha;
+    jr.ew = ewr();
+    jc.x = v;
+    jc.y = dv;
+    jc.alpha = alpha;
+    jc.z = cshift;
+    split(jr, jc, alpha_dev);
+    col_lse_sweep(cshift, out, mode, slot, minus);
+  }
+  void col_lse_sweep(const double* cshift, double* out, int mode, int slot, double minus) {
     SweepArgs<T> a = args();
     a.wr[0] = ewr();
     ColLseEpi e{h->Bl, mode == 0 ? cshift : nullptr, out, mode, h->sc, slot, minus};
@@ -912,8 +929,17 @@ struct Solver {
   void emit_newton(const double* u, const double* v, const double* rt) {
     if (full_system && points) throw EotError{EOT_ERR_UNSUPPORTED, "the full-system NewtonSolve needs a dense cost"};
     // factorisation P = rowfac * colfac * E with row shift = running row max
-    split_rows(u, nullptr, 0.0, h->rowmax, h->Al, nullptr, h->rowfac, h->rowmax);
-    split_cols(v, nullptr, 0.0, nullptr, h->Bl, ewc(), h->colfac, nullptr);
+    {
+      Job jr, jc;
+      jr.x = u;
+      jr.z = h->rowmax;
+      jr.fac = h->rowfac;
+      jr.fshift = h->rowmax;
+      jc.x = v;
+      jc.ew = ewc();
+      jc.fac = h->colfac;
+      split(jr, jc);
+    }
     launch_k(prep_setup_kernel<T>, dim3(vg_n), dim3(kOnThreads), st, n, h->logrP, rt, h->rowfac, h->rP, h->du0, xw0(),
              xw1());
     EOT_LAUNCH_CHECK();

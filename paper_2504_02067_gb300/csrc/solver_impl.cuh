@@ -26,17 +26,22 @@ void run_marginals(eot_handle h, const eot_problem* P, const double* u, const do
                    double* total_out, cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.begin(round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma), true);
   double* lr = lr_out ? lr_out : h->logrP;
   double* lc = lc_out ? lc_out : h->logcP;
-  S.row_lse(u, v, nullptr, lr, nullptr, nullptr, SC_MASS, SC_AUX1);
-  S.col_lse(u, nullptr, v, nullptr, 0.0, nullptr, lc, 0, SC_AUX0, 0.0);
-  if (r_out) {
-    launch_k(exp_kernel, dim3(S.vg_n), dim3(kOnThreads), st, P->n, lr, r_out);
-    h->launches++;
-  }
-  if (c_out) {
-    launch_k(exp_kernel, dim3(S.vg_m), dim3(kOnThreads), st, P->m, lc, c_out);
+  // one split serves both sweeps (neither side is shifted)
+  typename Solver<T>::Job jr, jc;
+  jr.x = u;
+  jr.ew = S.ewr();
+  jc.x = v;
+  jc.ew = S.ewc();
+  S.split(jr, jc);
+  S.row_lse_sweep(nullptr, lr, nullptr, nullptr, SC_MASS, SC_AUX1);
+  S.col_lse_sweep(nullptr, lc, 0, SC_AUX0, 0.0);
+  if (r_out || c_out) {
+    const int br = r_out ? S.vg_n : 0, bc = c_out ? S.vg_m : 0;
+    launch_k(exp_pair_kernel, dim3(br + bc), dim3(kOnThreads), st, P->n, (const double*)lr, r_out, br, P->m,
+             (const double*)lc, c_out);
     h->launches++;
   }
   EOT_LAUNCH_CHECK();
@@ -52,7 +57,7 @@ void run_value(eot_handle h, const eot_problem* P, const double* u, const double
                double* value_out, cudaStream_t st) {
   Solver<T> S(h, P, st);
   const double g = round_gamma<T>(gamma);
-  S.begin(g, P->cost_scale <= 0.0);  // (asynchronous with a given s_C)
+  S.begin(g, true, P->cost_scale <= 0.0);  // (asynchronous with a given s_C)
   S.row_lse(u, v, nullptr, nullptr, nullptr, nullptr, SC_MASS, SC_AUX1);
   launch_k(dot_kernel, dim3(S.vg_n), dim3(kOnThreads), st, P->n, P->r, u, h->sc, (int)SC_AUX0, h->dotpart,
            h->cnt_dot);
@@ -70,17 +75,25 @@ void run_hvp(eot_handle h, const eot_problem* P, const double* u, const double* 
              double* c_out, cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.begin(round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma), true);
   // row maxima for the factorisation P = rowfac * colfac * E
   S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
-  S.split_rows(u, nullptr, 0.0, h->rowmax, h->Al, nullptr, h->rowfac, h->rowmax);
-  S.split_cols(v, nullptr, 0.0, nullptr, h->Bl, nullptr, h->colfac, nullptr);
-  launch_k(weight_kernel<T>, dim3(S.vg_n), dim3(kOnThreads), st, P->n, h->rowfac, nullptr, S.xw0());
-  launch_k(weight_kernel<T>, dim3(S.vg_n), dim3(kOnThreads), st, P->n, h->rowfac, du, S.xw1());
-  launch_k(weight_kernel<T>, dim3(S.vg_m), dim3(kOnThreads), st, P->m, h->colfac, nullptr, S.zf());
-  launch_k(weight_kernel<T>, dim3(S.vg_m), dim3(kOnThreads), st, P->m, h->colfac, dv, S.wsq());
-  EOT_LAUNCH_CHECK();
-  h->launches += 4;
+  {
+    typename Solver<T>::Job jr, jc;
+    jr.x = u;
+    jr.z = h->rowmax;
+    jr.fac = h->rowfac;
+    jr.fshift = h->rowmax;
+    jr.w0 = S.xw0();
+    jr.w1 = S.xw1();
+    jr.wx = du;
+    jc.x = v;
+    jc.fac = h->colfac;
+    jc.w0 = S.zf();
+    jc.w1 = S.wsq();
+    jc.wx = dv;
+    S.split(jr, jc);
+  }
   if (S.points) {
     // point costs: a row sweep (r(P), P dv) and a column sweep (c(P), P^T du), then
     // out_u = r(P) du + s P dv, out_v = s P^T du + c(P) dv
@@ -120,7 +133,7 @@ void run_newton(eot_handle h, const eot_problem* P, const double* u, const doubl
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
   if (max_cg <= 0) max_cg = (int)std::min<int64_t>(4 * (full ? P->n + P->m : P->n), 2000);
   S.init_control(1, 1, max_cg);
-  S.begin(round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma), true);
   // the program runs on the handle's buffers (a captured graph keeps their addresses)
   S.copy(h->U, u, P->n);
   S.copy(h->V, v, P->m);
@@ -154,7 +167,7 @@ void run_solve(eot_handle h, const eot_problem* P, const eot_params* prm_in, dou
   const int max_cg = prm.max_cg > 0 ? prm.max_cg : (int)std::min<int64_t>(4 * (S.full_system ? n + m : n), 2000);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
   S.init_control(prm.max_newton, prm.max_ls, max_cg);
-  S.begin(round_gamma<T>(prm.gamma_f));  // the largest temperature of the call
+  S.begin(round_gamma<T>(prm.gamma_f), false);  // the largest temperature of the call
   if (capped) {
     launch_k(set_deadline_kernel, dim3(1), dim3(1), st, h->sc, prm.max_seconds);
     EOT_LAUNCH_CHECK();
@@ -332,7 +345,7 @@ double run_sweep_bench(eot_handle h, const eot_problem* P, const double* u, cons
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
   S.retain_cost();
-  S.begin(round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma), true);
   // untimed set-up: the Newton-step factorisation and a CG start at rho = 1/2
   S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
   launch_k(exp_kernel, dim3(S.vg_n), dim3(kOnThreads), st, P->n, h->logrP, h->rt);  // r~ := r(P) (any finite target)
@@ -429,10 +442,16 @@ void run_backward_dense(eot_handle h, const eot_problem* P, const double* u, con
                         double gamma, double scale, const double* scale_dev, float* dC, cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.begin(round_gamma<T>(gamma));
+  S.begin(round_gamma<T>(gamma), true);
   S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
-  S.split_rows(u, nullptr, 0.0, h->rowmax, h->Al, nullptr, h->rowfac, h->rowmax);
-  S.split_cols(v, nullptr, 0.0, nullptr, h->Bl, nullptr, h->colfac, nullptr);
+  typename Solver<T>::Job jr, jc;
+  jr.x = u;
+  jr.z = h->rowmax;
+  jr.fac = h->rowfac;
+  jr.fshift = h->rowmax;
+  jc.x = v;
+  jc.fac = h->colfac;
+  S.split(jr, jc);
   if (scale_dev) {
     launch_k(scale_by_dev_kernel, dim3(S.vg_n), dim3(kOnThreads), st, P->n, h->rowfac, scale_dev);
     h->launches++;
@@ -457,12 +476,18 @@ void run_backward_points(eot_handle h, const eot_problem* P, const double* u, co
                          cudaStream_t st) {
   Solver<T> S(h, P, st);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
-  S.begin(round_gamma<T>(gamma), true, true);
+  S.begin(round_gamma<T>(gamma), true, true, true);
   const double f = scale * 2.0 * S.sC;
   if (dX) {
     S.row_lse(u, v, nullptr, h->logrP, h->rowmax, nullptr, SC_AUX0, SC_AUX1);
-    S.split_rows(u, nullptr, 0.0, h->logrP, h->Al, nullptr, h->rowfac, h->logrP);
-    S.split_cols(v, nullptr, 0.0, nullptr, h->Bl, S.ewc(), nullptr, nullptr);
+    typename Solver<T>::Job jr, jc;
+    jr.x = u;
+    jr.z = h->logrP;
+    jr.fac = h->rowfac;
+    jr.fshift = h->logrP;
+    jc.x = v;
+    jc.ew = S.ewc();
+    S.split(jr, jc);
     if (scale_dev) {
       launch_k(scale_by_dev_kernel, dim3(S.vg_n), dim3(kOnThreads), st, P->n, h->rowfac, scale_dev);
       h->launches++;
@@ -471,8 +496,14 @@ void run_backward_points(eot_handle h, const eot_problem* P, const double* u, co
   }
   if (dY) {
     S.col_lse(u, nullptr, v, nullptr, 0.0, nullptr, h->logcP, 0, SC_AUX0, 0.0);
-    S.split_rows(u, nullptr, 0.0, nullptr, h->Al, S.ewr(), nullptr, nullptr);
-    S.split_cols(v, nullptr, 0.0, h->logcP, h->Bl, nullptr, h->colfac, h->logcP);
+    typename Solver<T>::Job jr, jc;
+    jr.x = u;
+    jr.ew = S.ewr();
+    jc.x = v;
+    jc.z = h->logcP;
+    jc.fac = h->colfac;
+    jc.fshift = h->logcP;
+    S.split(jr, jc);
     if (scale_dev) {
       launch_k(scale_by_dev_kernel, dim3(S.vg_m), dim3(kOnThreads), st, P->m, h->colfac, scale_dev);
       h->launches++;

@@ -579,10 +579,11 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
         }
       }
     } else {
+    T racc[U * (NR > 0 ? NR : 1)];  // row sums of the batch: [row][reduction]
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (i0 + (int64_t)u * kWarps >= r1) continue;
       T racc0 = T(0), racc1 = T(0);
+      if (i0 + (int64_t)u * kWarps < r1) {
 #pragma unroll
       for (int e = 0; e < V; ++e) {
         if constexpr (!LSE) {
@@ -594,16 +595,19 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
           if constexpr (NR > 1) racc1 = fmaT(x, wcv[1][e], racc1);
         }
       }
-      if constexpr (NR > 0) {
-        const double rs0 = warp_sum_t(racc0);
-        double rs1 = 0.0;
-        if constexpr (NR > 1) rs1 = warp_sum_t(racc1);
-        if (lane == 0) {
-          const int64_t i = i0 + (int64_t)u * kWarps;
-          a.rowpart[(0 * S + strip) * a.n + i] = rs0;
-          if constexpr (NR > 1) a.rowpart[(1 * S + strip) * a.n + i] = rs1;
-        }
       }
+      if constexpr (NR > 0) {
+        racc[u * NR] = racc0;
+        if constexpr (NR > 1) racc[u * NR + 1] = racc1;
+      }
+    }
+    if constexpr (NR > 0) {
+      // (a row beyond r1 holds zeros and is not stored)
+      const T rs = warp_sum_many<U * NR>(racc);
+      constexpr int LPV = 32 / (U * NR);  // lanes per value
+      const int k = lane / LPV;
+      const int64_t i = i0 + (int64_t)(k / NR) * kWarps;
+      if (lane % LPV == 0 && i < r1) a.rowpart[((int64_t)(k % NR) * S + strip) * a.n + i] = (double)rs;
     }
     }
 #pragma unroll
@@ -808,7 +812,7 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
 #pragma unroll
         for (int k = 0; k < NR; ++k) {
           double t = 0.0;
-          ordered_loads(a.rowpart + (int64_t)k * S * a.n + i, a.n, S, [&](double q) { t += q; });
+          ordered_loads<32>(a.rowpart + (int64_t)k * S * a.n + i, a.n, S, [&](double q) { t += q; });
           s[k] = t;
         }
         epi.row_part(i, s);
