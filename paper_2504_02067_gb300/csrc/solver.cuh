@@ -780,7 +780,7 @@ struct Solver {
     ctl.sc = h->sc;
     ctl.status = h->status;
     ctl.fp64 = sizeof(T) == 8 ? 1 : 0;
-    ctl.fused_cg = (points || full_system) ? 0 : 1;
+    ctl.fused_cg = ((points && !pg_on) || full_system) ? 0 : 1;
     ctl.floor32 = armijo_floor32(n, m);
     int64_t* saved = sweep_bucket;
     sweep_bucket = &discard;
@@ -964,7 +964,7 @@ struct Solver {
       emit_full_cg(rt);
     } else {
       loop_while(F_CGOUT, [&] {
-        if (points)
+        if (points && !pg_on)
           launch_k(cg_init_kernel<T>, dim3(vg_n), dim3(kOnThreads), st, n, h->rP, h->rPs, rt, h->diag, h->rowfac,
                    h->M, h->x, h->res, h->z, h->p, h->Yx, xw0(), h->sc, h->dotpart, h->cnt_dot, cond(F_CG));
         else
@@ -1053,31 +1053,46 @@ struct Solver {
   }
 
   // One CG iteration, each kernel a no-op once the device stop flag SC_ACTIVE
-  // is clear. Dense costs: the column half (which also takes beta and the stop
-  // test), the row half (which forms p) and the update (CgColFusedEpi,
-  // CgRowFusedEpi, cg_update_fused_kernel); the column half's stop goes to
+  // is clear. Dense costs and split-coordinate points: the column half (which also
+  // takes beta and the stop test), the row half (which forms p) and the update
+  // (CgColFusedEpi, CgRowFusedEpi or PgCgColEpi, PgCgRowEpi, and
+  // cg_update_fused_kernel); the column half's stop goes to
   // SC_ACTIVE_COL, which the row half reads and the update commits to
-  // SC_ACTIVE. Point costs: column half, row half, update, p update.
+  // SC_ACTIVE. Other point sweeps: column half, row half, update, p update.
   void cg_iteration() {
-    if (!points) {
-      {
+    if (!points || pg_on) {
+      int nrow = rg;  // partials of <p, q>
+      if constexpr (sizeof(T) == 4) {
+        if (pg_on) {
+          SweepArgs<T> a = args();
+          a.wr[0] = xw0();
+          a.active = h->sc + SC_ACTIVE;
+          launch_pg<1, false, 0, false, false>(st, a, PgCgColEpi{h->colfac, h->cP, zf(), h->wprev, h->cgpart, vg_n,
+                                                                h->sc, h->status, cond(F_CG), (int)SC_ACTIVE_COL, 0.0,
+                                                                false});
+          SweepArgs<T> b = args();
+          b.wc[0] = zf();
+          b.active = h->sc + SC_ACTIVE_COL;
+          launch_pg<1, false, 0, true, false>(st, b, PgCgRowEpi{h->rowfac, h->rPs, h->z, h->p, h->y, h->q, h->sc});
+          const pg::Geo g = pg::geo_of(h->sms, n, m, d, false);
+          nrow = (int)(g.B * g.S);
+        }
+      }
+      if (!points) {
         SweepArgs<T> a = args();
         a.wr[0] = xw0();
         a.active = h->sc + SC_ACTIVE;
         CgColFusedEpi<T> e{h->colfac, h->cP, zf(), h->wprev, h->cgpart, vg_n, h->sc, h->status, cond(F_CG), 0.0,
                            false, 0, (int)SC_ACTIVE_COL};
         launch_cg_col(st, a, e);
-      }
-      {
-        SweepArgs<T> a = args();
-        a.wc[0] = zf();
-        a.active = h->sc + SC_ACTIVE_COL;
-        CgRowFusedEpi e{h->rowfac, h->rPs, h->z, h->p, h->y, h->q, h->sc};
-        launch_row_dense<1, false, 0>(st, a, e);
+        SweepArgs<T> b = args();
+        b.wc[0] = zf();
+        b.active = h->sc + SC_ACTIVE_COL;
+        launch_row_dense<1, false, 0>(st, b, CgRowFusedEpi{h->rowfac, h->rPs, h->z, h->p, h->y, h->q, h->sc});
       }
       launch_k(cg_update_fused_kernel<T>, dim3(vg_n), dim3(kOnThreads), st, n, (const double*)h->p,
                (const double*)h->q, (const double*)h->y, (const double*)h->M, (const double*)h->rowfac, h->x, h->res,
-               h->Yx, h->z, xw0(), h->sc, (const double*)h->dotpart, rg, h->cgpart, h->status, (int)SC_ACTIVE_COL,
+               h->Yx, h->z, xw0(), h->sc, (const double*)h->dotpart, nrow, h->cgpart, h->status, (int)SC_ACTIVE_COL,
                cond(F_CG));
       EOT_LAUNCH_CHECK();
       h->launches += 3;

@@ -73,6 +73,11 @@ template <class E, class = void>
 struct HasRowPrefetch : std::false_type {};
 template <class E>
 struct HasRowPrefetch<E, std::void_t<decltype(E::kRowPrefetch)>> : std::bool_constant<E::kRowPrefetch> {};
+// point sweeps whose epilogue takes beta and the stop test while the CTA stages
+template <class E, class = void>
+struct HasPrepare : std::false_type {};
+template <class E>
+struct HasPrepare<E, std::void_t<decltype(E::kPrepare)>> : std::bool_constant<E::kPrepare> {};
 template <class E, class = void>
 struct HasPrefetch : std::false_type {};
 template <class E>

@@ -322,6 +322,8 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(SweepArgs<float> a, 
   __shared__ __align__(16) unsigned char buf[kRec > kRed ? kRec : kRed];
   __shared__ float rmx[LSE ? kThreads * RO : 1];
   __shared__ Scale sc_s;
+  __shared__ double beta_s;
+  __shared__ int first_s;
   float(*rec)[REC] = reinterpret_cast<float(*)[REC]>(buf);
   float2(*red)[kThreads * RO] = reinterpret_cast<float2(*)[kThreads * RO]>(buf);  // (after the sweep)
 
@@ -339,8 +341,15 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(SweepArgs<float> a, 
   pdl_wait();
   if (a.active && *a.active == 0.0) return;  // (no CTA changes it before all have read it: the cluster stays whole)
   if (threadIdx.x == 0) sc_s = make_scale(a.gamma_dev ? *a.gamma_dev : (double)a.gamma, a.sC, *g.dmax);
+  if constexpr (HasPrepare<Epi>::value) {
+    if (threadIdx.x >= 32 && threadIdx.x < 64) epi.prepare(blk == 0 && blockIdx.y == 0, beta_s, first_s);
+  }
   __syncthreads();
   const Scale sc = sc_s;
+  if constexpr (HasPrepare<Epi>::value) {
+    epi.beta = beta_s;
+    epi.first = first_s != 0;
+  }
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ow = kWarps / g.ws, grp = warp / ow;  // warps across own elements; this warp's share of the others
