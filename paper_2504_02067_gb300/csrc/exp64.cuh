@@ -112,4 +112,17 @@ __device__ __forceinline__ double widen(float x) {
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
+constexpr float kCutMax = 1.0e30f;  // callers fall back to FP64 where |cut_f32(x)| reaches this
+// x cut (towards 0) to FP32 on the integer pipes (a conversion instruction would
+// run at the FP64 pipe's rate); |x| < 2^-126 gives 0, |x| >= 2^128 +-inf, NaN NaN
+__device__ __forceinline__ float cut_f32(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t a = hi & 0x7fffffffu;
+  uint32_t r = __funnelshift_l(lo, a - (896u << 20), 3);
+  if (a < (897u << 20)) r = 0u;
+  if (a >= (1151u << 20)) r = a > 0x7ff00000u || (a == 0x7ff00000u && lo) ? 0x7fc00000u : 0x7f800000u;
+  return __uint_as_float(r | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float cut_f32(float x) { return x; }
+
 }  // namespace eot

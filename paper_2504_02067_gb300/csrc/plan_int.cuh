@@ -162,17 +162,6 @@ __global__ void __launch_bounds__(kThreads) plan_int_points_kernel(int64_t n, in
 
 constexpr float kScreenMax = 1.0e8f;
 
-// x cut (towards 0) to FP32 on the integer pipes (a conversion instruction would
-// run at the FP64 pipe's rate); |x| < 2^-126 gives 0, |x| >= 2^128 +-inf, NaN NaN
-__device__ __forceinline__ float cut_f32(double x) {
-  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-  const uint32_t a = hi & 0x7fffffffu;
-  uint32_t r = __funnelshift_l(lo, a - (896u << 20), 3);
-  if (a < (897u << 20)) r = 0u;
-  if (a >= (1151u << 20)) r = a > 0x7ff00000u || (a == 0x7ff00000u && lo) ? 0x7fc00000u : 0x7f800000u;
-  return __uint_as_float(r | (hi & 0x80000000u));
-}
-__device__ __forceinline__ float cut_f32(float x) { return x; }
 __device__ __forceinline__ float max_nan(float a, float b) {
   float r;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));

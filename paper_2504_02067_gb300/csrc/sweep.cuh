@@ -288,18 +288,10 @@ __device__ __forceinline__ void row_reduce_lse(const T (&c)[U][V], int j0, int t
     ld_vec_smem<V>(&sv[0][jl], b);
     ld_vec_smem<V>(&sv[1][jl], w);
     T tmax = T(-3.0e38);
-    bool over = sizeof(T) == 4;  // FP64: the maximum is formed only if a t may exceed theta
 #pragma unroll
     for (int e = 0; e < V; ++e) {
       t[e] = fmaT(-g, c[u][e], am + b[e]);
-      if constexpr (sizeof(T) == 4) tmax = fmax(tmax, t[e]);
-      else over |= maybe_above(t[e], T(kTheta));
-    }
-    if constexpr (sizeof(T) == 8) {
-      if (over) {
-#pragma unroll
-        for (int e = 0; e < V; ++e) tmax = fmax(tmax, t[e]);
-      }
+      tmax = fmax(tmax, t[e]);
     }
     for (int k = 0; k < 4 && tmax > T(kTheta); ++k) {
       const T dlt = ceil_grid(tmax);
@@ -322,8 +314,76 @@ __device__ __forceinline__ void row_reduce_lse(const T (&c)[U][V], int j0, int t
   kadd(S, Cc, acc);
 }
 
+// The same for FP64, with one running max for the whole warp: it moves at most once or
+// twice per row (a max per lane moves in most batches of some lane, and every move
+// costs the warp dozens of FP64 instructions), and the candidates are compared as FP32
+// on the integer pipes. Warp-uniform: every lane takes part in every batch.
+template <int V, int U, int NV, int TW>
+__device__ __forceinline__ void row_reduce_lse64(const double (&c)[U][V], int j0, int tw, double ah, double g,
+                                                 const double (&sv)[NV][TW], double& mx, bool& set, double& am,
+                                                 double& S, const ExpSmem<double>& ex) {
+  double t[U][V];
+  bool over = false;
+  auto form = [&] {
+    over = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int jl = j0 + u * 32 * V;
+      if (jl >= tw) continue;
+      double b[V];
+      ld_vec_smem<V>(&sv[0][jl], b);
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        t[u][e] = fma(-g, c[u][e], am + b[e]);
+        over |= maybe_above(t[u][e], (double)kTheta);
+      }
+    }
+  };
+  form();
+  for (int k = 0; k < 4 && __any_sync(0xffffffffu, over || !set); ++k) {
+    float m = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (j0 + u * 32 * V >= tw) continue;
+#pragma unroll
+      for (int e = 0; e < V; ++e) m = fmaxf(m, cut_f32(t[u][e]));
+    }
+    m = warp_max_f(m);
+    double dlt = (double)ceil_grid(m);
+    if (!(fabsf(m) < kCutMax)) {  // beyond FP32's range: the maximum in FP64
+      double md = -INFINITY;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (j0 + u * 32 * V >= tw) continue;
+#pragma unroll
+        for (int e = 0; e < V; ++e) md = fmax(md, t[u][e]);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) md = fmax(md, __shfl_xor_sync(0xffffffffu, md, o));
+      dlt = ceil_grid(md);
+    }
+    if (!isfinite(dlt) || (set && dlt <= 0.0)) break;  // nothing finite to move to
+    mx += dlt;
+    am = ah - mx;
+    if (set) S *= ex(-dlt);
+    set = true;
+    form();
+  }
+  double acc = 0.0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int jl = j0 + u * 32 * V;
+    if (jl >= tw) continue;
+    double w[V];
+    ld_vec_smem<V>(&sv[1][jl], w);
+#pragma unroll
+    for (int e = 0; e < V; ++e) acc = fma(ex(t[u][e]), w[e], acc);
+  }
+  S += acc;
+}
+
 template <class T, int V, int NR, bool LSE, int SQM, class Epi>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) row_sweep_kernel(SweepArgs<T> a, Epi epi) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : (LSE ? 2 : 3)) row_sweep_kernel(SweepArgs<T> a, Epi epi) {
   constexpr int U = 4;                               // chunks per batch (two batches in flight)
   constexpr int NV = 1 + (LSE ? 1 : NR);             // staged column vectors
   // tile width (<= 32 KB smem; FP64: 24 KB beside the exponential's table), a multiple of
@@ -392,9 +452,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) row_sweep_ke
     if (!rv) continue;
     const T* ct = crow + t0;
     int j0 = lane * V;
-    if (j0 >= tw) continue;
+    constexpr bool UNI = LSE && sizeof(T) == 8;  // warp-uniform batches
+    const int jo = UNI ? lane * V : 0;           // a batch runs while its first (UNI: the warp's first) entry is inside
+    if (j0 - jo >= tw) continue;
     if (t0 > 0) row_load<T, V, U>(ct, j0, tw, cA, pol);  // tile 0 was prefetched
-    if constexpr (LSE) {
+    if constexpr (LSE && !UNI) {
       if (!mx_set) {
         // start the running max at the lane's first element, so that the
         // dominant terms cannot underflow against a far-away start value
@@ -404,17 +466,20 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3) row_sweep_ke
         mx_set = true;
       }
     }
+    auto reduce = [&](const T (&c)[U][V], int j) {
+      if constexpr (!LSE) row_reduce_sum<T, V, U, NR, SQM, NV, TW>(c, j, tw, ah, g, sv, S, Cc, ex);
+      else if constexpr (UNI) row_reduce_lse64<V, U, NV, TW>(c, j, tw, ah, g, sv, mx, mx_set, am, S[0], ex);
+      else row_reduce_lse<T, V, U, NV, TW>(c, j, tw, ah, g, sv, mx, am, S[0], Cc[0], ex);
+    };
     for (;;) {
       const int j1 = j0 + STEP;
       if (j1 < tw) row_load<T, V, U>(ct, j1, tw, cB, pol);
-      if constexpr (!LSE) row_reduce_sum<T, V, U, NR, SQM, NV, TW>(cA, j0, tw, ah, g, sv, S, Cc, ex);
-      else row_reduce_lse<T, V, U, NV, TW>(cA, j0, tw, ah, g, sv, mx, am, S[0], Cc[0], ex);
-      if (j1 >= tw) break;
+      reduce(cA, j0);
+      if (j1 - jo >= tw) break;
       const int j2 = j1 + STEP;
       if (j2 < tw) row_load<T, V, U>(ct, j2, tw, cA, pol);
-      if constexpr (!LSE) row_reduce_sum<T, V, U, NR, SQM, NV, TW>(cB, j1, tw, ah, g, sv, S, Cc, ex);
-      else row_reduce_lse<T, V, U, NV, TW>(cB, j1, tw, ah, g, sv, mx, am, S[0], Cc[0], ex);
-      if (j2 >= tw) break;
+      reduce(cB, j1);
+      if (j2 - jo >= tw) break;
       j0 = j2;
     }
   }
@@ -546,37 +611,44 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
 #pragma unroll
         for (int e = 0; e < V; ++e) {
           T t[U];
-          T tmax = T(-3.0e38);
+          float tmax = -3.0e38f;  // (FP64: compared as FP32, on the integer pipes, if at all)
           bool over = false;
+          auto form = [&] {
+            tmax = -3.0e38f;
+            over = false;
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            t[u] = fmaT(-g, c[u][e], hh[u] + bm[e]);
-            if constexpr (sizeof(T) == 4) {
-              if (i0 + (int64_t)u * kWarps < r1) tmax = fmax(tmax, t[u]);
-            } else {
-              over |= i0 + (int64_t)u * kWarps < r1 && maybe_above(t[u], T(kTheta));
+            for (int u = 0; u < U; ++u) {
+              t[u] = fmaT(-g, c[u][e], hh[u] + bm[e]);
+              if (i0 + (int64_t)u * kWarps >= r1) continue;
+              if constexpr (sizeof(T) == 4) tmax = fmaxf(tmax, t[u]);
+              else over |= maybe_above(t[u], T(kTheta));
             }
-          }
-          if constexpr (sizeof(T) == 8) {
-            if (over) {
+            if constexpr (sizeof(T) == 8) {
+              if (over) {
 #pragma unroll
-              for (int u = 0; u < U; ++u)
-                if (i0 + (int64_t)u * kWarps < r1) tmax = fmax(tmax, t[u]);
+                for (int u = 0; u < U; ++u)
+                  if (i0 + (int64_t)u * kWarps < r1) tmax = fmaxf(tmax, cut_f32(t[u]));
+              }
             }
-          }
-          for (int k = 0; k < 4 && tmax > T(kTheta); ++k) {
-            const T dlt = ceil_grid(tmax);
+          };
+          form();
+          for (int k = 0; k < 4 && tmax > kTheta; ++k) {
+            T dlt = (T)ceil_grid(tmax);
+            if constexpr (sizeof(T) == 8) {
+              if (!(tmax < kCutMax)) {  // beyond FP32's range
+                dlt = t[0];
+#pragma unroll
+                for (int u = 1; u < U; ++u)
+                  if (i0 + (int64_t)u * kWarps < r1) dlt = fmax(dlt, t[u]);
+                dlt = ceil_grid(dlt);
+              }
+            }
             mx[e] += dlt;
             bm[e] = b[e] - mx[e];
             const T f = ex(-dlt);
             tot[1][e] *= f;
             cmp[1][e] *= f;
-            tmax = T(-3.0e38);
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              t[u] = fmaT(-g, c[u][e], hh[u] + bm[e]);
-              if (i0 + (int64_t)u * kWarps < r1) tmax = fmax(tmax, t[u]);
-            }
+            form();
           }
 #pragma unroll
           for (int u = 0; u < U; ++u)
@@ -629,7 +701,15 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
       if (jv) {
 #pragma unroll
         for (int e = 0; e < V; ++e) {
-          mx[e] = ceil_grid(fmaT(-g, cA[0][e], hA[0] + b[e]));
+          if constexpr (sizeof(T) == 4) {
+            mx[e] = ceil_grid(fmaT(-g, cA[0][e], hA[0] + b[e]));
+          } else {  // FP64 (a move of the max costs more): the first batch's largest
+            float m = -3.0e38f;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+              if (i0 + (int64_t)u * kWarps < r1) m = fmaxf(m, cut_f32(fmaT(-g, cA[u][e], hA[u] + b[e])));
+            mx[e] = fabsf(m) < kCutMax ? (T)ceil_grid(m) : ceil_grid(fmaT(-g, cA[0][e], hA[0] + b[e]));
+          }
           bm[e] = b[e] - mx[e];
         }
       }
