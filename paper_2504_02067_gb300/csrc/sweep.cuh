@@ -807,10 +807,19 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
           a.colpart[((int64_t)k * R + rb) * a.m + jj] = t;
         }
       } else {
-        LsePair p{0.0, 0.0};
-        for (int w = 0; w < kWarps; ++w) p = lse_combine<T>(p, LsePair{smax[w][cc], sred[1][w][cc]}, ex);
-        a.colpart[((int64_t)0 * R + rb) * a.m + jj] = p.m;
-        a.colpart[((int64_t)1 * R + rb) * a.m + jj] = p.s;
+        // the common maximum first, then independent rescalings (a chain of pairwise
+        // combines waits for two exponentials at every step)
+        double M = -INFINITY, t = 0.0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w)
+          if (sred[1][w][cc] != 0.0) M = fmax(M, smax[w][cc]);
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+          const double q = sred[1][w][cc];
+          if (q != 0.0) t += q * ex((T)(smax[w][cc] - M));
+        }
+        a.colpart[((int64_t)0 * R + rb) * a.m + jj] = M == -INFINITY ? 0.0 : M;
+        a.colpart[((int64_t)1 * R + rb) * a.m + jj] = t;
       }
     }
   }
@@ -873,10 +882,14 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
         }
         epi.col(jj, s, d.v);
       } else {
-        LsePair p{0.0, 0.0};
-        ordered_loads2(a.colpart + jj, a.colpart + (int64_t)R * a.m + jj, a.m, R,
-                       [&](double qm, double qs) { p = lse_combine<T>(p, LsePair{qm, qs}, ex); });
-        epi.col_lse(jj, p.m, p.s, d.v);
+        double M = -INFINITY, t = 0.0;
+        ordered_loads2<16>(a.colpart + jj, a.colpart + (int64_t)R * a.m + jj, a.m, R, [&](double qm, double qs) {
+          if (qs != 0.0) M = fmax(M, qm);
+        });
+        ordered_loads2<16>(a.colpart + jj, a.colpart + (int64_t)R * a.m + jj, a.m, R, [&](double qm, double qs) {
+          if (qs != 0.0) t += qs * ex((T)(qm - M));
+        });
+        epi.col_lse(jj, M == -INFINITY ? 0.0 : M, t, d.v);
       }
 #pragma unroll
       for (int k = 0; k < ND; ++k) wd[k] += d.v[k];
