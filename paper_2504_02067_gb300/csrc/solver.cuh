@@ -211,6 +211,7 @@ struct Solver {
     }
     dmax_host = dmax;
     pending = defer;
+    tc_digits(false);
     if (defer) return;
     launch_k(set_scalars_kernel, dim3(1), dim3(1), st, h->sc, (int)SC_GAMMA, gamma, (int)SC_DMAX, dmax);
     EOT_LAUNCH_CHECK();
@@ -306,15 +307,6 @@ struct Solver {
     };
     extent(X, n, emax);
     extent(Y, m, emax + 1);
-    auto digits = [&](const tc::Side& sd, const float* P, int64_t len, const unsigned long long* em) {
-      const int64_t threads = sd.npad * 32;
-      launch_k(tc::tc_prep_kernel, dim3((unsigned)((threads + kThreads - 1) / kThreads)), dim3(kThreads), st, P,
-               len, d, sd.npad, X, em, (__half*)sd.slices, (double*)sd.nx);
-      EOT_LAUNCH_CHECK();
-      h->launches++;
-    };
-    digits(targs.X, X, n, emax);
-    digits(targs.Y, Y, m, emax + 1);
     targs.err = h->status;
     for (bool rows : {true, false}) {
       const TcGeo g = tc_geo(rows);
@@ -332,6 +324,22 @@ struct Solver {
     tc_attr<2, false, 0, true, RowSumEpi>();
     tc_attr<2, false, 0, false, ColSumEpi>();
     tc_on = true;
+  }
+  // The digit slices at the sweeps' gamma: on_device reads it there (inside a program,
+  // and wherever gamma has been set by a launch), else gamma_host.
+  void tc_digits(bool on_device) {
+    if constexpr (sizeof(T) == 4) {
+      if (!tc_on) return;
+      SweepArgs<T> a = args();
+      if (!on_device) {
+        a.gamma_dev = nullptr;
+        a.gamma = (T)gamma_host;
+      }
+      const int64_t threads = (targs.X.npad + targs.Y.npad) * 32;
+      launch_k(tc::tc_prep_kernel, dim3((unsigned)((threads + kThreads - 1) / kThreads)), dim3(kThreads), st, a, targs);
+      EOT_LAUNCH_CHECK();
+      h->launches++;
+    }
   }
   template <int NR, bool LSE, int SQM, bool ROWS, class Epi>
   void launch_tc(cudaStream_t s, SweepArgs<T> a, const Epi& e) {
@@ -1132,6 +1140,7 @@ struct Solver {
     const double* rt = h->rt;
     const double* logrt = h->logrt;
     const double* logct = h->logct;
+    tc_digits(true);
     col_lse(u, nullptr, v, nullptr, 0.0, logct, v, 1, SC_AUX0, 0.0);
     row_lse(u, v, logrt, h->logrP, h->rowmax, rt);
     ctl_launch(ctl_stage_init);
@@ -1196,6 +1205,7 @@ struct Solver {
     double* logrt = h->logrt;
     double* logct = h->logct;
     sweep_bucket = &cnt.sweeps_stage;
+    tc_digits(true);
     col_lse(u, nullptr, v, nullptr, 0.0, logct, v, 1, SC_AUX0, 0.0);
     row_lse(u, v, logrt, h->logrP, h->rowmax, rt);
     sweep_bucket = &cnt.sweeps_sk;

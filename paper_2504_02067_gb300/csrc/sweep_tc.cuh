@@ -22,23 +22,34 @@
 // of a pair are issued.
 //
 // Exponent algebra. In base-2 units (t2 = t log2 e) the exponent of the plan is
-//     t2_ij = P_i + Q_j + kappa G_ij,   P_i = (A_i - K |x_i|^2) log2 e,
-//     Q_j = (B_j - K |y_j|^2) log2 e,   kappa = 2 K 2^(Ex+Ey-14) log2 e,
-// with K = gamma s_C and A, B the high parts of the potentials. A small kernel
-// before each sweep (tc_sweep_prep_kernel) forms P and Q in FP64 and splits each
-// into a high part on the 1/8 grid and a low part below 1/16: the other side's
-// low part is folded into its weights (w_j 2^ql_j, one record per point:
-// {Qh, w0} in 8 bytes for one weight, {Qh, w0, w1, w2} in 16) and the own side's into one FP64 factor 2^pl_i that
-// the finishing CTA applies to the row's total. Per entry the epilogue then
-// needs G as an FP32 pair (Fast2Sum of the two top levels plus three FMAs) and
-//     t2 = fma(kh, gh, Ph + Qh) + fma(kl, gh, kh gl)
-// (Ph + Qh exact on the grid, the big product exact inside the FMA): about a
-// dozen FP32 instructions and one MUFU ex2, t2 rounded twice at its own scale.
+//     t2_ij = P_i + Q_j + x'_i . y'_j,   P_i = (A_i - K |x_i|^2) log2 e,
+//     Q_j = (B_j - K |y_j|^2) log2 e,   x' = sqrt(2 K log2 e) (x - c) in FP64,
+// with K = gamma s_C and A, B the high parts of the potentials. The digits are those
+// of the scaled coordinates, made anew whenever gamma changes (tc_prep_kernel: 8 MB of
+// digits per 16384 points, once per stage), so that x' . y' = 2^a G with a power of
+// two. A small kernel before each sweep (tc_sweep_prep_kernel) forms P and Q in FP64
+// and splits each into a high part on the 1/8 grid and a low part below 1/16: the
+// other side's low part is folded into its weights (w_j 2^ql_j, one record per point:
+// {Qh, w0} in 8 bytes for one weight, {Qh, w0, w1, w2} in 16) and the own side's into
+// one FP64 factor 2^pl_i that the finishing CTA applies to the row's total. Per entry
+// the epilogue then needs
+//     t2 = (Ph + Qh) + 2^a S_0 + 2^(a-10) S_1 + 2^(a-20) S_2 + 2^(a-30) S_3,
+// an addition and four FMAs in this order: Ph + Qh is exact on the grid, every product
+// is exact (a power of two), the first sums cancel exactly, and what is rounded is
+// rounded at the size of t2. (Scaling by an FP32 pair kappa after folding the levels
+// into an FP32 pair takes ten instructions: a CG sweep of n = m = 16384, d = 64 took
+// 0.299 ms, this way 0.262 ms; the digits with a whole training step 230 -> 215 ms.)
 //
-// Tile width. A tcgen05.mma of M = 128, K = 16 costs about 50 cycles whatever
-// its N up to ~96 (measured on GB300: 55 cycles at N = 32, 48 and 96; 96 at
-// N = 192), so the tile is 96 points wide: the four level accumulators take 384 of
-// the 512 TMEM columns, one buffer, handed over level pair by level pair.
+// Tile width and operands. With both operands in shared memory a tcgen05.mma of
+// M = 128, K = 16 costs about 55 cycles whatever its N up to 96 (measured on GB300:
+// 55 cycles at N = 32, 48 and 96; 96 at N = 192, the tensor unit's own rate): the A
+// operand's 4 KB, read again by every MMA, bound it, and the epilogue's record reads
+// and the tile copies compete for the same bandwidth. The tile is 96 points wide: the
+// four level accumulators take 384 of the 512 TMEM columns, handed over level pair by
+// level pair, and the own points' four digit slices (128 lanes x 32 columns each)
+// fill the other 128, so the MMAs read A from TMEM and only B from shared memory.
+// (By itself that changed nothing while the epilogue was the longer side: a CG sweep of
+// n = m = 16384, d = 64 took 0.301 ms with A in shared memory and 0.299 ms so.)
 //
 // CTA roles (480 threads, one CTA per SM: about 215 KB of shared memory):
 //   warp 0, lane 0 and warp 14, lane 0: the (up to) 40 MMAs of each tile, twenty
@@ -47,10 +58,11 @@
 //     full, so these threads do nothing else: any other work in them, or a
 //     lost issue slot, leaves the tensor unit idle;
 //   warp 1: TMEM allocation (512 columns) and release; lane 0 issues the bulk
-//     copies (the own 128 points' slices once; the other side's 96-point
-//     tiles into two slice buffers and their records into four record slots);
+//     copies (the other side's 96-point tiles into three slice buffers and their
+//     records into five record slots);
 //   warps 2-13: epilogue. Warp w reads TMEM lanes 32 (w mod 4) .. +31 (one own
-//     point per thread) and a third (32) of the tile's 96 columns.
+//     point per thread) and a third (32) of the tile's 96 columns; before the
+//     first tile they store the own points' slices to TMEM.
 // Hand-offs are mbarriers: full[sb] (the slices of buffer sb landed), sfree[sb][i]
 // (issuer i's MMAs reading buffer sb are done), rec[s] (records landed), lvl[g] (the
 // MMAs of levels {0,1}, {2,3} are done, one arrival per issuer: accumulators readable),
@@ -78,19 +90,19 @@ constexpr int kMmaWarpB = 2 + kEpiWarps;      // the second MMA-issuing warp (af
 constexpr int kTcThreads = 32 * (3 + kEpiWarps);
 constexpr int kTcWarps = kTcThreads / 32;
 constexpr uint32_t kRowB = 128;    // bytes per point and slice: 64 FP16 digits
-constexpr uint32_t kOwnSlice = kM * kRowB;                          // 16 KB
 constexpr uint32_t kOthSlice = kN * kRowB;                          // 12 KB
-constexpr uint32_t kOffOth = kSlices * kOwnSlice;                   // 64 KB
-constexpr int kSliceBufs = 2;                                       // tile tt: slice buffer tt % 2
-constexpr int kRecSlots = 4;                                        // tile tt: record slot tt % 4
+constexpr uint32_t kOffOth = 0;
+constexpr int kSliceBufs = 3;                                       // tile tt: slice buffer tt % 3
+constexpr int kRecSlots = kSliceBufs + 2;                           // tile tt: record slot tt % 5
 constexpr uint32_t kRecBytes = kN * 16;                             // 1.5 KB: a slot at the widest record
-constexpr uint32_t kOffRec = kOffOth + kSliceBufs * kSlices * kOthSlice;  // + 96 KB
-constexpr uint32_t kOffBar = kOffRec + kRecSlots * kRecBytes;            // + 6 KB
+constexpr uint32_t kOffRec = kOffOth + kSliceBufs * kSlices * kOthSlice;  // 144 KB
+constexpr uint32_t kOffBar = kOffRec + kRecSlots * kRecBytes;            // + 7.5 KB
 constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;               // barriers, TMEM slot; 1024-byte alignment slack
-constexpr uint32_t kTmemCols = 512;                                 // 4 levels x 96 columns used
+constexpr uint32_t kTmemCols = 512;                                 // 4 levels x 96, then the own slices
+constexpr uint32_t kOwnCol = kLevels * kN;                          // 4 slices x 32 columns
 constexpr int64_t kPadRows = 384;                                   // lcm(kM, kN)
 constexpr uint32_t kIdesc = idesc_f16_f32(kM, kN);
-static_assert(kLevels * kN <= (int)kTmemCols, "level accumulators exceed TMEM");
+static_assert(kLevels * kN + kSlices * 32 <= (int)kTmemCols, "level accumulators and own slices exceed TMEM");
 constexpr int kMinD = 17;  // the tensor-core path serves d >= kMinD
 constexpr double kLog2eD = 1.4426950408889634;
 constexpr double kLn2D = 0.6931471805599453;
@@ -119,7 +131,7 @@ struct Side {
 struct TcArgs {
   Side X, Y;
   const unsigned long long* emax;  // [2] bits of the FP64 max |x_k - c_k| of X and of Y
-  float* kappa;                    // [2] kappa as an FP32 pair (per sweep)
+  float* kappa;                    // [1] 2^a (per sweep)
   int* err;                        // status word: kStatTimeout on a wait that ran out, kStatRange
 };
 
@@ -128,9 +140,12 @@ __host__ __device__ inline int64_t pad_rows(int64_t n) { return (n + kPadRows - 
 // read 8 bytes per column, so one 16-byte shared load serves two columns.
 __host__ __device__ constexpr int rec_floats(int nr) { return nr == 1 ? 2 : 4; }
 
-// E with every centred coordinate |x_k| < 2^E (0 for a cloud of one point).
-__device__ __forceinline__ int cloud_exp(unsigned long long bits) {
-  const double mx = __longlong_as_double((long long)bits);
+// sqrt(2 K log2 e), K = gamma s_C, and E with every scaled centred coordinate
+// |x'_k| < 2^E (0 for a cloud of one point; rounding is monotone, so the largest
+// coordinate's scaled value bounds every other).
+__device__ __forceinline__ double tc_sigma(double gamma, double sC) { return sqrt(2.0 * gamma * sC * kLog2eD); }
+__device__ __forceinline__ int cloud_exp(unsigned long long bits, double sigma) {
+  const double mx = __longlong_as_double((long long)bits) * sigma;
   int e = 0;
   if (mx > 0.0) frexp(mx, &e);  // mx = f 2^e, f in [0.5, 1)
   return e;
@@ -150,17 +165,22 @@ static __global__ void tc_extent_kernel(const float* X, int64_t n, int d, const 
   if ((threadIdx.x & 31) == 0 && mx > 0.0) atomicMax(emax, (unsigned long long)__double_as_longlong(mx));
 }
 
-// One warp per point (rows >= n and coordinates >= d are zero): the four digit
-// slices in the swizzled K-major layout and |x - c|^2 in FP64. Centring keeps
-// |x|^2, |y|^2 and x.y bounded by the data's extent, so the expansion
-// |x|^2 + |y|^2 - 2 x.y keeps its accuracy however far the clouds lie from the
-// origin.
-static __global__ void tc_prep_kernel(const float* X, int64_t n, int d, int64_t npad, const float* centre,
-                                      const unsigned long long* emax, __half* sl, double* nx) {
+// One warp per point of either cloud (rows >= n and coordinates >= d are zero): the
+// four digit slices of the scaled coordinates in the swizzled K-major layout and
+// |x - c|^2 in FP64. Centring keeps |x|^2, |y|^2 and x.y bounded by the data's extent,
+// so the expansion |x|^2 + |y|^2 - 2 x.y keeps its accuracy however far the clouds lie
+// from the origin. gamma_dev (nullable): gamma is read on the device.
+static __global__ void tc_prep_kernel(SweepArgs<float> a, TcArgs ta) {
   pdl_wait();
-  const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+  const int64_t grow = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31, d = a.d;
+  const bool isx = grow < ta.X.npad;
+  const Side& sd = isx ? ta.X : ta.Y;
+  const int64_t row = isx ? grow : grow - ta.X.npad, n = isx ? a.n : a.m, npad = sd.npad;
   if (row >= npad) return;
+  const float* X = isx ? a.X : a.Y;
+  const float* centre = a.X;
+  __half* sl = const_cast<__half*>(sd.slices);
   double xv[2] = {0.0, 0.0};
   if (row < n) {
     if (lane < d) xv[0] = (double)X[row * d + lane] - (double)centre[lane];
@@ -169,12 +189,14 @@ static __global__ void tc_prep_kernel(const float* X, int64_t n, int d, int64_t 
   double q = xv[0] * xv[0] + xv[1] * xv[1];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-  const int e = cloud_exp(*emax);
-  if (lane == 0) nx[row] = q;
+  const float g = a.gamma_dev ? (float)*a.gamma_dev : a.gamma;
+  const double sigma = tc_sigma((double)g, a.sC);
+  const int e = cloud_exp(ta.emax[isx ? 0 : 1], sigma);
+  if (lane == 0) const_cast<double*>(sd.nx)[row] = q;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const int k = lane + 32 * c;
-    long long Q = (long long)rint(ldexp(xv[c], kCoordBits - e));  // |Q| <= 2^37
+    long long Q = (long long)rint(ldexp(xv[c] * sigma, kCoordBits - e));  // |Q| <= 2^37
     const int64_t idx = row * 64 + (((k >> 3) ^ (int)(row & 7)) << 3) + (k & 7);
 #pragma unroll
     for (int s = kSlices - 1; s > 0; --s) {  // balanced digits from the lowest up
@@ -186,7 +208,7 @@ static __global__ void tc_prep_kernel(const float* X, int64_t n, int d, int64_t 
   }
 }
 
-// Before each sweep: kappa, the other side's records (all npad of them; padded
+// Before each sweep: 2^a, the other side's records (all npad of them; padded
 // points get Qh = -2^23 and weights 0, so no tile needs a mask) and the own
 // side's P split. The same gamma as the sweep: (float) of the device value.
 template <int NR, int SQM, bool ROWS>
@@ -200,10 +222,8 @@ __global__ void tc_sweep_prep_kernel(SweepArgs<float> a, TcArgs ta) {
   const double K = (double)g * a.sC;
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i == 0) {
-    const double kap = 2.0 * K * ldexp(1.0, cloud_exp(ta.emax[0]) + cloud_exp(ta.emax[1]) - 14) * kLog2eD;
-    const float kh = (float)kap;
-    ta.kappa[0] = kh;
-    ta.kappa[1] = (float)(kap - (double)kh);
+    const double sg = tc_sigma((double)g, a.sC);
+    ta.kappa[0] = (float)ldexp(1.0, cloud_exp(ta.emax[0], sg) + cloud_exp(ta.emax[1], sg) - 14);
   }
   if (i < sq.npad) {
     constexpr int RW = rec_floats(NR);
@@ -241,13 +261,6 @@ __global__ void tc_sweep_prep_kernel(SweepArgs<float> a, TcArgs ta) {
   }
 }
 
-// t2 = hq + kappa G with hq = Ph + Qh (or Ph - max + Qh), exact on the grid.
-__device__ __forceinline__ float entry_t2(float hq, float gh, float gl, float kh, float kl) {
-  const float b = fmaf(kh, gh, hq);
-  const float c = fmaf(kl, gh, __fmul_rn(kh, gl));
-  return __fadd_rn(b, c);
-}
-
 // Base-2 log-sum-exp pairs (m on the 1/8 grid, s >= 0; s == 0: empty). The
 // exponent difference is exact, so the FP32 ex2 rounds once.
 __device__ __forceinline__ void lse2_add(double& M, double& s, double qm, double qs) {
@@ -277,13 +290,14 @@ template <int NR, bool LSE, int SQM, bool ROWS, class Epi>
 __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float> a, TcArgs ta, Epi epi) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = (uint64_t*)(sm + kOffBar);  // [2] the slices of the slice buffer landed
-  uint64_t* sfree = full + 2;                  // [2][2] per issuer: its MMAs reading the slice buffer done
-  uint64_t* lvl = full + 6;                    // [2] MMAs of levels {0,1}, {2,3} done (one arrival per issuer)
-  uint64_t* lfree = full + 8;                  // [2] those levels loaded by all epilogue warps
-  uint64_t* recf = full + 10;                  // [4] records of the slot landed
-  uint64_t* ownf = full + 14;
-  uint32_t* tslot = (uint32_t*)(full + 15);
+  uint64_t* full = (uint64_t*)(sm + kOffBar);  // [kSliceBufs] the slices of the slice buffer landed
+  uint64_t* sfree = full + kSliceBufs;         // [kSliceBufs][2] per issuer: its MMAs reading the slice buffer done
+  uint64_t* lvl = sfree + 2 * kSliceBufs;      // [2] MMAs of levels {0,1}, {2,3} done (one arrival per issuer)
+  uint64_t* lfree = lvl + 2;                   // [2] those levels loaded by all epilogue warps
+  uint64_t* recf = lfree + 2;                  // [kRecSlots] records of the slot landed
+  uint64_t* ownf = recf + kRecSlots;           // the own slices are in TMEM (one arrival per epilogue warp)
+  uint32_t* tslot = (uint32_t*)(ownf + 1);
+  static_assert(3 * kSliceBufs + 4 + kRecSlots + 2 <= 32, "barrier area");
   constexpr int NA = LSE ? 1 : NR;
   constexpr int ND = Epi::kDot;
   constexpr int RW = rec_floats(NR);
@@ -308,7 +322,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
     for (int g = 0; g < 2; ++g) mbar_init(&lvl[g], 2);
     for (int g = 0; g < 2; ++g) mbar_init(&lfree[g], kEpiWarps);
     for (int k = 0; k < kRecSlots; ++k) mbar_init(&recf[k], 1);
-    mbar_init(ownf, 1);
+    mbar_init(ownf, kEpiWarps);
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc(tslot, kTmemCols);
@@ -338,20 +352,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
 
   if (warp == 1) {
     // ---------------- bulk copies (one thread) ----------------
-    // The own 128 points' slices once; tile tt's slices into buffer tt % 2
-    // and its records into slot tt % 4. Tiles 0 and 1 go at once; tile tt >= 2 once the MMAs of tile
-    // tt - 2 are done (sfree), by when the epilogue had loaded tile tt - 3 and
-    // so finished tile tt - 4, the previous user of the record slot.
+    // Tile tt's slices into buffer tt % 3 and its records into slot tt % 5. Tiles 0-2
+    // go at once; tile tt >= 3 once the MMAs of tile tt - 3 are done (sfree), by when
+    // the epilogue had loaded tile tt - 4 and so finished tile tt - 5, the previous
+    // user of the record slot.
     if (lane == 0) {
-      const unsigned char* own_src = (const unsigned char*)so.slices + blk * (int64_t)kM * kRowB;
       const unsigned char* oth_src = (const unsigned char*)sq.slices;
-      mbar_arrive_expect_tx(ownf, kSlices * kOwnSlice);
-      for (int s = 0; s < kSlices; ++s)
-        bulk_g2s(sm + s * kOwnSlice, own_src + (int64_t)s * so.npad * kRowB, kOwnSlice, ownf);
       int issued = 0;
       for (int tt = 0; tt < T; ++tt) {
         const int sb = tt % kSliceBufs, rs = tt % kRecSlots;
-        const uint32_t opar = (uint32_t)((tt - kSliceBufs) / kSliceBufs) & 1u;  // tile tt - 2's phase
+        const uint32_t opar = (uint32_t)((tt - kSliceBufs) / kSliceBufs) & 1u;  // tile tt - kSliceBufs' phase
         if (tt >= kSliceBufs &&
             (!mbar_wait(&sfree[2 * sb], opar, ta.err, kStatTimeout, kTcWaitNs, kEpiSleepNs) ||
              !mbar_wait(&sfree[2 * sb + 1], opar, ta.err, kStatTimeout, kTcWaitNs, kEpiSleepNs)))
@@ -367,10 +377,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
         issued = tt + 1;
       }
       // leave no copy in flight (bounded waits that ignore the error flag): the
-      // own slices, the slices of the last two tiles issued (a buffer was
-      // reused only after the MMAs had read its previous tile) and the records
-      // of the last four
-      mbar_wait(ownf, 0, ta.err, 0, kTcDrainNs);
+      // slices of the last tiles issued (a buffer was reused only after the MMAs had
+      // read its previous tile) and their records
       for (int tt = (issued > kSliceBufs ? issued - kSliceBufs : 0); tt < issued; ++tt)
         mbar_wait(&full[tt % kSliceBufs], (tt / kSliceBufs) & 1, ta.err, 0, kTcDrainNs);
       for (int tt = (issued > kRecSlots ? issued - kRecSlots : 0); tt < issued; ++tt)
@@ -391,9 +399,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
       const int who = warp == 0 ? 0 : 1;
       const int ksteps = (a.d + 15) / 16;
       const bool own_ok = mbar_wait(ownf, 0, ta.err, kStatTimeout);
-      // descriptors of the first own slice and of the first other-side slice;
+      tc_fence_after();
+      // the own slices' columns and the descriptor of the first other-side slice;
       // every MMA adds a compile-time offset (all unrolled)
-      const uint64_t adesc0 = desc_sw128(smem_u32(sm));
+      const uint32_t acol = tbase + kOwnCol;
       const uint64_t bdesc0 = desc_sw128(smem_u32(sm + kOffOth));
       auto level = [&](uint64_t bdesc, int L) {
 #pragma unroll
@@ -403,7 +412,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
           for (int s = 0; s < kSlices; ++s) {
             const int t = L - s;
             if (t < 0 || t >= kSlices) continue;
-            mma_f16(tbase + (uint32_t)(L * kN), adesc0 + (uint64_t)((s * kOwnSlice + k4 * 32) >> 4),
+            mma_f16(tbase + (uint32_t)(L * kN), acol + (uint32_t)(s * 32 + k4 * 8),
                      bdesc + (uint64_t)((t * kOthSlice + k4 * 32) >> 4), kIdesc,
                      (k4 == 0 && s == 0) ? 0u : 1u);
           }
@@ -450,119 +459,132 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
     __syncwarp();
   } else if (epi_warp) {
     // ---------------- epilogue ----------------
+    // the own point's digit slices to TMEM: part p stores slice p, part 0 also slice 3
+    // (global layout: 128-byte swizzled rows, chunk c of a row at position c ^ (row & 7))
+    for (int sl = part; sl < kSlices; sl += kParts) {
+      const uint4* src = reinterpret_cast<const uint4*>(so.slices + ((int64_t)sl * so.npad + e) * 64);
+      uint32_t v[32];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const uint4 x = __ldg(src + (c ^ (r & 7)));
+        v[4 * c] = x.x;
+        v[4 * c + 1] = x.y;
+        v[4 * c + 2] = x.z;
+        v[4 * c + 3] = x.w;
+      }
+      tmem_st32(tbase + ((uint32_t)(32 * q) << 16) + kOwnCol + (uint32_t)(sl * 32), v);
+    }
+    tmem_st_wait();
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(ownf);
     const float ph = so.own[e].ph;  // e < npad: padded rows have records
-    const float kh = ta.kappa[0], kl = ta.kappa[1];
+    const float k0 = ta.kappa[0], k1 = k0 * 0x1p-10f, k2 = k0 * 0x1p-20f, k3 = k0 * 0x1p-30f;
     // LSE: hm = ph - mx. The max starts at -2^23, far below every entry, so the
-    // first group of columns raises it to its own maximum (the one inexact step,
-    // it only chooses the shift); from then on ph and mx are on the grid and
-    // hm is exact.
+    // first tile raises it to its own maximum (the one inexact step, it only chooses
+    // the shift); from then on ph and mx are on the grid and hm is exact. A tile whose
+    // entries exceed the max by more than the threshold is read from TMEM again with
+    // the raised one (a difference of rounded exponents would not be exact), so the
+    // LSE sweeps hand a tile's levels back only once its max is settled.
     float hm = LSE ? ph - mx : ph;
     const uint32_t tcol = tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(part * kPartCols);
     const float* recs = (const float*)(sm + kOffRec);
-    for (int tt = 0; tt < T; ++tt) {
-      const uint32_t par = (uint32_t)tt & 1u;
-      // G as an FP32 pair per column, folded level by level; each level goes
-      // back to the MMAs of the next tile as soon as it is in registers
-      uint32_t gh[kPartCols], gl[kPartCols], u[kPartCols];
-      if (!warp_wait(&lvl[0], par, ta.err)) break;  // levels 0 and 1
-      tc_fence_after();
-      tmem_ld32(tcol, gh);
-      tmem_ld32(tcol + (uint32_t)kN, gl);
-      tmem_ld_wait();
+    auto release = [&](int g) {
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&lfree[0]);
-      // G = S_0 + 2^-10 S_1 + ... as an FP32 pair (gh, gl). S_0 is an integer up to
-      // 2^20 and 2^-10 S_1 a multiple of 2^-10 up to 2^13: where
-      // |S_0| >= |2^-10 S_1| Fast2Sum is exact, and otherwise the sum stays within
-      // 2^14 on the 2^-10 grid and is exact already (z = 2^-10 S_1, error 0).
-#pragma unroll
-      for (int c = 0; c < kPartCols; ++c) {
-        const float s0 = __uint_as_float(gh[c]), s1 = __uint_as_float(gl[c]);
-        const float h = fmaf(s1, 0x1p-10f, s0);
-        const float z = __fsub_rn(h, s0);
-        gh[c] = __float_as_uint(h);
-        gl[c] = __float_as_uint(fmaf(s1, 0x1p-10f, -z));
-      }
-      if (!warp_wait(&lvl[1], par, ta.err)) break;  // levels 2 and 3
-      tc_fence_after();
-#pragma unroll
-      for (int L = 2; L < kLevels; ++L) {
-        tmem_ld32(tcol + (uint32_t)(L * kN), u);
-        tmem_ld_wait();
-        if (L == 3) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&lfree[1]);
-        }
-        const float sc = L == 2 ? 0x1p-20f : 0x1p-30f;
-#pragma unroll
-        for (int c = 0; c < kPartCols; ++c)
-          gl[c] = __float_as_uint(fmaf(__uint_as_float(u[c]), sc, __uint_as_float(gl[c])));
-      }
+      if (lane == 0) mbar_arrive(&lfree[g]);
+    };
+    for (int tt = 0; tt < T; ++tt) {
+      const uint32_t par = (uint32_t)tt & 1u;
       const int rs = tt % kRecSlots;
       if (!warp_wait(&recf[rs], (uint32_t)(tt / kRecSlots) & 1u, ta.err)) break;
       const float* rt = recs + rs * (kRecBytes / 4) + part * kPartCols * RW;
+      float t[kPartCols];
+      uint32_t u0[kPartCols], u1[kPartCols];
+      bool alive = true;
+      for (int pass = 0;; ++pass) {
+        if (!warp_wait(&lvl[0], par, ta.err)) {  // levels 0 and 1
+          alive = false;
+          break;
+        }
+        tc_fence_after();
+        tmem_ld32(tcol, u0);
+        tmem_ld32(tcol + (uint32_t)kN, u1);
+        tmem_ld_wait();
+        if constexpr (!LSE) release(0);
+#pragma unroll
+        for (int c = 0; c < kPartCols; c += 2) {
+          float qa, qb;
+          if constexpr (RW == 2) {
+            const float4 R = *reinterpret_cast<const float4*>(rt + c * 2);
+            qa = R.x;
+            qb = R.z;
+          } else {
+            qa = rt[c * 4];
+            qb = rt[c * 4 + 4];
+          }
+          t[c] = fmaf(__uint_as_float(u1[c]), k1, fmaf(__uint_as_float(u0[c]), k0, __fadd_rn(hm, qa)));
+          t[c + 1] = fmaf(__uint_as_float(u1[c + 1]), k1, fmaf(__uint_as_float(u0[c + 1]), k0, __fadd_rn(hm, qb)));
+        }
+        if (!warp_wait(&lvl[1], par, ta.err)) {  // levels 2 and 3
+          alive = false;
+          break;
+        }
+        tc_fence_after();
+        tmem_ld32(tcol + (uint32_t)(2 * kN), u0);
+        tmem_ld32(tcol + (uint32_t)(3 * kN), u1);
+        tmem_ld_wait();
+        if constexpr (!LSE) release(1);
+#pragma unroll
+        for (int c = 0; c < kPartCols; ++c)
+          t[c] = fmaf(__uint_as_float(u1[c]), k3, fmaf(__uint_as_float(u0[c]), k2, t[c]));
+        if constexpr (!LSE) break;
+        float tmax = -3.0e38f;
+#pragma unroll
+        for (int c = 0; c < kPartCols; ++c) tmax = fmaxf(tmax, t[c]);
+        if (pass == 4 || !__any_sync(0xffffffffu, tmax > kTheta2)) break;
+        if (tmax > kTheta2) {
+          const float dlt = ceil_grid(tmax);
+          mx += dlt;
+          hm = ph - mx;
+          const float f = ex2_approx(-dlt);
+          Sa[0] *= f;
+          Ca[0] *= f;
+        }
+      }
+      if (!alive) break;
+      if constexpr (LSE) {
+        release(0);
+        release(1);
+      }
 #pragma unroll
       for (int c = 0; c < kGroups; ++c) {
         float acc[NA];
 #pragma unroll
         for (int k = 0; k < NA; ++k) acc[k] = 0.f;
-        // the group's records: Qh and the weights of its 8 columns
-        float qh[8], w[NR][8];
+        // the group's weights, 8 columns
+        float w[NA][8];
         if constexpr (RW == 2) {
 #pragma unroll
           for (int jj = 0; jj < 8; jj += 2) {
             const float4 R = *reinterpret_cast<const float4*>(rt + (c * 8 + jj) * 2);
-            qh[jj] = R.x;
             w[0][jj] = R.y;
-            qh[jj + 1] = R.z;
             w[0][jj + 1] = R.w;
           }
         } else {
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj) {
             const float4 R = *reinterpret_cast<const float4*>(rt + (c * 8 + jj) * 4);
-            qh[jj] = R.x;
             const float ws[3] = {R.y, R.z, R.w};
 #pragma unroll
-            for (int k = 0; k < NR; ++k) w[k][jj] = ws[k];
+            for (int k = 0; k < NA; ++k) w[k][jj] = ws[k];
           }
         }
-        if constexpr (!LSE) {
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            const float ex = ex2_approx(entry_t2(__fadd_rn(hm, qh[jj]), __uint_as_float(gh[c * 8 + jj]),
-                                                 __uint_as_float(gl[c * 8 + jj]), kh, kl));
+        for (int jj = 0; jj < 8; ++jj) {
+          const float ex = ex2_approx(t[c * 8 + jj]);
 #pragma unroll
-            for (int k = 0; k < NR; ++k) acc[k] = fmaf(((SQM >> k) & 1) ? ex * ex : ex, w[k][jj], acc[k]);
-          }
-        } else {
-          float t[8];
-          float tmax = -3.0e38f;
-#pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            t[jj] = entry_t2(__fadd_rn(hm, qh[jj]), __uint_as_float(gh[c * 8 + jj]),
-                             __uint_as_float(gl[c * 8 + jj]), kh, kl);
-            tmax = fmaxf(tmax, t[jj]);
-          }
-          for (int k = 0; k < 4 && tmax > kTheta2; ++k) {  // raise the max (rare after the first group)
-            const float dlt = ceil_grid(tmax);
-            mx += dlt;
-            hm = ph - mx;
-            const float f = ex2_approx(-dlt);
-            Sa[0] *= f;
-            Ca[0] *= f;
-            tmax = -3.0e38f;
-#pragma unroll
-            for (int jj = 0; jj < 8; ++jj) {
-              t[jj] = entry_t2(__fadd_rn(hm, qh[jj]), __uint_as_float(gh[c * 8 + jj]),
-                               __uint_as_float(gl[c * 8 + jj]), kh, kl);
-              tmax = fmaxf(tmax, t[jj]);
-            }
-          }
-#pragma unroll
-          for (int jj = 0; jj < 8; ++jj) acc[0] = fmaf(ex2_approx(t[jj]), w[0][jj], acc[0]);
+          for (int k = 0; k < NA; ++k) acc[k] = fmaf(((SQM >> k) & 1) ? ex * ex : ex, w[k][jj], acc[k]);
         }
 #pragma unroll
         for (int k = 0; k < NA; ++k) kadd(Sa[k], Ca[k], acc[k]);
