@@ -51,7 +51,7 @@
 // (By itself that changed nothing while the epilogue was the longer side: a CG sweep of
 // n = m = 16384, d = 64 took 0.301 ms with A in shared memory and 0.299 ms so.)
 //
-// CTA roles (480 threads, one CTA per SM: about 215 KB of shared memory):
+// CTA roles (480 threads, one CTA per SM: about 155 KB of shared memory):
 //   warp 0, lane 0 and warp 14, lane 0: the (up to) 40 MMAs of each tile, twenty
 //     each (levels 0, 3 and levels 1, 2), with a commit per level. A
 //     tcgen05.mma blocks its thread while the tensor unit's short queue is
@@ -481,11 +481,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
     const float ph = so.own[e].ph;  // e < npad: padded rows have records
     const float k0 = ta.kappa[0], k1 = k0 * 0x1p-10f, k2 = k0 * 0x1p-20f, k3 = k0 * 0x1p-30f;
     // LSE: hm = ph - mx. The max starts at -2^23, far below every entry, so the
-    // first tile raises it to its own maximum (the one inexact step, it only chooses
-    // the shift); from then on ph and mx are on the grid and hm is exact. A tile whose
-    // entries exceed the max by more than the threshold is read from TMEM again with
-    // the raised one (a difference of rounded exponents would not be exact), so the
-    // LSE sweeps hand a tile's levels back only once its max is settled.
+    // first group of columns raises it to its own maximum (the one inexact step, it
+    // only chooses the shift); from then on ph and mx are on the grid and hm is exact.
+    // A raise forms the group's exponents again (a difference of rounded exponents
+    // would not be exact), for which the LSE sweeps keep G as an FP32 pair instead of
+    // adding the levels to the exponent as they come (three instructions more per
+    // entry; holding the tile's levels in TMEM until its max is settled keeps the next
+    // tile's MMAs waiting: 0.434 ms per LSE sweep at n = m = 16384, d = 64, this way
+    // 0.317).
     float hm = LSE ? ph - mx : ph;
     const uint32_t tcol = tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(part * kPartCols);
     const float* recs = (const float*)(sm + kOffRec);
@@ -499,19 +502,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
       const int rs = tt % kRecSlots;
       if (!warp_wait(&recf[rs], (uint32_t)(tt / kRecSlots) & 1u, ta.err)) break;
       const float* rt = recs + rs * (kRecBytes / 4) + part * kPartCols * RW;
-      float t[kPartCols];
+      if (!warp_wait(&lvl[0], par, ta.err)) break;  // levels 0 and 1
+      tc_fence_after();
       uint32_t u0[kPartCols], u1[kPartCols];
-      bool alive = true;
-      for (int pass = 0;; ++pass) {
-        if (!warp_wait(&lvl[0], par, ta.err)) {  // levels 0 and 1
-          alive = false;
-          break;
-        }
-        tc_fence_after();
-        tmem_ld32(tcol, u0);
-        tmem_ld32(tcol + (uint32_t)kN, u1);
-        tmem_ld_wait();
-        if constexpr (!LSE) release(0);
+      tmem_ld32(tcol, u0);
+      tmem_ld32(tcol + (uint32_t)kN, u1);
+      tmem_ld_wait();
+      release(0);
+      if constexpr (!LSE) {
+        float t[kPartCols];
 #pragma unroll
         for (int c = 0; c < kPartCols; c += 2) {
           float qa, qb;
@@ -526,68 +525,108 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
           t[c] = fmaf(__uint_as_float(u1[c]), k1, fmaf(__uint_as_float(u0[c]), k0, __fadd_rn(hm, qa)));
           t[c + 1] = fmaf(__uint_as_float(u1[c + 1]), k1, fmaf(__uint_as_float(u0[c + 1]), k0, __fadd_rn(hm, qb)));
         }
-        if (!warp_wait(&lvl[1], par, ta.err)) {  // levels 2 and 3
-          alive = false;
-          break;
-        }
+        if (!warp_wait(&lvl[1], par, ta.err)) break;  // levels 2 and 3
         tc_fence_after();
         tmem_ld32(tcol + (uint32_t)(2 * kN), u0);
         tmem_ld32(tcol + (uint32_t)(3 * kN), u1);
         tmem_ld_wait();
-        if constexpr (!LSE) release(1);
+        release(1);
 #pragma unroll
         for (int c = 0; c < kPartCols; ++c)
           t[c] = fmaf(__uint_as_float(u1[c]), k3, fmaf(__uint_as_float(u0[c]), k2, t[c]));
-        if constexpr (!LSE) break;
-        float tmax = -3.0e38f;
 #pragma unroll
-        for (int c = 0; c < kPartCols; ++c) tmax = fmaxf(tmax, t[c]);
-        if (pass == 4 || !__any_sync(0xffffffffu, tmax > kTheta2)) break;
-        if (tmax > kTheta2) {
-          const float dlt = ceil_grid(tmax);
-          mx += dlt;
-          hm = ph - mx;
-          const float f = ex2_approx(-dlt);
-          Sa[0] *= f;
-          Ca[0] *= f;
+        for (int c = 0; c < kGroups; ++c) {
+          float acc[NA];
+#pragma unroll
+          for (int k = 0; k < NA; ++k) acc[k] = 0.f;
+          // the group's weights, 8 columns
+          float w[NA][8];
+          if constexpr (RW == 2) {
+#pragma unroll
+            for (int jj = 0; jj < 8; jj += 2) {
+              const float4 R = *reinterpret_cast<const float4*>(rt + (c * 8 + jj) * 2);
+              w[0][jj] = R.y;
+              w[0][jj + 1] = R.w;
+            }
+          } else {
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+              const float4 R = *reinterpret_cast<const float4*>(rt + (c * 8 + jj) * 4);
+              const float ws[3] = {R.y, R.z, R.w};
+#pragma unroll
+              for (int k = 0; k < NA; ++k) w[k][jj] = ws[k];
+            }
+          }
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) {
+            const float ex = ex2_approx(t[c * 8 + jj]);
+#pragma unroll
+            for (int k = 0; k < NA; ++k) acc[k] = fmaf(((SQM >> k) & 1) ? ex * ex : ex, w[k][jj], acc[k]);
+          }
+#pragma unroll
+          for (int k = 0; k < NA; ++k) kadd(Sa[k], Ca[k], acc[k]);
         }
-      }
-      if (!alive) break;
-      if constexpr (LSE) {
-        release(0);
-        release(1);
-      }
+      } else {
+        // G = S_0 + 2^-10 S_1 + ... as an FP32 pair (gh, gl) in (u0, u1). S_0 is an
+        // integer up to 2^20 and 2^-10 S_1 a multiple of 2^-10 up to 2^13: where
+        // |S_0| >= |2^-10 S_1| Fast2Sum is exact, and otherwise the sum stays within
+        // 2^14 on the 2^-10 grid and is exact already (z = 2^-10 S_1, error 0).
 #pragma unroll
-      for (int c = 0; c < kGroups; ++c) {
-        float acc[NA];
+        for (int c = 0; c < kPartCols; ++c) {
+          const float s0 = __uint_as_float(u0[c]), s1 = __uint_as_float(u1[c]);
+          const float h = fmaf(s1, 0x1p-10f, s0);
+          const float z = __fsub_rn(h, s0);
+          u0[c] = __float_as_uint(h);
+          u1[c] = __float_as_uint(fmaf(s1, 0x1p-10f, -z));
+        }
+        if (!warp_wait(&lvl[1], par, ta.err)) break;  // levels 2 and 3
+        tc_fence_after();
 #pragma unroll
-        for (int k = 0; k < NA; ++k) acc[k] = 0.f;
-        // the group's weights, 8 columns
-        float w[NA][8];
-        if constexpr (RW == 2) {
+        for (int L = 2; L < kLevels; ++L) {
+          uint32_t u[kPartCols];
+          tmem_ld32(tcol + (uint32_t)(L * kN), u);
+          tmem_ld_wait();
+          if (L == 3) release(1);
+          const float sc = L == 2 ? 0x1p-20f : 0x1p-30f;
+#pragma unroll
+          for (int c = 0; c < kPartCols; ++c)
+            u1[c] = __float_as_uint(fmaf(__uint_as_float(u[c]), sc, __uint_as_float(u1[c])));
+        }
+#pragma unroll
+        for (int c = 0; c < kGroups; ++c) {
+          float qh[8], w[8], t[8], tmax;
 #pragma unroll
           for (int jj = 0; jj < 8; jj += 2) {
             const float4 R = *reinterpret_cast<const float4*>(rt + (c * 8 + jj) * 2);
-            w[0][jj] = R.y;
-            w[0][jj + 1] = R.w;
+            qh[jj] = R.x;
+            w[jj] = R.y;
+            qh[jj + 1] = R.z;
+            w[jj + 1] = R.w;
           }
-        } else {
+          auto form = [&] {
+            tmax = -3.0e38f;
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            const float4 R = *reinterpret_cast<const float4*>(rt + (c * 8 + jj) * 4);
-            const float ws[3] = {R.y, R.z, R.w};
-#pragma unroll
-            for (int k = 0; k < NA; ++k) w[k][jj] = ws[k];
+            for (int jj = 0; jj < 8; ++jj) {
+              t[jj] = fmaf(__uint_as_float(u1[c * 8 + jj]), k0,
+                           fmaf(__uint_as_float(u0[c * 8 + jj]), k0, __fadd_rn(hm, qh[jj])));
+              tmax = fmaxf(tmax, t[jj]);
+            }
+          };
+          form();
+          for (int k = 0; k < 4 && tmax > kTheta2; ++k) {  // raise the max (rare after the first group)
+            const float dlt = ceil_grid(tmax);
+            mx += dlt;
+            hm = ph - mx;
+            const float f = ex2_approx(-dlt);
+            Sa[0] *= f;
+            Ca[0] *= f;
+            form();
           }
+          float acc = 0.f;
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) acc = fmaf(ex2_approx(t[jj]), w[jj], acc);
+          kadd(Sa[0], Ca[0], acc);
         }
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          const float ex = ex2_approx(t[c * 8 + jj]);
-#pragma unroll
-          for (int k = 0; k < NA; ++k) acc[k] = fmaf(((SQM >> k) & 1) ? ex * ex : ex, w[k][jj], acc[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < NA; ++k) kadd(Sa[k], Ca[k], acc[k]);
       }
     }
     if (part > 0) {  // parts 1 and 2 hand their sums to part 0
