@@ -46,7 +46,7 @@ void ensure_capacity(eot_handle h, int64_t n, int64_t m) {
   h->cnt_strip = (int*)dev_alloc(h, h->max_strips * sizeof(int));
   h->rowblk_slots = std::max<int64_t>(h->max_rowblk, L / 128 + 2);  // 128-point blocks of the tensor-core sweeps
   h->cnt_rowblk = (int*)dev_alloc(h, h->rowblk_slots * sizeof(int));
-  h->maxbuf_len = L / 256 + 8 * (int64_t)h->sms + 64;
+  h->maxbuf_len = L / 64 + 8 * (int64_t)h->sms + 64;
   h->maxbuf = (double*)dev_alloc(h, h->maxbuf_len * sizeof(double));
   h->cnt_dot = (int*)dev_alloc(h, sizeof(int));
   EOT_CUDA(cudaMemset(h->sc, 0, SC_TOTAL * sizeof(double)));

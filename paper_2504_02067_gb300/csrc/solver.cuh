@@ -363,16 +363,17 @@ struct Solver {
   // s_C = 1 / max_ij |x_i - y_j|^2 (cost normalised to max 1, Sec. 4.1): FP32 scan,
   // FP64 re-evaluation of each thread's arg-max pair, maximum on the host.
   double max_cost_scale() {
-    const int64_t B = (n + kThreads - 1) / kThreads;
-    int64_t S = std::max<int64_t>(1, (2 * (int64_t)h->sms + B - 1) / B);
+    const int64_t B = (n + kMaxRows - 1) / kMaxRows, B2 = (n + 2 * kMaxRows - 1) / (2 * kMaxRows);
+    // chunks of the other side: which pairs are re-evaluated depends on these only
+    int64_t S = std::max<int64_t>(1, (2 * (int64_t)h->sms + B2 - 1) / B2);
     S = std::min<int64_t>(S, (m + 255) / 256);
     const int64_t chunk = (m + S - 1) / S;
     S = (m + chunk - 1) / chunk;
     if (B * S > h->maxbuf_len) throw EotError{EOT_ERR_INVALID_ARG, "cost-max buffer too small"};
     const dim3 grid((unsigned)B, (unsigned)S);
-    if (d <= 4) launch_k(pts_maxdist_kernel<4>, grid, dim3(kThreads), st, X, Y, n, m, d, chunk, h->maxbuf);
-    else if (d <= 16) launch_k(pts_maxdist_kernel<16>, grid, dim3(kThreads), st, X, Y, n, m, d, chunk, h->maxbuf);
-    else launch_k(pts_maxdist_kernel<64>, grid, dim3(kThreads), st, X, Y, n, m, d, chunk, h->maxbuf);
+    if (d <= 4) launch_k(pts_maxdist_kernel<4>, grid, dim3(kMaxRows), st, X, Y, n, m, d, chunk, h->maxbuf);
+    else if (d <= 16) launch_k(pts_maxdist_kernel<16>, grid, dim3(kMaxRows), st, X, Y, n, m, d, chunk, h->maxbuf);
+    else launch_k(pts_maxdist_kernel<64>, grid, dim3(kMaxRows), st, X, Y, n, m, d, chunk, h->maxbuf);
     h->launches++;
     std::vector<double> v((size_t)(B * S));
     EOT_CUDA(cudaMemcpyAsync(v.data(), h->maxbuf, v.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
