@@ -266,7 +266,7 @@ def roofline_at_scale(h, E, dev, flush, peak, side=128):
 # run's JSON line; each takes seconds)
 # ---------------------------------------------------------------------------
 
-MUFU_PER_CLK_SM = 16     # ex2 results per clock per SM (4 per SM sub-partition)
+MUFU_PER_CLK_SM = 32     # ex2 results per clock per SM (31.8 measured)
 FP32_LANES_SM = 128      # FP32 lanes per SM
 SM_MAX_GHZ = 2.07
 
@@ -388,7 +388,7 @@ def record_d64(E, dev, peaks):
             rates[name] = {"ms": round(ms, 4), "p_entries_per_s": round(n * n / (ms * 1e-3), 1)}
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         bf16 = (peaks or {}).get("bf16_tflops", 1900.0) * 1e12
-        flop_per_entry = 15 * 2 * 64           # 15 digit-slice BF16 MMAs of K = 64 per entry
+        flop_per_entry = 10 * 2 * 64           # 10 digit-slice FP16 MMAs (the BF16 rate) of K = 64 per entry
         fp32_issue = sms * FP32_LANES_SM * SM_MAX_GHZ * 1e9
         ex2 = sms * MUFU_PER_CLK_SM * SM_MAX_GHZ * 1e9
         best = max(rates["cg_col_sweep"]["p_entries_per_s"], rates["cg_row_sweep"]["p_entries_per_s"])
