@@ -158,7 +158,9 @@ __global__ void __launch_bounds__(kThreads) plan_int_points_kernel(int64_t n, in
 // `slack` covers FP32 underflow. The bound holds for 1e-30 <= gamma (s_C) <= 1e30
 // or 0 and for |V|, |M| and thresholds up to 1e8 (an exponent that overflows FP32
 // is then below every one that matters); rows outside, or with a NaN or +inf, are
-// decided by the all-FP64 scan of the row.
+// decided by the all-FP64 scan of the row. So is a row whose maximum only came within
+// 1e8 after entries were passed over that the margin at the final maximum does not
+// rule out.
 
 constexpr float kScreenMax = 1.0e8f;
 
@@ -211,8 +213,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) pla
   constexpr int U = 16 / V;
   __shared__ __align__(16) float vt[kScreenTile];
   __shared__ float vmax[kWarps];
+  __shared__ float skipped[kWarps];  // argmax: the row's largest entry passed over because the maximum was out of reach
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) skipped[warp] = -INFINITY;
   const int64_t i = (int64_t)blockIdx.x * kWarps + warp;
   const bool rv = i < n;
   const T* crow = C + (rv ? i : 0) * ldc;
@@ -283,7 +287,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) pla
         for (int o = 16; o > 0; o >>= 1) mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         M = max_nan(M, mx);
         const float thr = M - screen_margin(sc, Vb, M);
-        if (mx >= thr && fabsf(M) <= kScreenMax) {  // (uniform) the batch holds a contender
+        if (!(fabsf(M) <= kScreenMax)) {
+          if (lane == 0) skipped[warp] = M;
+        } else if (mx >= thr) {  // (uniform) the batch holds a contender
 #pragma unroll
           for (int q = 0; q < U; ++q)
 #pragma unroll
@@ -313,7 +319,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) pla
     }
   }
   if (!rv) return;
-  if constexpr (MODE == 0) ok = ok && fabsf(M) <= kScreenMax;
+  // (a maximum that came into reach late: what was skipped before must lie below it for sure)
+  if constexpr (MODE == 0) {
+    __syncwarp();
+    ok = ok && fabsf(M) <= kScreenMax && skipped[warp] < M - screen_margin(sc, Vb, M);
+  }
   if (!ok) {  // outside the bound's reach: every entry in FP64
     acc = Acc<MODE>();
     for (int64_t j = lane; j < m; j += 32) {
@@ -357,6 +367,7 @@ struct ScreenSmem {
     int32_t open[kOpen][2];                 // (row of the CTA, column)
   };
   int ncand[kSR];
+  float skipped[kSR];                       // argmax: the largest entry passed over, see the dense kernel
   int nopen;
   double best[kSR];                         // results of this CTA's chunk, read by rank 0
   long long idx[kSR];
@@ -417,6 +428,7 @@ __global__ void __launch_bounds__(kThreads, 2) plan_screen_points_kernel(int64_t
   if (lane == 0) s.red[warp] = Vb;
   if (tid < kSR) {
     s.ncand[tid] = 0;
+    s.skipped[tid] = -INFINITY;
     s.best[tid] = 0.0;
     s.idx[tid] = -1;
     s.cnt[tid] = 0;
@@ -543,7 +555,8 @@ __global__ void __launch_bounds__(kThreads, 2) plan_screen_points_kernel(int64_t
         for (int o = 8; o > 0; o >>= 1) mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         M[r] = max_nan(M[r], mx);
         const float thr = M[r] - screen_margin(sc, Vb, M[r]);
-        const bool hit = rok[r] && mx >= thr && fabsf(M[r]) <= kScreenMax;  // (the same in the row's 16 threads)
+        const bool in = fabsf(M[r]) <= kScreenMax, hit = rok[r] && mx >= thr && in;  // (the same in the row's 16 threads)
+        if (!in && cg == 0) s.skipped[row] = M[r];
         if (__any_sync(0xffffffffu, hit)) {
           if (hit) {
 #pragma unroll
@@ -604,11 +617,15 @@ __global__ void __launch_bounds__(kThreads, 2) plan_screen_points_kernel(int64_t
   }
   __syncthreads();
   if constexpr (MODE == 0) {
-    // (a chunk whose exponents are all -inf has nothing to offer)
+    // (a chunk whose exponents are all -inf has nothing to offer; a maximum that came
+    // into reach late: what was skipped before must lie below it for sure)
     if (cg == 0) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-        if (rok[r] && !(fabsf(M[r]) <= kScreenMax) && M[r] != -INFINITY) s.scan[4 * rg + r] = 1;
+      for (int r = 0; r < 4; ++r) {
+        const bool done = fabsf(M[r]) <= kScreenMax ? s.skipped[4 * rg + r] < M[r] - screen_margin(sc, Vb, M[r])
+                                                    : M[r] == -INFINITY;
+        if (rok[r] && !done) s.scan[4 * rg + r] = 1;
+      }
     }
     // the contenders' exact exponents; every thread takes (row, slot) pairs
     for (int q = tid; q < kSR * kCand; q += kThreads) {

@@ -1,0 +1,65 @@
+"""The screened integer outputs (argmax, support) at the ends of the screening's reach.
+Whole numbers, so every comparison with the oracle is exact."""
+import numpy as np
+import pytest
+
+from oracle import eot_oracle as O
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def H():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2504_02067_gb300 import Handle, build
+    build()
+    h = Handle(0, 64, 64)
+    yield h
+    h.close()
+
+
+def t(x, dtype=torch.float64):
+    return torch.as_tensor(np.ascontiguousarray(x)).to(device=DEV, dtype=dtype)
+
+
+def argmax(H, prob, v, gamma):
+    idx = torch.full((prob.n,), -7, dtype=torch.int64, device=DEV)
+    H.eot_plan_argmax(prob, t(v), gamma, idx)
+    return idx.cpu().numpy()
+
+
+@pytest.mark.parametrize("f64", [False, True])
+def test_dense_maximum_that_comes_into_reach_late(H, f64):
+    """Row maxima around -1e8: the screening passes over entries below it, and a later
+    entry whose FP32 value is just above it must not hide one of them that is larger."""
+    from paper_2504_02067_gb300 import Problem
+    n, m = 64, 4096
+    C = np.full((n, m), 3.0e8)
+    v = np.zeros(m)
+    C[:, 0] = 100000008.0 - 8.0 * (np.arange(n) - n // 2)
+    v[1000] = -67108871.0
+    C[:, 1000] = 32891141.9 - 8.0 * (np.arange(n) - n // 2)
+    C = C if f64 else C.astype(np.float32)
+    prob = Problem(t(C, torch.float64 if f64 else torch.float32), precision="fp64" if f64 else "mixed")
+    assert np.array_equal(argmax(H, prob, v, 1.0), O.plan_row_argmax(v, 1.0, C.astype(np.float64)))
+
+
+def test_point_maximum_that_comes_into_reach_late(H):
+    """The same through the point kernel, the two contenders in different tiles of a
+    cluster's chunks and of one chunk."""
+    from paper_2504_02067_gb300 import Problem
+    X = np.zeros((70, 3), dtype=np.float32)
+    for m in (1500, 200000):
+        Y = np.zeros((m, 3), dtype=np.float32)
+        Y[:, 2] = 20000.0
+        Y[0] = 2.0, 1.0, 10000.0  # exponent -100000005, in FP32 -100000008
+        Y[1000, 2] = 5735.0       # exponent -100000008.9, in FP32 -100000000
+        v = np.full(m, -np.inf)   # (the other columns have no mass)
+        v[0], v[1000] = 0.0, -67109783.9
+        prob = Problem(X=t(X, torch.float32), Y=t(Y, torch.float32), precision="mixed", cost_scale=1.0)
+        C = np.concatenate([O.sqeuclid_ordered(X, Y[k:k + 10000]) for k in range(0, m, 10000)], axis=1)
+        assert np.array_equal(argmax(H, prob, v, 1.0), O.plan_row_argmax(v, 1.0, C)), m
