@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(kThreads) plan_int_points_kernel(int64_t n, in
 // 2^-24 D). x -> x +- c |x| is increasing, so an entry below
 //     M - 3 c (V + |M|) - slack        (M: the largest tf met so far)
 // is below the entry that gave M in FP64 too, and no later entry changes that;
-// likewise tf decides against a threshold outside 3 c (V + |threshold|) + slack.
+// likewise tf decides against a threshold outside 3 c (V + |threshold|) + slack. A NaN
+// (gamma = 0 with a cost beyond FP32's range, whose exponent is v_j) decides nothing.
 // `slack` covers FP32 underflow. The bound holds for 1e-30 <= gamma (s_C) <= 1e30
 // or 0 and for |V|, |M| and thresholds up to 1e8 (an exponent that overflows FP32
 // is then below every one that matters); rows outside, or with a NaN or +inf, are
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) pla
     auto test = [&](int j0, const T (&c)[U][V]) {
       float tf[U][V];
       float mx = -INFINITY;
-      int above = 0, open = 0;
+      int above = 0, not_below = 0;
 #pragma unroll
       for (int q = 0; q < U; ++q) {
         const int j = j0 + q * 32 * V;
@@ -278,7 +279,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) pla
           if constexpr (MODE == 0) mx = max_nan(mx, tf[q][e]);
           else {
             above += tf[q][e] > hi ? 1 : 0;
-            open += tf[q][e] >= lo ? 1 : 0;
+            // (a NaN is open; of an FP32 cost it is a NaN in FP64 too, which counts nowhere)
+            if constexpr (sizeof(T) == 8) not_below += tf[q][e] < lo ? 0 : 1;
+            else not_below += tf[q][e] >= lo ? 1 : 0;
           }
         }
       }
@@ -298,12 +301,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) pla
         }
       } else {
         acc.cnt += above;
-        if (open != above) {
+        if (not_below != above) {
 #pragma unroll
           for (int q = 0; q < U; ++q)
 #pragma unroll
             for (int e = 0; e < V; ++e)
-              if (tf[q][e] >= lo && tf[q][e] <= hi) exact(c[q][e], t0 + j0 + q * 32 * V + e);
+              if (!(tf[q][e] < lo) && !(tf[q][e] > hi)) exact(c[q][e], t0 + j0 + q * 32 * V + e);
         }
       }
     };
@@ -591,18 +594,18 @@ __global__ void __launch_bounds__(kThreads, 2) plan_screen_points_kernel(int64_t
           __syncwarp();
         }
       } else {
-        int above = 0, open = 0;
+        int above = 0, below = 0;  // the rest, NaNs among it, is open
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           acc[r][e] = fmaf(-sc.g, acc[r][e], h[e]);
           above += acc[r][e] > hi[r] ? 1 : 0;
-          open += acc[r][e] >= lo[r] ? 1 : 0;
+          below += acc[r][e] < lo[r] ? 1 : 0;
         }
         above_r[r] += above;
-        if (open != above && rok[r]) {
+        if (above + below != 8 && rok[r]) {
 #pragma unroll
           for (int e = 0; e < 8; ++e)
-            if (acc[r][e] >= lo[r] && acc[r][e] <= hi[r]) {
+            if (!(acc[r][e] < lo[r]) && !(acc[r][e] > hi[r])) {
               const int at = atomicAdd(&s.nopen, 1);
               if (at < kOpen) {
                 s.open[at][0] = row;

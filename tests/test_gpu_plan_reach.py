@@ -63,3 +63,33 @@ def test_point_maximum_that_comes_into_reach_late(H):
         prob = Problem(X=t(X, torch.float32), Y=t(Y, torch.float32), precision="mixed", cost_scale=1.0)
         C = np.concatenate([O.sqeuclid_ordered(X, Y[k:k + 10000]) for k in range(0, m, 10000)], axis=1)
         assert np.array_equal(argmax(H, prob, v, 1.0), O.plan_row_argmax(v, 1.0, C)), m
+
+
+def support(H, prob, u, v, gamma, log_tau):
+    cnt = torch.full((prob.n,), -7, dtype=torch.int64, device=DEV)
+    tot = torch.full((1,), -7, dtype=torch.int64, device=DEV)
+    H.eot_plan_support(prob, t(u), t(v), gamma, log_tau, cnt, tot)
+    cnt = cnt.cpu().numpy()
+    assert int(tot.item()) == int(cnt.sum())
+    return cnt
+
+
+@pytest.mark.parametrize("m", [130, 4096, 4099])
+def test_gamma_zero_with_costs_beyond_fp32(H, m):
+    """gamma = 0: every exponent is v_j (argmax) or u_i + v_j (support), also where the
+    cost overflows FP32 (a dense FP64 cost of 1e39, coordinates 1e20 apart)."""
+    from paper_2504_02067_gb300 import Problem
+    rng = np.random.default_rng(m)
+    n = 70
+    u, v = rng.normal(size=n), rng.normal(size=m)
+    C = rng.uniform(0, 1, size=(n, m))
+    C[:, ::3] = 1.0e39
+    X, Y = rng.normal(size=(n, 2)).astype(np.float32), rng.normal(size=(m, 2)).astype(np.float32)
+    Y[::3, 1] = 1.0e20
+    for prob, cost in ((Problem(t(C), precision="fp64"), C),
+                       (Problem(X=t(X, torch.float32), Y=t(Y, torch.float32), precision="mixed", cost_scale=1.0),
+                        O.sqeuclid_ordered(X, Y))):
+        assert np.array_equal(argmax(H, prob, v, 0.0), O.plan_row_argmax(v, 0.0, cost))
+        for log_tau in (-0.5, 0.0, 1.0):
+            assert np.array_equal(support(H, prob, u, v, 0.0, log_tau), O.plan_support_counts(u, v, 0.0, cost, log_tau))
+
