@@ -170,11 +170,12 @@ __device__ __forceinline__ float max_nan(float a, float b) {
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
-// |v_j| as it enters V: -inf (a column without mass, or below FP32's range: never
-// the answer) counts 0; NaN, +inf and what is above FP32's range make V infinite
-__device__ __forceinline__ float bound_of(float vf) {
-  if (vf == -INFINITY) return 0.f;
-  return vf == vf ? fabsf(vf) : INFINITY;
+// |v_j| as it enters V: -inf (a column without mass: never the answer) counts 0; NaN,
+// +inf and what lies beyond FP32's range make V infinite
+__device__ __forceinline__ float bound_of(float vf, double v) {
+  const float a = fabsf(vf);
+  if (a <= 3.4e38f) return a;
+  return __double2hiint(v) == (int)0xfff00000 && __double2loint(v) == 0 ? 0.f : INFINITY;
 }
 struct Screen {
   float g;      // gamma (dense) or gamma s_C (points), rounded to FP32
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) pla
     for (int q = threadIdx.x; q < tw; q += kThreads) {
       const float vf = cut_f32(__ldg(v + t0 + q));
       vt[q] = vf;
-      vb = fmaxf(vb, bound_of(vf));
+      vb = fmaxf(vb, bound_of(vf, __ldg(v + t0 + q)));
     }
     vb = warp_max_f(vb);
     if (lane == 0) vmax[warp] = vb;
@@ -425,7 +426,8 @@ __global__ void __launch_bounds__(kThreads, 2) plan_screen_points_kernel(int64_t
   // V of the chunk
   float Vb = 0.f;
   for (int64_t j = c0 + tid; j < c1; j += kThreads) {
-    Vb = fmaxf(Vb, bound_of(cut_f32(__ldg(v + j))));
+    const double vj = __ldg(v + j);
+    Vb = fmaxf(Vb, bound_of(cut_f32(vj), vj));
   }
   Vb = warp_max_f(Vb);
   if (lane == 0) s.red[warp] = Vb;

@@ -93,3 +93,16 @@ def test_gamma_zero_with_costs_beyond_fp32(H, m):
         for log_tau in (-0.5, 0.0, 1.0):
             assert np.array_equal(support(H, prob, u, v, 0.0, log_tau), O.plan_support_counts(u, v, 0.0, cost, log_tau))
 
+
+def test_potentials_beyond_fp32(H):
+    """Finite potentials below FP32's range beside costs as large and negative."""
+    from paper_2504_02067_gb300 import Problem
+    rng = np.random.default_rng(4)
+    n, m = 9, 700
+    u, v, C = rng.normal(size=n), rng.normal(size=m), rng.uniform(0, 1, size=(n, m))
+    v[5] = -1.0e39
+    C[:, 5] = -1.0e38
+    C[::2, 5] = -2.0e37
+    prob = Problem(t(C), precision="fp64")
+    assert np.array_equal(argmax(H, prob, v, 20.0), O.plan_row_argmax(v, 20.0, C))
+    assert np.array_equal(support(H, prob, u, v, 20.0, -1.0), O.plan_support_counts(u, v, 20.0, C, -1.0))
