@@ -178,8 +178,10 @@ void run_plan_int(eot_handle h, const eot_problem* P, const double* u, const dou
   // the FP32 screening kernels, unless the temperature leaves their bound's reach
   const dim3 grid((unsigned)((P->n + pint::kWarps - 1) / pint::kWarps));
   auto in_reach = [](double g) { return g == 0.0 || (g >= 1e-30 && g <= 1e30); };
-  auto screen = [](double g, float c, int terms) {
-    return pint::Screen{(float)g, 3.0f * c, 1e-30f + (float)(g * terms * 1e-44)};
+  // under: what underflow may take from a cost (points: from a squared distance, and from
+  // its FP64 product with a tiny s_C)
+  auto screen = [](double g, float c, double under) {
+    return pint::Screen{(float)g, 3.0f * c, 1e-30f + (float)(g * under)};
   };
   if (P->kind == EOT_COST_SQEUCLID_POINTS) {
     double sC = P->cost_scale;
@@ -205,13 +207,13 @@ void run_plan_int(eot_handle h, const eot_problem* P, const double* u, const dou
       }
       launch_kc(pint::plan_screen_points_kernel<MODE>, dim3((unsigned)B, (unsigned)S), dim3(pint::kThreads),
                 (unsigned)S, 0, st, P->n, P->m, (int)P->d, P->X, P->Y, sC, u, v, gamma, log_tau,
-                screen(K, (float)(P->d + 12) * 5.9604645e-8f, (int)P->d), chunk, idx_out, counts, tot);
+                screen(K, (float)(P->d + 12) * 5.9604645e-8f, P->d * 1e-44 + 5e-324 / sC), chunk, idx_out, counts, tot);
     } else {
       launch_k(pint::plan_int_points_kernel<MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (int)P->d, P->X, P->Y,
                sC, u, v, gamma, log_tau, idx_out, counts, tot);
     }
   } else {
-    auto dense = [&](auto* C, float c) {
+    auto dense = [&](auto* C, float c, double under) {
       using T = std::remove_cv_t<std::remove_pointer_t<decltype(C)>>;
       constexpr int VEC = 16 / (int)sizeof(T);
       const bool vec = ((uintptr_t)C % 16) == 0 && P->m % VEC == 0 && P->ldc % VEC == 0;
@@ -220,13 +222,13 @@ void run_plan_int(eot_handle h, const eot_problem* P, const double* u, const dou
                  u, v, gamma, log_tau, idx_out, counts, tot);
       else if (vec)
         launch_k(pint::plan_screen_dense_kernel<T, VEC, MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (const T*)C,
-                 P->ldc, u, v, gamma, log_tau, screen(gamma, c, 1), idx_out, counts, tot);
+                 P->ldc, u, v, gamma, log_tau, screen(gamma, c, under), idx_out, counts, tot);
       else
         launch_k(pint::plan_screen_dense_kernel<T, 1, MODE>, grid, dim3(pint::kThreads), st, P->n, P->m, (const T*)C,
-                 P->ldc, u, v, gamma, log_tau, screen(gamma, c, 1), idx_out, counts, tot);
+                 P->ldc, u, v, gamma, log_tau, screen(gamma, c, under), idx_out, counts, tot);
     };
-    if (P->kind == EOT_COST_DENSE_F64) dense((const double*)P->C, 4.7683716e-7f);
-    else dense((const float*)P->C, 2.3841858e-7f);
+    if (P->kind == EOT_COST_DENSE_F64) dense((const double*)P->C, 4.7683716e-7f, 1.2e-38);  // (below 2^-126 cut to 0)
+    else dense((const float*)P->C, 2.3841858e-7f, 1e-44);
   }
   EOT_LAUNCH_CHECK();
   h->launches++;

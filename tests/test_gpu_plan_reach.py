@@ -106,3 +106,16 @@ def test_potentials_beyond_fp32(H):
     prob = Problem(t(C), precision="fp64")
     assert np.array_equal(argmax(H, prob, v, 20.0), O.plan_row_argmax(v, 20.0, C))
     assert np.array_equal(support(H, prob, u, v, 20.0, -1.0), O.plan_support_counts(u, v, 20.0, C, -1.0))
+
+
+def test_costs_below_fp32_at_a_large_gamma(H):
+    """FP64 costs below 2^-126 whose product with gamma decides."""
+    from paper_2504_02067_gb300 import Problem
+    rng = np.random.default_rng(5)
+    n, m, gamma = 33, 1001, 1.0e30
+    C = rng.uniform(0, 1, size=(n, m)) * 2.0 ** -127
+    u, v = np.zeros(n), rng.uniform(0, 1e-9, size=m)
+    prob = Problem(t(C), precision="fp64")
+    assert np.array_equal(argmax(H, prob, v, gamma), O.plan_row_argmax(v, gamma, C))
+    for log_tau in (-5e-9, -2e-9, 0.0):
+        assert np.array_equal(support(H, prob, u, v, gamma, log_tau), O.plan_support_counts(u, v, gamma, C, log_tau))
