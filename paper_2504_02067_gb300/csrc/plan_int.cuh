@@ -52,24 +52,29 @@ struct Acc {
       cnt += (t > log_tau) ? 1 : 0;
     }
   }
-  // warp-wide combine; lane 0 writes row i's result
-  __device__ __forceinline__ void finish(int64_t i, int lane, int64_t* idx_out, int64_t* counts,
-                                         unsigned long long* total) {
-    if constexpr (MODE == 0) {
+  // warp-wide combine
+  __device__ __forceinline__ void reduce() {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
+    for (int o = 16; o > 0; o >>= 1) {
+      if constexpr (MODE == 0) {
         const double bv = __shfl_xor_sync(0xffffffffu, best, o);
         const long long bi = __shfl_xor_sync(0xffffffffu, (long long)idx, o);
         argmax_merge(best, idx, bv, (int64_t)bi);
+      } else {
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
       }
-      if (lane == 0) idx_out[i] = idx < 0 ? 0 : idx;
+    }
+  }
+  // the same; lane 0 writes row i's result
+  __device__ __forceinline__ void finish(int64_t i, int lane, int64_t* idx_out, int64_t* counts,
+                                         unsigned long long* total) {
+    reduce();
+    if (lane != 0) return;
+    if constexpr (MODE == 0) {
+      idx_out[i] = idx < 0 ? 0 : idx;
     } else {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-      if (lane == 0) {
-        if (counts) counts[i] = (int64_t)cnt;
-        if (total) atomicAdd(total, (unsigned long long)cnt);
-      }
+      if (counts) counts[i] = (int64_t)cnt;
+      if (total) atomicAdd(total, (unsigned long long)cnt);
     }
   }
 };
@@ -189,6 +194,10 @@ __device__ __forceinline__ float screen_margin(const Screen& sc, float V, float 
 // Returns false when the row needs the all-FP64 scan.
 __device__ __forceinline__ bool support_bounds(const Screen& sc, float V, double ui, double log_tau, float& lo,
                                                float& hi) {
+  if (ui == -INFINITY) {  // a row without mass counts nothing
+    lo = hi = INFINITY;
+    return true;
+  }
   const double thr = log_tau - ui;
   if (!(V <= kScreenMax) || !(fabs(thr) <= (double)kScreenMax)) return false;
   const float tf = (float)thr;
@@ -360,6 +369,11 @@ struct ScreenSmem {
   union {
     float ys[kSK][kSPad];                   // a chunk of the tile's coordinates
     double cand_t[kSR][kCand];              // (after the sweep) FP64 exponents of the contenders
+    struct {                                // (at the end) this CTA's part of the all-FP64 scans
+      double best[kSR];
+      long long idx[kSR];
+      long long cnt[kSR];
+    } part;
   };
   float vt[kSC];
   float red[kWarps];
@@ -376,7 +390,8 @@ struct ScreenSmem {
   double best[kSR];                         // results of this CTA's chunk, read by rank 0
   long long idx[kSR];
   long long cnt[kSR];
-  int scan[kSR];                            // the row needs the all-FP64 scan
+  int scan[kSR];                            // the row needs the all-FP64 scan, says this CTA's chunk
+  int any[kSR];                             // ... says any chunk
 };
 
 // The exact exponent pieces of one entry, as plan_int_points_kernel forms them.
@@ -666,46 +681,62 @@ __global__ void __launch_bounds__(kThreads, 2) plan_screen_points_kernel(int64_t
       if (cg == 0 && rok[r]) atomicAdd((unsigned long long*)&s.cnt[4 * rg + r], (unsigned long long)c);
     }
   }
-  cluster_sync();  // every chunk's results are visible to rank 0
-  if (cluster_rank() == 0) {
-    const uint32_t ranks = gridDim.y;
-    if (tid < kSR) {
-      double bv = s.best[tid];
-      int64_t bi = s.idx[tid];
-      long long c = s.cnt[tid];
-      int scan = s.scan[tid];
-      for (uint32_t q = 1; q < ranks; ++q) {
-        scan |= ld_cluster(&s.scan[tid], q);
-        if constexpr (MODE == 0) argmax_merge(bv, bi, ld_cluster(&s.best[tid], q), (int64_t)ld_cluster(&s.idx[tid], q));
-        else c += ld_cluster(&s.cnt[tid], q);
-      }
-      s.best[tid] = bv;
-      s.idx[tid] = bi;
-      s.cnt[tid] = c;
-      s.scan[tid] = scan | (MODE == 0 && bi < 0 ? 1 : 0);
+  cluster_sync();  // every chunk's results are visible to the cluster
+  const uint32_t ranks = gridDim.y;
+  // Rows that need the all-FP64 scan: every CTA scans its own chunk of them, one warp per
+  // row (a cloud with repeated points, say 8-bit colours, has most of its rows here).
+  int need = 0;
+  if (tid < kSR) {
+    bool none = MODE == 0;
+    for (uint32_t q = 0; q < ranks; ++q) {
+      need |= ld_cluster(&s.scan[tid], q);
+      if constexpr (MODE == 0) none = none && ld_cluster(&s.idx[tid], q) < 0;
     }
-    __syncthreads();
-    // one warp per row: rows with an all-FP64 scan, then the outputs
-    long long sum = 0;
+    need = i0 + tid < n && (need || none) ? 1 : 0;
+    s.any[tid] = need;
+  }
+  if (__syncthreads_or(need)) {  // (the same in every CTA of the cluster)
     for (int r = warp; r < kSR; r += kWarps) {
-      const int64_t i = i0 + r;
-      if (i >= n) break;
-      if (s.scan[r]) {
-        Acc<MODE> acc;
-        const double ui = MODE == 1 ? u[i] : 0.0;
-        for (int64_t j = lane; j < m; j += 32)
-          acc.add(ui, __ldg(v + j), exact_gC(&s.xs[0][r], kSR, Y + j * d, d, sC, gamma), j, log_tau);
-        acc.finish(i, lane, idx_out, counts, total);
-      } else if (lane == 0) {
-        if constexpr (MODE == 0) idx_out[i] = s.idx[r];
-        else {
-          if (counts) counts[i] = s.cnt[r];
-          sum += s.cnt[r];
+      if (!s.any[r]) continue;
+      Acc<MODE> acc;
+      const double ui = MODE == 1 ? u[i0 + r] : 0.0;
+      for (int64_t j = c0 + lane; j < c1; j += 32)
+        acc.add(ui, __ldg(v + j), exact_gC(&s.xs[0][r], kSR, Y + j * d, d, sC, gamma), j, log_tau);
+      acc.reduce();
+      if (lane == 0) {
+        if constexpr (MODE == 0) {
+          s.part.best[r] = acc.best;
+          s.part.idx[r] = acc.idx;
+        } else {
+          s.part.cnt[r] = acc.cnt;
         }
       }
     }
-    if constexpr (MODE == 1)
-      if (lane == 0 && total && sum) atomicAdd(total, (unsigned long long)sum);
+    cluster_sync();  // the parts are visible to rank 0
+  }
+  if (cluster_rank() == 0) {
+    long long c = 0;
+    if (tid < kSR && i0 + tid < n) {
+      const bool f = s.any[tid];
+      if constexpr (MODE == 0) {
+        double bv = 0.0;
+        int64_t bi = -1;
+        for (uint32_t q = 0; q < ranks; ++q)
+          argmax_merge(bv, bi, ld_cluster(f ? &s.part.best[tid] : &s.best[tid], q),
+                       (int64_t)ld_cluster(f ? &s.part.idx[tid] : &s.idx[tid], q));
+        idx_out[i0 + tid] = bi < 0 ? 0 : bi;
+      } else {
+        for (uint32_t q = 0; q < ranks; ++q) c += ld_cluster(f ? &s.part.cnt[tid] : &s.cnt[tid], q);
+        if (counts) counts[i0 + tid] = c;
+      }
+    }
+    if constexpr (MODE == 1) {
+      if (total && warp < kSR / 32) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        if (lane == 0 && c) atomicAdd(total, (unsigned long long)c);
+      }
+    }
   }
   cluster_sync();  // no CTA leaves while rank 0 reads its shared memory
 }

@@ -119,3 +119,26 @@ def test_costs_below_fp32_at_a_large_gamma(H):
     assert np.array_equal(argmax(H, prob, v, gamma), O.plan_row_argmax(v, gamma, C))
     for log_tau in (-5e-9, -2e-9, 0.0):
         assert np.array_equal(support(H, prob, u, v, gamma, log_tau), O.plan_support_counts(u, v, gamma, C, log_tau))
+
+
+@pytest.mark.parametrize("n,m,d", [(1, 20, 2), (70, 129, 3), (130, 1100, 3), (65, 2050, 40)])
+def test_points_with_many_repeats(H, n, m, d):
+    """Clouds of few distinct points: every row has more ties and open entries than the
+    screening keeps, in every chunk of the columns; some rows have no mass."""
+    from paper_2504_02067_gb300 import Problem
+    rng = np.random.default_rng(m + d)
+    base = rng.integers(0, 4, size=(5, d))
+    X, Y = (base[rng.integers(0, 5, size=k)].astype(np.float32) for k in (n, m))
+    u, v = rng.normal(size=n), np.zeros(m)
+    v[rng.choice(m, m // 3, replace=False)] = -np.inf
+    u[rng.choice(n, n // 4, replace=False)] = -np.inf
+    sC = O.sqeuclid_scale(X, Y) if n > 1 else 0.25
+    prob = Problem(X=t(X, torch.float32), Y=t(Y, torch.float32), precision="mixed", cost_scale=sC)
+    C = sC * O.sqeuclid_ordered(X, Y)
+    for gamma in (0.0, 64.0):
+        assert np.array_equal(argmax(H, prob, v, gamma), O.plan_row_argmax(v, gamma, C))
+        on = float(u[np.isfinite(u)][0]) - gamma * float(C.min()) if np.isfinite(u).any() else -1.0
+        for log_tau in (on, -1.0, -np.inf):
+            with np.errstate(invalid="ignore"):
+                want = O.plan_support_counts(u, v, gamma, C, log_tau)
+            assert np.array_equal(support(H, prob, u, v, gamma, log_tau), want)
