@@ -261,7 +261,8 @@ struct Dev {
   const Params& prm;
   int ro;
   double dmax = 0.0;   // >= max |x_i - y_j|^2
-  bool split_on = false;  // this problem's sweeps take split coordinates
+  bool split_ok = false;  // this problem's sweeps may take split coordinates
+  bool split_on = false;  // they do, at the present temperature
   // problem
   int64_t n, m;
   int d;
@@ -616,6 +617,7 @@ struct Dev {
   }
   // the temperature of the sweeps that follow
   __device__ void set_gamma(double gamma) {
+    split_on = split_ok && pg::in_range(gamma * sC * pg::kLog2eD * dmax);
     __syncthreads();
     if (threadIdx.x == 0) {
       s.sc[SC_GAMMA] = gamma;
@@ -1066,7 +1068,11 @@ struct Dev {
     smooth(m, c0, 0.01, ct, logct);
     for (int64_t i = gp.gt; i < n; i += gp.GT) nt0[i] = logrt[i];
     for (int64_t j = gp.gt; j < m; j += gp.GT) mt0[j] = logct[j];
+    // the first temperature, with the sweeps of the last one, where the time goes
+    set_gamma(rg(prm.gamma_f));
+    const bool last = split_on;
     set_gamma(rg(fmin(prm.gamma_i, prm.gamma_f)));
+    if (split_on != last) set_gamma(rg(prm.gamma_f));
     if (!bar()) return false;
     for (int k = 0; k < reps; ++k) {
       if (!col_lse(nt0, nullptr, mt0, nullptr, 0.0, logct, mt0, 1, SC_AUX0, 0.0)) return false;
@@ -1119,7 +1125,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) batch_kernel
     if (P.sC <= 0.0) alive = D.compute_sC();
     if (sizeof(T) == 4 && L.prm.pgrid && alive) {
       alive = D.find_dmax(P.sC > 0.0);
-      D.split_on = alive && (double)(float)L.prm.gamma_f * D.sC * pg::kLog2eD * D.dmax <= pg::kMaxBound;
+      D.split_ok = alive;
     }
     if (alive) alive = L.prm.probe > 0 ? D.probe(L.prm.probe) : D.solve(&gamma, &gl1, &stages, &merr);
     if (s.fail) return;  // a barrier gave up: leave the launch (the host reports it)

@@ -190,32 +190,37 @@ struct Solver {
     const char* e = std::getenv("EOT_PGRID");
     return !(e && e[0] == '0');
   }
-  // Sets gamma for the sweeps of this call (the largest it will use) and decides
-  // whether its point sweeps take split coordinates: their accuracy holds up to
-  // pg::kMaxBound base-2 exponent units, gamma s_C log2(e) max |x - y|^2. A library-
-  // computed s_C gives the maximum itself; for a caller's s_C the clouds' extent
-  // bounds it, which takes a read back (not possible when the call must stay
-  // asynchronous).
+  // Sets gamma for the sweeps of this call and decides whether its point sweeps take
+  // split coordinates: their accuracy holds in pg::in_range of gamma s_C log2(e) max
+  // |x - y|^2. A library-computed s_C gives the maximum itself; for a caller's s_C the
+  // clouds' extent bounds it, which takes a read back (not possible when the call must
+  // stay asynchronous).
   // defer: the next split's launch writes gamma (the caller splits before any sweep).
   bool pending = false;
-  double dmax_host = 0.0;
+  double dmax_host = 0.0;  // 0: no split sweeps
   void begin(double gamma, bool defer, bool may_sync = true, bool gradients = false) {
-    gamma_host = gamma;
-    double dmax = 0.0;
-    pg_on = pg_grad = false;
+    dmax_host = 0.0;
     if (sizeof(T) == 4 && points && !plain && (d <= pg::kMaxD || gradients) && pg_enabled()) {
-      if (!sc_given) dmax = 1.00001 / sC;
-      else if (may_sync) dmax = extent_bound();
-      pg_grad = dmax > 0.0 && gamma * sC * pg::kLog2eD * dmax <= pg::kMaxBound;
-      pg_on = pg_grad && d <= pg::kMaxD;
+      if (!sc_given) dmax_host = 1.00001 / sC;
+      else if (may_sync) dmax_host = extent_bound();
     }
-    dmax_host = dmax;
+    choose(gamma);
     pending = defer;
     tc_digits(false);
     if (defer) return;
-    launch_k(set_scalars_kernel, dim3(1), dim3(1), st, h->sc, (int)SC_GAMMA, gamma, (int)SC_DMAX, dmax);
+    launch_k(set_scalars_kernel, dim3(1), dim3(1), st, h->sc, (int)SC_GAMMA, gamma, (int)SC_DMAX, dmax_host);
     EOT_LAUNCH_CHECK();
     h->launches++;
+  }
+  // The next stage's gamma (a program is kept per choice of the sweeps: run_program's key).
+  void set_gamma(double gamma) {
+    choose(gamma);
+    set_scalar(SC_GAMMA, gamma);
+  }
+  void choose(double gamma) {
+    gamma_host = gamma;
+    pg_grad = pg::in_range(gamma * sC * pg::kLog2eD * dmax_host);
+    pg_on = pg_grad && d <= pg::kMaxD;
   }
   // (max |x - x_0| + max |y - x_0|)^2 >= max |x_i - y_j|^2, from one pass over the points
   double extent_bound() {

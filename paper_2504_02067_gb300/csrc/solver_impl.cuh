@@ -167,7 +167,7 @@ void run_solve(eot_handle h, const eot_problem* P, const eot_params* prm_in, dou
   const int max_cg = prm.max_cg > 0 ? prm.max_cg : (int)std::min<int64_t>(4 * (S.full_system ? n + m : n), 2000);
   EOT_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), st));
   S.init_control(prm.max_newton, prm.max_ls, max_cg);
-  S.begin(round_gamma<T>(prm.gamma_f), false);  // the largest temperature of the call
+  S.begin(round_gamma<T>(prm.gamma_f), false);
   if (capped) {
     launch_k(set_deadline_kernel, dim3(1), dim3(1), st, h->sc, prm.max_seconds);
     EOT_LAUNCH_CHECK();
@@ -266,7 +266,7 @@ void run_solve(eot_handle h, const eot_problem* P, const eot_params* prm_in, dou
         S.copy(h->nt0, h->logrt, n);
         S.copy(h->mt0, h->logct, m);
       }
-      S.set_scalar(SC_GAMMA, gamma);
+      S.set_gamma(gamma);
       double dmin = INFINITY;
       const SolveCounters c0 = S.cnt;
       if (prm.projector == EOT_PROJECT_SINKHORN) {
@@ -324,7 +324,7 @@ void run_solve(eot_handle h, const eot_problem* P, const eot_params* prm_in, dou
 
   // marginal L1 error of the output against the unsmoothed r, c, at gamma_f (set
   // here too: the one-row / one-column closed form runs no stage that sets it)
-  S.set_scalar(SC_GAMMA, gamma);
+  S.set_gamma(gamma);
   S.sweep_bucket = &S.cnt.sweeps_other;
   S.copy(u, U, n);
   S.copy(v, V, m);

@@ -30,7 +30,12 @@ namespace eot {
 namespace pg {
 
 constexpr int kMaxD = 16;
-constexpr double kMaxBound = 32768.0;  // largest gamma s_C log2(e) max |x - y|^2 (base-2 exponent units)
+// The split's range of gamma s_C log2(e) max |x - y|^2 (base-2 exponent units), tested at
+// every temperature; the general sweeps serve the rest (below, the scale of the
+// coordinates runs out of FP32: a gamma that FP32 rounds to 0, coinciding points).
+constexpr double kMinBound = 0x1p-40;
+constexpr double kMaxBound = 32768.0;
+__host__ __device__ inline bool in_range(double bound) { return bound >= kMinBound && bound <= kMaxBound; }
 // The online max of an LSE moves in whole units of the base-2 exponent, so that every
 // rescaling (here and where partial sums meet) is by an exact power of two.
 constexpr float kThetaB2 = 12.0f;      // lazy-rescale threshold
