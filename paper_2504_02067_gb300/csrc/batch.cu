@@ -103,7 +103,7 @@ struct Tile {
   T sy[kDmax][kTO];
 };
 constexpr int kMaxRo = 2;  // own elements per thread of a split sweep
-constexpr int kSplitBytes = 16 * kTO * 4;  // kTO records of up to 16 floats; >= 3 sums per own element
+constexpr int kSplitBytes = 20 * kTO * 4;  // kTO records of up to 20 floats; >= 3 sums per own element
 template <class T>
 struct Smem {
   union {
@@ -262,7 +262,7 @@ struct Dev {
   int ro;
   double dmax = 0.0;   // >= max |x_i - y_j|^2
   bool split_ok = false;  // this problem's sweeps may take split coordinates
-  bool split_on = false;  // they do, at the present temperature
+  int split_parts = 0;    // parts per coordinate at the present temperature, 0: the general sweeps
   // problem
   int64_t n, m;
   int d;
@@ -506,9 +506,9 @@ struct Dev {
   }
 
   // ---- the same sweep from split coordinates (FP32; pg::sweep_kernel's scheme) ----
-  template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, class Epi>
+  template <int D, int RO, int P, int NR, bool LSE, int SQM, bool ROWS, class Epi>
   __device__ __noinline__ bool sweep_split(const T* w0, const T* w1, const T* w2, Epi& epi) {
-    using C = pg::Core<D, RO, NR, LSE, SQM, false>;
+    using C = pg::Core<D, RO, NR, LSE, SQM, false, P>;
     constexpr int NA = C::NA, NW = C::NW, REC = C::REC, ND = Epi::kDot, L = kThreads * RO;
     static_assert(REC * kTO * 4 <= kSplitBytes && NA * L * 8 <= kSplitBytes && RO <= kMaxRo, "split tile too small");
     float(*rec)[REC] = reinterpret_cast<float(*)[REC]>(s.split);
@@ -589,39 +589,36 @@ struct Dev {
     }
   }
 
-  // max |x - x_0| + max |y - x_0| bounds every distance (for a caller's s_C; a computed
-  // s_C gives the largest distance itself)
+  // the squared diagonal of the clouds' common box bounds every squared distance (for a
+  // caller's s_C; a computed s_C gives the largest distance itself)
   __device__ bool find_dmax(bool given) {
     if (!given) {
       dmax = 1.00001 / sC;
       return true;
     }
-    double ext[2];
-    for (int side = 0; side < 2; ++side) {
-      const float* p = side ? Y : X;
-      const int64_t len = side ? m : n;
-      double best = 0.0;
-      for (int64_t i = gp.gt; i < len; i += gp.GT) {
-        float q = 0.f;
-        for (int k = 0; k < d; ++k) {
-          const float df = __ldg(p + i * d + k) - __ldg(X + k);
-          q = fmaf(df, df, q);
+    dmax = 0.0;
+    for (int k = 0; k < d; ++k) {
+      double ext[2];
+      for (int side = 0; side < 2; ++side) {  // the largest and the smallest coordinate
+        double best = -INFINITY;
+        for (int64_t i = gp.gt; i < n + m; i += gp.GT) {
+          const float x = i < n ? __ldg(X + i * d + k) : __ldg(Y + (i - n) * d + k);
+          best = fmax(best, x == x ? (double)(side ? -x : x) : INFINITY);
         }
-        best = fmax(best, q == q ? (double)q * 1.00001 : INFINITY);
+        if (!gmax(gp, s, best)) return false;
+        ext[side] = best;
       }
-      if (!gmax(gp, s, best)) return false;
-      ext[side] = sqrt(best);
+      dmax += (ext[0] + ext[1]) * (ext[0] + ext[1]);
     }
-    dmax = (ext[0] + ext[1]) * (ext[0] + ext[1]);
     return true;
   }
   // the temperature of the sweeps that follow
   __device__ void set_gamma(double gamma) {
-    split_on = split_ok && pg::in_range(gamma * sC * pg::kLog2eD * dmax);
+    split_parts = split_ok ? pg::parts_of(gamma * sC * pg::kLog2eD * dmax) : 0;
     __syncthreads();
     if (threadIdx.x == 0) {
       s.sc[SC_GAMMA] = gamma;
-      if (split_on) s.scale = pg::make_scale(gamma, sC, dmax);
+      if (split_parts) s.scale = pg::make_scale(gamma, sC, dmax);
     }
     __syncthreads();
   }
@@ -630,16 +627,18 @@ struct Dev {
   __device__ bool sweep(const T* w0, const T* w1, const T* w2, Epi epi) {
     sweeps++;
     if constexpr (sizeof(T) == 4) {
-      if (split_on) {
-        // (four own elements per thread run as two rounds of two: the other side's
-        // records are read as often, for half the code)
+      // (four own elements per thread run as two rounds of two: the other side's
+      // records are read as often, for half the code)
+      if (split_parts == 2) {
         if (d <= 2) {
-          if (ro == 1) return sweep_split<2, 1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
-          return sweep_split<2, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+          if (ro == 1) return sweep_split<2, 1, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+          return sweep_split<2, 2, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
         }
-        if (ro == 1) return sweep_split<4, 1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
-        return sweep_split<4, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+        if (ro == 1) return sweep_split<4, 1, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+        return sweep_split<4, 2, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
       }
+      // (three parts: one form, again for less code)
+      if (split_parts == 3) return sweep_split<4, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
       return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
     }
     if (ro == 1) return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
@@ -1070,9 +1069,9 @@ struct Dev {
     for (int64_t j = gp.gt; j < m; j += gp.GT) mt0[j] = logct[j];
     // the first temperature, with the sweeps of the last one, where the time goes
     set_gamma(rg(prm.gamma_f));
-    const bool last = split_on;
+    const int last = split_parts;
     set_gamma(rg(fmin(prm.gamma_i, prm.gamma_f)));
-    if (split_on != last) set_gamma(rg(prm.gamma_f));
+    if (split_parts != last) set_gamma(rg(prm.gamma_f));
     if (!bar()) return false;
     for (int k = 0; k < reps; ++k) {
       if (!col_lse(nt0, nullptr, mt0, nullptr, 0.0, logct, mt0, 1, SC_AUX0, 0.0)) return false;

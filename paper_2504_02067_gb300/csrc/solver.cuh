@@ -184,6 +184,7 @@ struct Solver {
   // ---- point-cloud geometry (pts_geo_of / tc_geo_of above the class) ----
   PtsGeo pts_geo(bool rows) const { return pts_geo_of(h, rows ? n : m, rows ? m : n, d); }
   // ---- split-coordinate point sweeps (mixed precision, d <= pg::kMaxD) ----
+  int pg_parts = 0;      // parts per coordinate, 0: the general sweeps
   bool pg_on = false;
   bool pg_grad = false;  // the gradient sweeps (any d)
   static bool pg_enabled() {
@@ -191,8 +192,8 @@ struct Solver {
     return !(e && e[0] == '0');
   }
   // Sets gamma for the sweeps of this call and decides whether its point sweeps take
-  // split coordinates: their accuracy holds in pg::in_range of gamma s_C log2(e) max
-  // |x - y|^2. A library-computed s_C gives the maximum itself; for a caller's s_C the
+  // split coordinates, and of how many parts (pg::parts_of gamma s_C log2(e) max
+  // |x - y|^2). A library-computed s_C gives the maximum itself; for a caller's s_C the
   // clouds' extent bounds it, which takes a read back (not possible when the call must
   // stay asynchronous).
   // defer: the next split's launch writes gamma (the caller splits before any sweep).
@@ -219,50 +220,89 @@ struct Solver {
   }
   void choose(double gamma) {
     gamma_host = gamma;
-    pg_grad = pg::in_range(gamma * sC * pg::kLog2eD * dmax_host);
+    pg_parts = pg::parts_of(gamma * sC * pg::kLog2eD * dmax_host);
+    pg_grad = pg_parts > 0;
     pg_on = pg_grad && d <= pg::kMaxD;
   }
-  // (max |x - x_0| + max |y - x_0|)^2 >= max |x_i - y_j|^2, from one pass over the points
+  // A bound on max |x_i - y_j|^2 from two passes over the points (pg::extent_kernel).
   double extent_bound() {
-    int* r2 = (int*)h->maxbuf;
-    EOT_CUDA(cudaMemsetAsync(r2, 0, 2 * sizeof(int), st));
+    uint32_t* ext = (uint32_t*)h->maxbuf;
+    static_assert(pg::kExtents * sizeof(uint32_t) <= SC_TOTAL * sizeof(double), "pinned buffer");
+    EOT_CUDA(cudaMemsetAsync(ext, 0, pg::kExtents * sizeof(uint32_t), st));
     const int64_t blocks = std::min<int64_t>((n + m + kThreads - 1) / kThreads, 2 * (int64_t)h->sms);
-    launch_k(pg::extent_kernel, dim3((unsigned)blocks), dim3(kThreads), st, X, Y, n, m, d, r2);
+    launch_k(pg::extent_kernel, dim3((unsigned)blocks), dim3(kThreads), st, X, Y, n, m, d, ext);
     EOT_LAUNCH_CHECK();
     h->launches++;
-    EOT_CUDA(cudaMemcpyAsync(h->h_sc, r2, sizeof(double), cudaMemcpyDeviceToHost, st));
+    uint32_t* bits = (uint32_t*)h->h_sc;
+    EOT_CUDA(cudaMemcpyAsync(bits, ext, pg::kExtents * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     EOT_CUDA(cudaStreamSynchronize(st));
-    float f[2];
-    std::memcpy(f, h->h_sc, sizeof(f));
-    const double rx = std::sqrt((double)f[0]), ry = std::sqrt((double)f[1]);
-    return (rx + ry) * (rx + ry);
+    auto value = [&](int k) {
+      const uint32_t b = pg::unordered_bits(bits[k]);
+      float f;
+      std::memcpy(&f, &b, sizeof(f));
+      return (double)f;
+    };
+    const double r = std::sqrt(value(0)) + std::sqrt(value(1));
+    double diag = 0.0;
+    for (int k = 0; k < d; ++k) diag += std::pow(value(2 + k) + value(66 + k), 2);
+    return std::min(r * r, diag);
   }
-  template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
+  template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, int P, class Epi>
   void launch_pg_at(cudaStream_t s, const SweepArgs<T>& a, const pg::Geo& g, const Epi& e) {
-    launch_kc(pg::sweep_kernel<D, RO, NR, LSE, SQM, ROWS, GRAD, Epi>, dim3((unsigned)g.B, (unsigned)g.S),
+    launch_kc(pg::sweep_kernel<D, RO, NR, LSE, SQM, ROWS, GRAD, P, Epi>, dim3((unsigned)g.B, (unsigned)g.S),
               dim3(kThreads), (unsigned)g.S, 0, s, a, pg::Args{h->sc + SC_DMAX, g.ws}, e);
+  }
+  pg::Geo pg_geo(bool rows, bool grad) const {
+    return pg::geo_of(h->sms, rows ? n : m, rows ? m : n, d, grad, pg_parts);
   }
   template <int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
   void launch_pg(cudaStream_t s, SweepArgs<T> a, const Epi& e) {
-    const pg::Geo g = pg::geo_of(h->sms, ROWS ? n : m, ROWS ? m : n, d, GRAD);
+    const pg::Geo g = pg_geo(ROWS, GRAD);
     a.chunk = g.chunk;
     if (Epi::kDot > 0 && g.B * g.S > h->dot_cap)
       throw EotError{EOT_ERR_INVALID_ARG, "point sweep scratch smaller than the launch needs"};
+    if (pg_parts == 3) {
+      constexpr int R = GRAD ? 1 : 2;
+      if (d <= 2) {
+        if (g.ro == 1) launch_pg_at<2, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+        else launch_pg_at<2, R, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+      } else if (d <= 4) {
+        if (g.ro == 1) launch_pg_at<4, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+        else launch_pg_at<4, R, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+      } else if (d <= 8) {
+        launch_pg_at<8, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+      } else {
+        launch_pg_at<16, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+      }
+      return;
+    }
     constexpr int R4 = GRAD ? 2 : 4, R2 = GRAD ? 1 : 2;  // own elements per thread at small d, at d > 4
     if (d <= 2) {
-      if (g.ro == 1) launch_pg_at<2, 1, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
-      else launch_pg_at<2, R4, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      if (g.ro == 1) launch_pg_at<2, 1, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
+      else launch_pg_at<2, R4, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
     } else if (d == 3) {
-      if (g.ro == 1) launch_pg_at<3, 1, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
-      else launch_pg_at<3, R4, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      if (g.ro == 1) launch_pg_at<3, 1, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
+      else launch_pg_at<3, R4, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
     } else if (d == 4) {
-      if (g.ro == 1) launch_pg_at<4, 1, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
-      else launch_pg_at<4, R4, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      if (g.ro == 1) launch_pg_at<4, 1, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
+      else launch_pg_at<4, R4, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
     } else if (d <= 8) {
-      launch_pg_at<8, R2, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      launch_pg_at<8, R2, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
     } else {
-      launch_pg_at<16, R2, NR, LSE, SQM, ROWS, GRAD>(s, a, g, e);
+      launch_pg_at<16, R2, NR, LSE, SQM, ROWS, GRAD, 2>(s, a, g, e);
     }
+  }
+  template <bool ROWS, int P>
+  void launch_grad_tile(double scale, const double* ownfac, float* out) {
+    SweepArgs<T> a = args();
+    a.wc[0] = ewc();
+    a.wr[0] = ewr();
+    const pg::Geo g = pg::grad_geo(h->sms, ROWS ? n : m, ROWS ? m : n, P == 3 ? 1 : 2);
+    a.chunk = g.chunk;
+    EOT_CUDA(cudaFuncSetAttribute(pg::grad_tile_kernel<ROWS, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(pg::GradSmem<P>)));
+    launch_kc(pg::grad_tile_kernel<ROWS, P>, dim3((unsigned)g.B, (unsigned)g.S), dim3(kThreads), (unsigned)g.S,
+              sizeof(pg::GradSmem<P>), st, a, pg::Args{h->sc + SC_DMAX, 1}, scale, ownfac, out);
   }
   // ---- tensor-core point path (mixed precision, d >= tc::kMinD) ----
   bool tc_on = false;
@@ -606,18 +646,15 @@ struct Solver {
   void grad_pts(double scale, const double* ownfac, float* out) {
     if constexpr (sizeof(T) == 4) {
       if (pg_grad) {
-        SweepArgs<T> a = args();
-        a.wc[0] = ewc();
-        a.wr[0] = ewr();
         if (pg_on) {
+          SweepArgs<T> a = args();
+          a.wc[0] = ewc();
+          a.wr[0] = ewr();
           launch_pg<1, false, 0, ROWS, true>(st, a, pg::GradEpi{scale, ownfac, out, d});
+        } else if (pg_parts == 3) {
+          launch_grad_tile<ROWS, 3>(scale, ownfac, out);
         } else {
-          const pg::Geo g = pg::grad_geo(h->sms, ROWS ? n : m, ROWS ? m : n);
-          a.chunk = g.chunk;
-          EOT_CUDA(cudaFuncSetAttribute(pg::grad_tile_kernel<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)sizeof(pg::GradSmem)));
-          launch_kc(pg::grad_tile_kernel<ROWS>, dim3((unsigned)g.B, (unsigned)g.S), dim3(kThreads), (unsigned)g.S,
-                    sizeof(pg::GradSmem), st, a, pg::Args{h->sc + SC_DMAX, 1}, scale, ownfac, out);
+          launch_grad_tile<ROWS, 2>(scale, ownfac, out);
         }
         EOT_LAUNCH_CHECK();
         h->launches++;
@@ -813,7 +850,7 @@ struct Solver {
     const uintptr_t src = points ? ((uintptr_t)X ^ ((uintptr_t)Y << 1) ^ (uintptr_t)sbits) : (uintptr_t)C;
     const ProgKey key{tag | ((int)sizeof(T) << 4) | ((plain ? 1 : 0) << 8) | ((points ? 1 : 0) << 9) | (d << 10) |
                           ((full_system ? 1 : 0) << 20),
-                      V | ((tc_on ? 1 : 0) << 4) | ((keep_l2 ? 1 : 0) << 5) | ((pg_on ? 1 : 0) << 6), 0, n, m, ldc, src};
+                      V | ((tc_on ? 1 : 0) << 4) | ((keep_l2 ? 1 : 0) << 5) | ((pg_on ? pg_parts - 1 : 0) << 6), 0, n, m, ldc, src};
     auto it = h->graphs.find(key);
     if (it == h->graphs.end()) {
       if (h->graphs.size() >= 32) free_graphs(h);
@@ -1088,7 +1125,7 @@ struct Solver {
           b.wc[0] = zf();
           b.active = h->sc + SC_ACTIVE_COL;
           launch_pg<1, false, 0, true, false>(st, b, PgCgRowEpi{h->rowfac, h->rPs, h->z, h->p, h->y, h->q, h->sc});
-          const pg::Geo g = pg::geo_of(h->sms, n, m, d, false);
+          const pg::Geo g = pg_geo(true, false);
           nrow = (int)(g.B * g.S);
         }
       }

@@ -3,17 +3,28 @@
 // C_ij = s_C |x_i - y_j|^2 on the fly; the exponent is kept in base 2,
 //     t2_ij = (Ah_i + Bh_j) log2 e - |x'_i - y'_j|^2,   x' = sqrt(gamma s_C log2 e) (x - x_0),
 // so that no scaling is left per entry and ex2 takes t2 as it is. Every scaled
-// coordinate is split once per point, x' = xh + xl with xh on a grid of step s (a
+// coordinate is split where it is staged, x' = xh + xl with xh on a grid of step s (a
 // power of two) and |xl| <= s / 2, and
 //     |x' - y'|^2 = sum dh^2 + sum dl (2 dh + dl),   dh = xh - yh, dl = xl - yl.
-// s = 2^ceil(log2(sqrt(D') 2^-11)) for D' >= max |x' - y'|^2 makes dh and dh^2 exact
+// s = 2^ceil(log2(sqrt(D')) - 11.5) for D' >= max |x' - y'|^2 makes dh and dh^2 exact
 // in FP32 and keeps the running sum of Ah + Bh (on the 1/8 grid, s^2 <= 1/8) and the
-// -dh^2 exact while below 4 D'; dl is rounded at 2^-25 s. The pairs that carry the
-// plan's mass have D' of a few tens, so the second sum is of order 10 s and its
-// rounding below 1e-7 of an exponent unit up to D' = 2^15: less than the rounding of
-// t2 itself, and t2 is rounded once where the scheme of sweep_pts.cuh (TwoSum
-// differences, compensated squares, a two-term gamma s_C) rounds four times.
-// Five FP32 instructions per coordinate against eighteen.
+// -dh^2 exact while below 2 D'. What is rounded is dl and the second sum, at 2^-25 of
+// dh s: up to sqrt(D') s where every pair is far apart (translated clouds), so this
+// serves D' <= 2^11. Beyond, up to 2^15, a third part xm on the grid 2^-11 s takes
+// the products dh dm, exact as well, out of the second sum:
+//     sum dh^2 + 2 sum dh dm + sum dm (dm + 2 dl) + 2 sum dh dl.
+// Relative error of the plan's entries (rms over the mass, FP32 emulated against 64
+// bits, Sinkhorn potentials; uniform clouds in the unit cube, then one of them moved
+// by 5; the general sweeps / these):
+//     D'      parts  d = 2                             d = 16
+//     739     2      5.5e-8 / 2.7e-8, 6.1e-8 / 3.2e-8  3.4e-8 / 2.0e-8, 6.7e-8 / 3.9e-8
+//     2047    2      4.7e-8 / 2.3e-8, 6.5e-8 / 3.8e-8  3.1e-8 / 2.1e-8, 4.3e-8 / 3.8e-8
+//     2955    3      4.1e-8 / 2.2e-8, 6.4e-8 / 3.1e-8  3.2e-8 / 1.6e-8, 4.0e-8 / 2.0e-8
+//     31740   3      2.8e-8 / 1.6e-8, 5.2e-8 / 2.5e-8  2.9e-8 / 1.5e-8, 3.0e-8 / 1.6e-8
+// (two parts at 31740, one cloud moved: 3.0e-7 and 5.4e-7). t2 is rounded once; the
+// scheme of sweep_pts.cuh (TwoSum differences, compensated squares, a two-term
+// gamma s_C) rounds four times. Five FP32 instructions per coordinate (eight with
+// three parts) against eighteen.
 //
 // Work split: FP32-issue-bound for large clouds (each thread owns RO elements, the
 // other side's records are broadcast from shared memory), latency-bound for small
@@ -34,8 +45,11 @@ constexpr int kMaxD = 16;
 // every temperature; the general sweeps serve the rest (below, the scale of the
 // coordinates runs out of FP32: a gamma that FP32 rounds to 0, coinciding points).
 constexpr double kMinBound = 0x1p-40;
-constexpr double kMaxBound = 32768.0;
-__host__ __device__ inline bool in_range(double bound) { return bound >= kMinBound && bound <= kMaxBound; }
+constexpr double kMaxTwo = 2048.0;     // two parts per coordinate
+constexpr double kMaxBound = 32768.0;  // three
+__host__ __device__ inline int parts_of(double bound) {  // 0: the general sweeps
+  return !(bound >= kMinBound && bound <= kMaxBound) ? 0 : bound <= kMaxTwo ? 2 : 3;
+}
 // The online max of an LSE moves in whole units of the base-2 exponent, so that every
 // rescaling (here and where partial sums meet) is by an exact power of two.
 constexpr float kThetaB2 = 12.0f;      // lazy-rescale threshold
@@ -55,12 +69,14 @@ struct Geo {
 // Fewest waves x per-thread entries. A CTA's fixed cost (prologue, combine, epilogue:
 // about 2 us) is worth about 48 entries per thread at two CTAs per SM; staging an
 // other-side record costs a thread about 3.5 entries.
-// grad: the gradient sweeps, with a sum per coordinate in registers.
-inline Geo geo_of(int sms, int64_t n_own, int64_t n_oth, int d, bool grad) {
+// grad: the gradient sweeps, with a sum per coordinate in registers; parts: of a coordinate.
+inline Geo geo_of(int sms, int64_t n_own, int64_t n_oth, int d, bool grad, int parts) {
   Geo best{};
   double bc = -1.0;
   for (int ro : {1, 2, 4}) {
-    const bool built = grad ? (ro == 1 || (d <= 4 && ro == 2)) : (d <= 4 ? ro != 2 : ro == 2);
+    const bool built = parts == 3 ? (ro == 1 || (d <= 4 && !grad && ro == 2))
+                       : grad     ? (ro == 1 || (d <= 4 && ro == 2))
+                                  : (d <= 4 ? ro != 2 : ro == 2);
     if (!built) continue;
     for (int ws : {1, 2, 4, 8}) {
       const int64_t own = (int64_t)(kThreads / ws) * ro, B = (n_own + own - 1) / own;
@@ -103,15 +119,23 @@ struct Scale {
   double sigma;
 };
 
-// (x - c) sigma as a grid part and a remainder
-__device__ __forceinline__ void split_coord(float x, float c, const Scale& sc, float& xh, float& xl) {
+// (x - c) sigma as a grid part, (P = 3) a part on the grid 2^-11 s, and a remainder
+template <int P>
+__device__ __forceinline__ void split_coord(float x, float c, const Scale& sc, float& xh, float& xm, float& xl) {
   const float t = sub_rn(x, c);  // TwoSum: x - c = t + e
   const float bv = sub_rn(t, x);
   const float e = sub_rn(sub_rn(x, sub_rn(t, bv)), add_rn(c, bv));
   const float p = mul_rn(t, sc.sh);
   const float pe = fmaf(t, sc.sh, -p) + fmaf(t, sc.sl, e * sc.sh);
   xh = sub_rn(add_rn(p, sc.magic), sc.magic);
-  xl = add_rn(sub_rn(p, xh), pe);
+  const float r = sub_rn(p, xh);
+  if constexpr (P == 3) {
+    const float magic = sc.magic * 0x1p-11f;
+    xm = sub_rn(add_rn(r, magic), magic);
+    xl = add_rn(sub_rn(r, xm), pe);
+  } else {
+    xl = add_rn(r, pe);
+  }
 }
 // A log2 e (A on the 1/8 grid, |A| < 2^19) as a part on the 1/8 grid and a remainder
 __device__ __forceinline__ void split_offset(float A, float& ph, float& pr) {
@@ -134,20 +158,23 @@ __device__ __forceinline__ float ld_cluster_f(const V* p, uint32_t rank) {
 
 // What one thread does with its RO own elements and a tile of the other side's
 // records; shared by the sweep kernel below and the batched solver's sweeps.
-template <int D, int RO, int NR, bool LSE, int SQM, bool GRAD>
+template <int D, int RO, int NR, bool LSE, int SQM, bool GRAD, int P = 2>
 struct Core {
   static constexpr int NA = GRAD ? D : (LSE ? 1 : NR);  // sums per own element
   static constexpr int NW = GRAD || LSE ? 1 : NR;       // weights per other element
-  static constexpr int REC = (2 * D + 2 + NW + 3) / 4 * 4;
-  float xh[RO][D], xl[RO][D], ph[RO], pr[RO];
+  static constexpr int OFF = P * D;                     // a record's offsets, then its weights
+  static constexpr int REC = (OFF + 2 + NW + 3) / 4 * 4;
+  float xh[RO][D], xl[RO][D], xm[RO][P == 3 ? D : 1], ph[RO], pr[RO];
   float S[RO][NA], Cc[RO][NA], mx[RO], hm[RO];
 
   __device__ __forceinline__ void own(int r, bool ev, const float* x, int d, const float (&ctr)[D], const Scale& sc,
                                       float A) {
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      if (ev && k < d) split_coord(__ldg(x + k), ctr[k], sc, xh[r][k], xl[r][k]);
+      float m = 0.f;
+      if (ev && k < d) split_coord<P>(__ldg(x + k), ctr[k], sc, xh[r][k], m, xl[r][k]);
       else xh[r][k] = xl[r][k] = 0.f;
+      if constexpr (P == 3) xm[r][k] = m;
     }
     split_offset(ev ? A : 0.f, ph[r], pr[r]);
     mx[r] = kLowest;
@@ -155,7 +182,7 @@ struct Core {
 #pragma unroll
     for (int k = 0; k < NA; ++k) S[r][k] = Cc[r][k] = 0.f;
   }
-  // one record: [yh (D), yl (D), high offset, low offset, weights]
+  // one record: [yh (D), yl (D), ym (P = 3: D), high offset, low offset, weights]
   static __device__ __forceinline__ void stage(float (&rec)[REC], const float* y, int d, const float (&ctr)[D],
                                                const Scale& sc, float B, const float (&w)[NW]) {
     float v[REC];
@@ -163,10 +190,14 @@ struct Core {
     for (int k = 0; k < REC; ++k) v[k] = 0.f;
 #pragma unroll
     for (int k = 0; k < D; ++k)
-      if (k < d) split_coord(__ldg(y + k), ctr[k], sc, v[k], v[D + k]);
-    split_offset(B, v[2 * D], v[2 * D + 1]);
+      if (k < d) {
+        float m = 0.f;
+        split_coord<P>(__ldg(y + k), ctr[k], sc, v[k], m, v[D + k]);
+        if constexpr (P == 3) v[2 * D + k] = m;
+      }
+    split_offset(B, v[OFF], v[OFF + 1]);
 #pragma unroll
-    for (int k = 0; k < NW; ++k) v[2 * D + 2 + k] = w[k];
+    for (int k = 0; k < NW; ++k) v[OFF + 2 + k] = w[k];
 #pragma unroll
     for (int k = 0; k < REC; k += 4)
       *reinterpret_cast<float4*>(&rec[k]) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
@@ -183,13 +214,27 @@ struct Core {
   }
   // t2 of own element r and the record v (h: the own side's high offset)
   __device__ __forceinline__ float expo2(int r, float h, const float (&v)[REC]) const {
-    float acc = h + v[2 * D];
-    float lo = pr[r] + v[2 * D + 1];
+    float acc = h + v[OFF];
+    float lo = pr[r] + v[OFF + 1];
+    if constexpr (P == 2) {
 #pragma unroll
-    for (int k = 0; k < D; ++k) {
-      const float dh = xh[r][k] - v[k], dl = xl[r][k] - v[D + k];
-      acc = fmaf(-dh, dh, acc);
-      lo = fmaf(-dl, fmaf(2.0f, dh, dl), lo);
+      for (int k = 0; k < D; ++k) {
+        const float dh = xh[r][k] - v[k], dl = xl[r][k] - v[D + k];
+        acc = fmaf(-dh, dh, acc);
+        lo = fmaf(-dl, fmaf(2.0f, dh, dl), lo);
+      }
+    } else {
+      float mid = 0.f, low = 0.f;  // sum dh dm (exact), sum dh dl
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const float dh = xh[r][k] - v[k], dl = xl[r][k] - v[D + k], dm = xm[r][k] - v[2 * D + k];
+        acc = fmaf(-dh, dh, acc);
+        mid = fmaf(dh, dm, mid);
+        lo = fmaf(-dm, fmaf(2.0f, dl, dm), lo);
+        low = fmaf(dh, dl, low);
+      }
+      acc = fmaf(-2.0f, mid, acc);
+      lo = fmaf(-2.0f, low, lo);
     }
     return acc + lo;
   }
@@ -211,7 +256,7 @@ struct Core {
           for (int u = 0; u < G; ++u) {
             float v[REC];
             load(rec[min(q + u, qe - 1)], v);
-            w[u] = q + u < qe ? v[2 * D + 2] : 0.f;
+            w[u] = q + u < qe ? v[OFF + 2] : 0.f;
 #pragma unroll
             for (int r = 0; r < RO; ++r) t[r][u] = expo2(r, hm[r], v);
           }
@@ -258,15 +303,18 @@ struct Core {
           for (int r = 0; r < RO; ++r) {
             const float ex = ex2_approx(expo2(r, ph[r], v));
             if constexpr (GRAD) {
-              const float pw = ex * v[2 * D + 2];
+              const float pw = ex * v[OFF + 2];
 #pragma unroll
-              for (int k = 0; k < D; ++k)
-                acc[r][k] = fmaf(pw, (xh[r][k] - v[k]) + (xl[r][k] - v[D + k]), acc[r][k]);
+              for (int k = 0; k < D; ++k) {
+                float low = xl[r][k] - v[D + k];
+                if constexpr (P == 3) low += xm[r][k] - v[2 * D + k];
+                acc[r][k] = fmaf(pw, (xh[r][k] - v[k]) + low, acc[r][k]);
+              }
             } else {
 #pragma unroll
               for (int k = 0; k < NR; ++k) {
-                if ((SQM >> k) & 1) acc[r][k] = fmaf(ex * ex, v[2 * D + 2 + k], acc[r][k]);
-                else acc[r][k] = fmaf(ex, v[2 * D + 2 + k], acc[r][k]);
+                if ((SQM >> k) & 1) acc[r][k] = fmaf(ex * ex, v[OFF + 2 + k], acc[r][k]);
+                else acc[r][k] = fmaf(ex, v[OFF + 2 + k], acc[r][k]);
               }
             }
           }
@@ -280,15 +328,16 @@ struct Core {
   }
 };
 
-// sigma and the grid of one temperature: kap = gamma s_C log2 e, dmax >= max |x - y|^2
+// sigma and the grid of one temperature: kap = gamma s_C log2 e, dmax >= max |x - y|^2,
+// parts_of(kap dmax) > 0
 __device__ __forceinline__ Scale make_scale(double gamma, double sC, double dmax) {
   const double kap = gamma * sC * kLog2eD;
   Scale s;
   s.sigma = sqrt(kap);
   s.sh = (float)s.sigma;
   s.sl = (float)(s.sigma - (double)s.sh);
-  // s = 2^ceil(log2(sqrt(kap dmax) 2^-11)), at least 2^-30
-  const int ex = max(ilogb(sqrt(kap * dmax)) + 1 - 11, -30);
+  // s = 2^ceil(log2(sqrt(kap dmax)) - 11.5) (twice that at some powers of two), at least 2^-30
+  const int ex = max((ilogb(kap * dmax) - 21) >> 1, -30);
   s.magic = 1.5f * __int_as_float((127 + 23 + ex) << 23);
   return s;
 }
@@ -317,9 +366,9 @@ __device__ __forceinline__ void combine_groups(float2 (*red)[L], float* rmx, int
   }
 }
 
-template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, class Epi>
+template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, int P, class Epi>
 __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(SweepArgs<float> a, Args g, Epi epi) {
-  using C = Core<D, RO, NR, LSE, SQM, GRAD>;
+  using C = Core<D, RO, NR, LSE, SQM, GRAD, P>;
   constexpr int NA = C::NA, NW = C::NW, REC = C::REC;
   constexpr int TO = D <= 4 ? 256 : 128;
   constexpr int ND = Epi::kDot;
@@ -448,11 +497,14 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(SweepArgs<float> a, 
 // entries. Two CTAs per SM; a cluster of up to 8 CTAs splits the other side.
 // A training step of
 // n = m = 16384, d = 64: 339 -> 236 ms.
-constexpr int kGR = 64, kGC = 128, kGK = 32, kGD = 64;
+// Three parts (P = 3): 8 d for the exponent, chunks half as long, one CTA per SM.
+constexpr int kGR = 64, kGC = 128, kGD = 64;
+template <int P>
 struct GradSmem {
-  float xs[2][kGD][kGR];  // the own side's xh, xl, coordinate-major; at the end the sums as pairs
+  static constexpr int kGK = P == 3 ? 16 : 32;
+  float xs[P][kGD][kGR];  // the own side's xh, xl (, xm), coordinate-major; at the end the sums as pairs
   union {
-    float ys[2][kGK][kGC + 4];  // a chunk of the tile's yh, yl
+    float ys[P][kGK][kGC + 4];  // a chunk of the tile's yh, yl (, ym)
     float p[kGC][kGR + 4];      // weighted plan entries of the tile
   };
   float yr[kGC][kGD];           // the tile's coordinates (zeros beyond d)
@@ -460,11 +512,12 @@ struct GradSmem {
   Scale sc;
 };
 
-template <bool ROWS>
-__global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float> a, Args g, double scale,
-                                                                const double* ownfac, float* out) {
+template <bool ROWS, int P>
+__global__ void __launch_bounds__(kThreads, P == 3 ? 1 : 2) grad_tile_kernel(SweepArgs<float> a, Args g, double scale,
+                                                                             const double* ownfac, float* out) {
+  constexpr int kGK = GradSmem<P>::kGK;
   extern __shared__ __align__(16) unsigned char raw[];
-  GradSmem& s = *reinterpret_cast<GradSmem*>(raw);
+  GradSmem<P>& s = *reinterpret_cast<GradSmem<P>*>(raw);
   const int64_t n_own = ROWS ? a.n : a.m, n_oth = ROWS ? a.m : a.n;
   const float* xo = ROWS ? a.X : a.Y;
   const float* xt = ROWS ? a.Y : a.X;
@@ -481,10 +534,11 @@ __global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float>
   const Scale sc = s.sc;
   for (int q = tid; q < kGR * kGD; q += kThreads) {
     const int r = q / kGD, k = q % kGD;
-    float xh = 0.f, xl = 0.f;
-    if (e0 + r < n_own && k < d) split_coord(__ldg(xo + (e0 + r) * d + k), __ldg(a.X + k), sc, xh, xl);
+    float xh = 0.f, xm = 0.f, xl = 0.f;
+    if (e0 + r < n_own && k < d) split_coord<P>(__ldg(xo + (e0 + r) * d + k), __ldg(a.X + k), sc, xh, xm, xl);
     s.xs[0][k][r] = xh;
     s.xs[1][k][r] = xl;
+    if constexpr (P == 3) s.xs[2][k][r] = xm;
   }
   const int rg = tid >> 4, cg = tid & 15;  // elements 4 rg .. + 3; columns 4 cg .. + 3 and 64 + 4 cg .. + 3
   float ph[4], pr[4];
@@ -510,11 +564,16 @@ __global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float>
 
   for (int64_t jt = j0; jt < j1; jt += kGC) {
     const int tn = (int)min((int64_t)kGC, j1 - jt);
-    unsigned long long q2[4][4], l2[4][4];  // sum dh^2 and sum dl (2 dh + dl), pairs of columns
+    // pairs of columns: sum dh^2, sum dl (2 dh + dl); P = 3: the latter is sum dm (dm + 2 dl),
+    // and sum dh dm, sum dh dl
+    unsigned long long q2[4][4], l2[4][4], mid2[4][P == 3 ? 4 : 1], low2[4][P == 3 ? 4 : 1];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) q2[r][e] = l2[r][e] = 0ull;
+      for (int e = 0; e < 4; ++e) {
+        q2[r][e] = l2[r][e] = 0ull;
+        if constexpr (P == 3) mid2[r][e] = low2[r][e] = 0ull;
+      }
     for (int k0 = 0; k0 < d; k0 += kGK) {
       const int kn = min(kGK, d - k0);
       __syncthreads();  // the previous chunk (or the previous tile's entries) is done with
@@ -533,15 +592,17 @@ __global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float>
         const float c = __ldg(a.X + k0 + lane);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          float h[4], l[4];
+          float h[4], l[4], md[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const int jj = 4 * (warp + 8 * q) + e;
-            h[e] = l[e] = 0.f;
-            if (jj < tn) split_coord(__ldg(xt + (jt + jj) * d + k0 + lane), c, sc, h[e], l[e]);
+            h[e] = l[e] = md[e] = 0.f;
+            if (jj < tn) split_coord<P>(__ldg(xt + (jt + jj) * d + k0 + lane), c, sc, h[e], md[e], l[e]);
           }
           *reinterpret_cast<float4*>(&s.ys[0][lane][4 * (warp + 8 * q)]) = make_float4(h[0], h[1], h[2], h[3]);
           *reinterpret_cast<float4*>(&s.ys[1][lane][4 * (warp + 8 * q)]) = make_float4(l[0], l[1], l[2], l[3]);
+          if constexpr (P == 3)
+            *reinterpret_cast<float4*>(&s.ys[2][lane][4 * (warp + 8 * q)]) = make_float4(md[0], md[1], md[2], md[3]);
         }
       }
       __syncthreads();
@@ -555,6 +616,15 @@ __global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float>
         const ulonglong2 lb = *reinterpret_cast<const ulonglong2*>(&s.ys[1][k][64 + 4 * cg]);
         const float xh[4] = {xh4.x, xh4.y, xh4.z, xh4.w}, xl[4] = {xl4.x, xl4.y, xl4.z, xl4.w};
         const unsigned long long yh[4] = {ha.x, ha.y, hb.x, hb.y}, yl[4] = {la.x, la.y, lb.x, lb.y};
+        float xm[4];
+        unsigned long long ym[4];
+        if constexpr (P == 3) {
+          const float4 xm4 = *reinterpret_cast<const float4*>(&s.xs[2][k0 + k][4 * rg]);
+          const ulonglong2 ma = *reinterpret_cast<const ulonglong2*>(&s.ys[2][k][4 * cg]);
+          const ulonglong2 mb = *reinterpret_cast<const ulonglong2*>(&s.ys[2][k][64 + 4 * cg]);
+          xm[0] = xm4.x, xm[1] = xm4.y, xm[2] = xm4.z, xm[3] = xm4.w;
+          ym[0] = ma.x, ym[1] = ma.y, ym[2] = mb.x, ym[3] = mb.y;
+        }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           unsigned long long nh, nl;
@@ -566,8 +636,18 @@ __global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float>
             asm("add.rn.f32x2 %0, %1, %2;" : "=l"(dh) : "l"(yh[e]), "l"(nh));
             asm("add.rn.f32x2 %0, %1, %2;" : "=l"(dl) : "l"(yl[e]), "l"(nl));
             asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(q2[r][e]) : "l"(dh));
-            asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(two2), "l"(dh), "l"(dl));
-            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(l2[r][e]) : "l"(dl), "l"(t));
+            if constexpr (P == 3) {
+              unsigned long long nm, dm;
+              asm("mov.b64 %0, {%1, %1};" : "=l"(nm) : "f"(-xm[r]));
+              asm("add.rn.f32x2 %0, %1, %2;" : "=l"(dm) : "l"(ym[e]), "l"(nm));
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(mid2[r][e]) : "l"(dh), "l"(dm));
+              asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(two2), "l"(dl), "l"(dm));
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(l2[r][e]) : "l"(dm), "l"(t));
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(low2[r][e]) : "l"(dh), "l"(dl));
+            } else {
+              asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(two2), "l"(dh), "l"(dl));
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(l2[r][e]) : "l"(dl), "l"(t));
+            }
           }
         }
       }
@@ -582,8 +662,19 @@ __global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float>
         float qa, qb, la, lb;
         asm("mov.b64 {%0, %1}, %2;" : "=f"(qa), "=f"(qb) : "l"(q2[r][e]));
         asm("mov.b64 {%0, %1}, %2;" : "=f"(la), "=f"(lb) : "l"(l2[r][e]));
-        const float ta = ((ph[r] + s.qh[col]) - qa) + ((pr[r] + s.qr[col]) - la);
-        const float tb = ((ph[r] + s.qh[col + 1]) - qb) + ((pr[r] + s.qr[col + 1]) - lb);
+        float ta = (ph[r] + s.qh[col]) - qa, tb = (ph[r] + s.qh[col + 1]) - qb;
+        float ua = (pr[r] + s.qr[col]) - la, ub = (pr[r] + s.qr[col + 1]) - lb;
+        if constexpr (P == 3) {
+          float ma, mb, wa, wb;
+          asm("mov.b64 {%0, %1}, %2;" : "=f"(ma), "=f"(mb) : "l"(mid2[r][e]));
+          asm("mov.b64 {%0, %1}, %2;" : "=f"(wa), "=f"(wb) : "l"(low2[r][e]));
+          ta = fmaf(-2.0f, ma, ta);
+          tb = fmaf(-2.0f, mb, tb);
+          ua = fmaf(-2.0f, wa, ua);
+          ub = fmaf(-2.0f, wb, ub);
+        }
+        ta += ua;
+        tb += ub;
         pa[r] = ex2_approx(ta) * s.w[col];
         pb[r] = ex2_approx(tb) * s.w[col + 1];
       }
@@ -653,14 +744,14 @@ __global__ void __launch_bounds__(kThreads, 2) grad_tile_kernel(SweepArgs<float>
   cluster_sync();  // no CTA leaves while another reads its shared memory
 }
 
-// Chunks of the other side: the fewest waves x (tiles per CTA + 1), two CTAs per SM.
-inline Geo grad_geo(int sms, int64_t n_own, int64_t n_oth) {
+// Chunks of the other side: the fewest waves x (tiles per CTA + 1); per_sm CTAs per SM.
+inline Geo grad_geo(int sms, int64_t n_own, int64_t n_oth, int per_sm) {
   Geo best{};
   int64_t bc = -1;
-  const int64_t B = (n_own + kGR - 1) / kGR, tiles = (n_oth + kGC - 1) / kGC;
+  const int64_t B = (n_own + kGR - 1) / kGR, tiles = (n_oth + kGC - 1) / kGC, slots = (int64_t)per_sm * sms;
   for (int64_t k = 1; k <= 8 && k <= tiles; ++k) {
     const int64_t tk = (tiles + k - 1) / k, S = (tiles + tk - 1) / tk;
-    const int64_t c = (B * S + 2 * sms - 1) / (2 * sms) * (tk + 1);
+    const int64_t c = (B * S + slots - 1) / slots * (tk + 1);
     if (bc >= 0 && c >= bc) continue;
     bc = c;
     best = Geo{B, S, tk * kGC, 0, 0};
@@ -668,30 +759,54 @@ inline Geo grad_geo(int sms, int64_t n_own, int64_t n_oth) {
   return best;
 }
 
-// max over both clouds of |x - x_0|^2 (FP32, rounded up by a part in 10^5) as a bound
-// on their extent: |x_i - y_j| <= |x_i - x_0| + |y_j - x_0|. r2[0]: X, r2[1]: Y (zeroed;
-// a NaN or overflow gives an infinite bound).
+// Two bounds on max |x_i - y_j|^2 for a caller's s_C. ext[0], ext[1]: max |x - x_0|^2 and
+// max |y - x_0|^2 (FP32, rounded up by a part in 10^5), since |x_i - y_j| <= |x_i - x_0| +
+// |y_j - x_0|; ext[2 + k], ext[66 + k]: the largest x_k and -x_k of either cloud, the box
+// whose squared diagonal bounds it too (the tighter one in few dimensions). All of them
+// as ordered integers, zeroed before; a NaN makes them infinite. The grid's threads are a
+// multiple of d in the second loop, so that each stays with one coordinate.
+__host__ __device__ inline uint32_t ordered_bits(uint32_t b) { return b >> 31 ? ~b : b | 0x80000000u; }
+__host__ __device__ inline uint32_t unordered_bits(uint32_t b) { return b >> 31 ? b & 0x7fffffffu : ~b; }
+constexpr int kExtents = 2 + 2 * 64;
 static __global__ void __launch_bounds__(kThreads) extent_kernel(const float* X, const float* Y, int64_t n, int64_t m,
-                                                                 int d, int* r2) {
+                                                                 int d, uint32_t* ext) {
+  __shared__ uint32_t box[kExtents];
+  for (int q = threadIdx.x; q < kExtents; q += kThreads) box[q] = 0u;
+  __syncthreads();
   pdl_wait();
-  float bx = 0.f, by = 0.f;
-  for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < n + m; q += (int64_t)gridDim.x * kThreads) {
+  auto up = [](float x) { return ordered_bits(__float_as_uint(x == x ? x : INFINITY)); };
+  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x, T = (int64_t)gridDim.x * kThreads;
+  float r[2] = {0.f, 0.f};
+  for (int64_t q = t; q < n + m; q += T) {
     const float* p = q < n ? X + q * d : Y + (q - n) * d;
     float s = 0.f;
     for (int k = 0; k < d; ++k) {
-      const float t = __ldg(p + k) - __ldg(X + k);
-      s = fmaf(t, t, s);
+      const float e = __ldg(p + k) - __ldg(X + k);
+      s = fmaf(e, e, s);
     }
     s = s == s ? s * 1.00001f : INFINITY;
-    if (q < n) bx = fmaxf(bx, s);
-    else by = fmaxf(by, s);
+    r[q < n ? 0 : 1] = fmaxf(r[q < n ? 0 : 1], s);
   }
-  bx = warp_max_f(bx);
-  by = warp_max_f(by);
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(r2, __float_as_int(bx));
-    atomicMax(r2 + 1, __float_as_int(by));
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const float w = warp_max_f(r[c]);
+    if ((threadIdx.x & 31) == 0) atomicMax(&box[c], up(w));
   }
+  const int64_t Td = T / d * d;
+  if (t < Td) {
+    float hi = -INFINITY, lo = -INFINITY;
+    for (int64_t q = t; q < (n + m) * d; q += Td) {
+      const float x = __ldg(q < n * d ? X + q : Y + (q - n * d));
+      hi = fmaxf(hi, x == x ? x : INFINITY);
+      lo = fmaxf(lo, x == x ? -x : INFINITY);
+    }
+    const int k = (int)(t % d);
+    atomicMax(&box[2 + k], up(hi));
+    atomicMax(&box[66 + k], up(lo));
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < kExtents; q += kThreads)
+    if (box[q]) atomicMax(ext + q, box[q]);
 }
 
 }  // namespace pg

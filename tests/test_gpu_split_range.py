@@ -96,3 +96,52 @@ def test_solve_across_the_range(H, n, m, d, gamma_f):
         assert status == [0, 0]
         for a, b in zip(us, vs):
             assert O.marginal_l1_error(a.cpu().numpy(), b.cpu().numpy(), gamma_f, C, r, c) <= 1e-6
+
+
+@pytest.mark.parametrize("d", [1, 2, 3, 8, 16, 33])
+@pytest.mark.parametrize("shift", [0.0, 5.0])
+@pytest.mark.parametrize("gamma", [1400.0, 2600.0, 16384.0, 22000.0])
+@pytest.mark.parametrize("given", [False, True])
+def test_accuracy_over_the_range(H, d, shift, gamma, given):
+    """Overlapping clouds, and one of them moved away so that every pair is far apart and
+    the potentials cancel most of the cost. Errors against 64 bits, relative to the sum of
+    absolute terms: at most 1.5 times the general sweeps' plus 2e-8, a sixth of an FP32
+    rounding (the entries' own errors are smaller than the general sweeps'; in sums over
+    entries the two schemes' roundings average differently)."""
+    from paper_2504_02067_gb300 import Problem
+    n, m = 300, 260
+    rng = np.random.default_rng(d)
+    X, Y = (rng.uniform(0, 1, size=(k, d)).astype(np.float32) for k in (n, m))
+    Y[:, 0] += np.float32(shift)
+    sC = O.sqeuclid_scale(X, Y)
+    C = sC * O.sqeuclid(X, Y)
+    u, v, g = np.zeros(n), np.zeros(m), 16.0
+    while True:  # Sinkhorn steps along a rising gamma
+        for _ in range(30):
+            u = -np.log(n) - O.lse_r(v[None, :] - g * C)
+            v = -np.log(m) - O.lse_c(u[:, None] - g * C)
+        if g >= gamma:
+            break
+        g, f = min(2.0 * g, gamma), min(2.0, gamma / g)
+        u, v = u * f, v * f
+    P = np.exp(u[:, None] + v[None, :] - gamma * C)
+    prob = Problem(X=t(X, torch.float32), Y=t(Y, torch.float32), precision="mixed", cost_scale=sC if given else 0.0)
+    du, dv = rng.normal(size=n), rng.normal(size=m)
+
+    def run():
+        mg = H.marginals(prob, t(u), t(v), gamma)
+        hv = H.hvp(prob, t(u), t(v), gamma, 0.9, t(du), t(dv))
+        dX, dY = (torch.empty(k, d, dtype=torch.float32, device=DEV) for k in (n, m))
+        H.eot_backward(prob, t(u), t(v), gamma, dX=dX, dY=dY)
+        return [x.cpu().numpy() for x in (mg[0], mg[1], hv[0], hv[1], dX, dY)]
+
+    D = X[:, None, :].astype(np.float64) - Y[None, :, :]
+    r, c = P.sum(1), P.sum(0)
+    want = [r, c, r * du + 0.9 * (P @ dv), 0.9 * (P.T @ du) + c * dv,
+            2 * sC * np.einsum("ij,ijk->ik", P, D), -2 * sC * np.einsum("ij,ijk->jk", P, D)]
+    size = [r, c, np.abs(r * du) + 0.9 * (P @ np.abs(dv)), 0.9 * (P.T @ np.abs(du)) + np.abs(c * dv),
+            2 * sC * np.einsum("ij,ijk->ik", P, np.abs(D)), 2 * sC * np.einsum("ij,ijk->jk", P, np.abs(D))]
+    got, gen = run(), general(run)
+    for k, (a, b, w, z) in enumerate(zip(got, gen, want, size)):
+        ea, eb = np.abs(a - w).sum() / z.sum(), np.abs(b - w).sum() / z.sum()
+        assert ea <= 1.5 * eb + 2e-8, (k, ea, eb)
