@@ -637,8 +637,11 @@ struct Dev {
         if (ro == 1) return sweep_split<4, 1, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
         return sweep_split<4, 2, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
       }
-      // (three parts: one form, again for less code)
-      if (split_parts == 3) return sweep_split<4, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+      // (three parts: one own element per thread, again for less code)
+      if (split_parts == 3) {
+        if (d <= 2) return sweep_split<2, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+        return sweep_split<4, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+      }
       return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
     }
     if (ro == 1) return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);

@@ -262,13 +262,15 @@ struct Solver {
     if (Epi::kDot > 0 && g.B * g.S > h->dot_cap)
       throw EotError{EOT_ERR_INVALID_ARG, "point sweep scratch smaller than the launch needs"};
     if (pg_parts == 3) {
-      constexpr int R = GRAD ? 1 : 2;
       if (d <= 2) {
         if (g.ro == 1) launch_pg_at<2, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
-        else launch_pg_at<2, R, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
-      } else if (d <= 4) {
+        else launch_pg_at<2, 2, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+      } else if (d == 3) {
+        if (g.ro == 1) launch_pg_at<3, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+        else launch_pg_at<3, 2, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+      } else if (d == 4) {
         if (g.ro == 1) launch_pg_at<4, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
-        else launch_pg_at<4, R, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
+        else launch_pg_at<4, 2, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
       } else if (d <= 8) {
         launch_pg_at<8, 1, NR, LSE, SQM, ROWS, GRAD, 3>(s, a, g, e);
       } else {

@@ -74,7 +74,7 @@ inline Geo geo_of(int sms, int64_t n_own, int64_t n_oth, int d, bool grad, int p
   Geo best{};
   double bc = -1.0;
   for (int ro : {1, 2, 4}) {
-    const bool built = parts == 3 ? (ro == 1 || (d <= 4 && !grad && ro == 2))
+    const bool built = parts == 3 ? (ro == 1 || (d <= 4 && ro == 2))
                        : grad     ? (ro == 1 || (d <= 4 && ro == 2))
                                   : (d <= 4 ? ro != 2 : ro == 2);
     if (!built) continue;
