@@ -250,9 +250,10 @@ eot_status eot_solve(eot_handle h, const eot_problem* prob, const eot_params* pa
  * with no host round trip: a cooperative launch of all co-resident CTAs, formed
  * into groups of G CTAs that take problems from a queue, largest n m first.
  * G and the own elements per thread are chosen by an autotuner that times
- * probe sweeps of the actual batch (once per batch shape, cached in the
- * handle; EOT_BATCH_CFG="G,k" in the environment forces G in {1,2,4,8} and
- * k in {1,2,4}).
+ * probe sweeps of the actual batch (once per batch shape and kind of sweep, cached
+ * in the handle; EOT_BATCH_CFG="G,k" in the environment forces G in {1,2,4,8} and
+ * k in {1,2,4}; of k, the sweeps from split coordinates use at most 2, with three
+ * parts per coordinate 1).
  * probs: host array [nprob]; every problem EOT_COST_SQEUCLID_POINTS with
  *   1 <= d <= 4, 1 <= n, m <= 32768, all MIXED or all FP64; r, c, X, Y device.
  *   cost_scale <= 0: s_C = 1 / max |x_i - y_j|^2 computed per problem.

@@ -642,7 +642,6 @@ struct Dev {
         if (d <= 2) return sweep_split<2, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
         return sweep_split<4, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
       }
-      return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
     }
     if (ro == 1) return sweep_ro<1, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
     if (ro == 2) return sweep_ro<2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
@@ -1278,8 +1277,19 @@ double launch_batch(eot_handle h, const std::vector<Prob>& probs, const std::vec
   return ms;
 }
 
+// The sweeps that a problem's last stages take, as far as the host knows: the general
+// ones, split coordinates of 2 or 3 parts, or (a caller's scale, whose bound the device
+// forms) some of these at this magnitude of gamma_f.
+std::string sweep_kind(const Prob& p, const bt::Params& prm, size_t elem) {
+  if (elem != 4 || !prm.pgrid) return "g";
+  const double gf = (double)(float)prm.gamma_f;
+  if (p.sC <= 0.0) return std::to_string(pg::parts_of(gf * pg::kLog2eD * 1.00001));
+  return "e" + std::to_string(std::ilogb(gf));
+}
+
 // Autotuner: times the probe (two column-fix + row LSE pairs per problem) of the
-// actual batch for each candidate (G, elements per thread) and keeps the fastest.
+// actual batch for each candidate (G, elements per thread) and keeps the fastest, per
+// shapes and kinds of sweeps.
 template <class T>
 std::pair<int, int> tune(eot_handle h, const std::vector<Prob>& probs, const std::vector<int32_t>& order,
                          bt::Params prm, int64_t maxN, int64_t maxM, cudaStream_t st) {
@@ -1291,7 +1301,12 @@ std::pair<int, int> tune(eot_handle h, const std::vector<Prob>& probs, const std
       return {G, ro};
   }
   std::string key = std::to_string(sizeof(T)) + ":";
-  for (const Prob& p : probs) key += std::to_string(p.n) + "x" + std::to_string(p.m) + "x" + std::to_string(p.d) + ",";
+  bool general = false;  // some problem may take the general sweeps
+  for (const Prob& p : probs) {
+    const std::string kind = sweep_kind(p, prm, sizeof(T));
+    general = general || (kind != "2" && kind != "3");
+    key += std::to_string(p.n) + "x" + std::to_string(p.m) + "x" + std::to_string(p.d) + kind + ",";
+  }
   auto it = h->bt_tune.find(key);
   if (it != h->bt_tune.end()) return it->second;
   prm.probe = 2;
@@ -1299,11 +1314,10 @@ std::pair<int, int> tune(eot_handle h, const std::vector<Prob>& probs, const std
   const int resident = max_resident_ctas<T>(h);
   std::pair<int, int> best{2, 2};
   double best_ms = INFINITY;
-  const bool split = sizeof(T) == 4 && prm.pgrid;
   for (int G : {1, 2, 4, 8}) {
     if (G > resident) continue;
     for (int ro : {1, 2, 4}) {
-      if (split && ro == 4) continue;
+      if (!general && ro == 4) continue;  // (the split sweeps run it as 2)
       const double ms = launch_batch<T>(h, probs, order, outs, G, ro, prm, maxN, maxM, st);
       if (ms < best_ms) {
         best_ms = ms;
