@@ -326,11 +326,11 @@ struct Solver {
     const int64_t npX = tc::pad_rows(n), npY = tc::pad_rows(m);
     ensure_tc_mem(h, n, m, st);
     unsigned char* b = (unsigned char*)h->tc_mem;
-    unsigned long long* emax = (unsigned long long*)b;  // [2]
+    unsigned long long* emax = (unsigned long long*)b;  // [4]
     targs.emax = emax;
-    targs.kappa = (float*)(b + 2 * sizeof(unsigned long long));
+    targs.kappa = (float*)(b + 4 * sizeof(unsigned long long));
     b += 256;
-    EOT_CUDA(cudaMemsetAsync(emax, 0, 2 * sizeof(unsigned long long), st));
+    EOT_CUDA(cudaMemsetAsync(emax, 0, 4 * sizeof(unsigned long long), st));
     auto take = [&](size_t bytes) {
       unsigned char* p = b;
       b += (bytes + 255) / 256 * 256;
@@ -353,7 +353,7 @@ struct Solver {
       h->launches++;
     };
     extent(X, n, emax);
-    extent(Y, m, emax + 1);
+    extent(Y, m, emax + 2);
     targs.err = h->status;
     for (bool rows : {true, false}) {
       const TcGeo g = tc_geo(rows);

@@ -5,20 +5,32 @@
 // Exactness (an exact-slice / Ozaki-style splitting). Both point sets are moved
 // by one common centre c (the first point of X; exact in FP64, distances do not
 // change). Each cloud gets one exponent E (every centred coordinate |x_k| < 2^E)
-// and every coordinate is rounded to 2^(E-37) and cut into four balanced digits of
+// and every coordinate is rounded to 2^(E-b) and cut into four balanced digits of
 // radix 1024,
-//     x_k = 2^(E-7) sum_s d_sk 2^-10s,   |d_0| <= 128, -512 <= d_s < 512,
+//     x_k = 2^(E-b+30) sum_s d_sk 2^-10s,   |d_0| <= 2^(b-30), -512 <= d_s < 512,
 // integers that FP16 holds exactly. The 10 slice pairs (s, t) with s + t <= 3 are
-// added into four "level" accumulators S_L = sum_{s+t=L} D_s D_t^T: over 64
-// coordinates |S_0| <= 2^20 and |S_1| <= 2^23 are exact in the FP32 accumulator
-// whatever the data, S_2 and S_3 while below 2^24 (one unit off, 2^-20 and less of a
-// level-0 unit, beyond), and
-//     x . y = 2^(Ex + Ey - 14) G,   G = S_0 + 2^-10 S_1 + 2^-20 S_2 + 2^-30 S_3
-// to about 2^-36 of the largest |x||y| (the dropped pairs s + t >= 4 and the
-// coordinates' rounding): at gamma = 2^10 about 1e-9 of an exponent unit, a hundredth
-// of the exponent's own FP32 rounding. (Five signed 8-bit digits in BF16 take 15
-// pairs for 2^-38: a training step of n = m = 16384, d = 64 took 384 ms, with ten
-// pairs 339 ms.) Coordinates beyond d are zero: only ceil(d / 16) of the four K = 16 steps
+// added into four "level" accumulators S_L = sum_{s+t=L} D_s D_t^T, and
+//     x . y = 2^(Ex + Ey - 2b + 60) G,   G = S_0 + 2^-10 S_1 + 2^-20 S_2 + 2^-30 S_3.
+// b = 38 keeps S_0 and S_1 exact in the FP32 accumulator whatever the data (over 64
+// coordinates |S_0| <= 2^22, |S_1| <= 2^24). S_1 is at most 512 times the sum of two
+// points' |d_0|, so b is 39 or 40 where the largest points' sums of |x_k| allow it
+// (tc_scale; |S_0| stays within 2^24 then), which they do unless points lie near the
+// corners of the clouds' cube: each bit makes what is dropped four times smaller. S_2
+// and S_3 are exact while below 2^24 (one unit off, 2^-20 and less of a level-0 unit,
+// beyond). What is dropped, the pairs s + t >= 4, is 2^-23.6 sqrt(3 d) (rms) of a
+// level-0 unit 2^(Ex + Ey - 2b + 60), in scaled coordinates (below) of an exponent
+// unit. Where that exceeds 2^-27 the three pairs s + t = 4 are issued too: into level
+// 3's accumulator, whose first MMA scales it by 2^-10 (scale-input-d). The rest is
+// the coordinates' rounding. Row sums off (L1 over the mass; emulated, 300 Sinkhorn-
+// balanced points, uniform d = 17 / eight Gaussians d = 64), FP32 rounding included:
+//     gamma    five 8-bit digits,   these             (b = 37, ten pairs always)
+//              fifteen pairs
+//     2^10     4.4e-9 / 6.8e-9      3.8e-9 / 5.5e-9   1.8e-8 / 3.0e-8
+//     2^12     6.6e-9 / 1.6e-8      3.5e-9 / 4.9e-9   7.1e-8 / 1.3e-7
+//     2^14     2.3e-8 / 5.9e-8      4.0e-9 / 4.6e-9   2.9e-7 / 5.3e-7
+//     2^18     3.7e-7 / 9.7e-7      5.6e-8 / 5.7e-8   4.7e-6 / 8.7e-6
+// A CG column sweep of n = m = 16384, d = 64: 0.263 ms with ten pairs, 0.34 with thirteen
+// (0.36 with fifteen pairs of BF16 digits). Coordinates beyond d are zero: only ceil(d / 16) of the four K = 16 steps
 // of a pair are issued.
 //
 // Exponent algebra. In base-2 units (t2 = t log2 e) the exponent of the plan is
@@ -81,7 +93,7 @@ constexpr int kM = 128;     // own points per CTA = TMEM lanes = MMA M
 constexpr int kN = 96;      // other-side points per tile = MMA N
 constexpr int kSlices = 4;  // radix-1024 digits per coordinate
 constexpr int kLevels = 4;  // s + t = 0 .. 3
-constexpr int kCoordBits = 37;  // |x_k| 2^-E in units of 2^-37
+constexpr int kMinBits = 38, kMaxBits = 40;  // |x_k| 2^-E in units of 2^-b
 constexpr int kEpiWarps = 12;                  // 3 per TMEM lane quarter
 constexpr int kParts = kEpiWarps / 4;          // column parts of a tile
 constexpr int kPartCols = kN / kParts;         // 32 columns per epilogue warp and tile
@@ -130,8 +142,8 @@ struct Side {
 };
 struct TcArgs {
   Side X, Y;
-  const unsigned long long* emax;  // [2] bits of the FP64 max |x_k - c_k| of X and of Y
-  float* kappa;                    // [1] 2^a (per sweep)
+  const unsigned long long* emax;  // [4] bits of the FP64 max |x_k - c_k| and max sum_k |x_k - c_k| of X, then of Y
+  float* kappa;                    // [2] 2^a, 1 where the pairs s + t = 4 are needed (per sweep)
   int* err;                        // status word: kStatTimeout on a wait that ran out, kStatRange
 };
 
@@ -151,18 +163,50 @@ __device__ __forceinline__ int cloud_exp(unsigned long long bits, double sigma) 
   return e;
 }
 
-// max_{i,k} |x_ik - c_k| of one cloud (FP64, exact differences) into *emax as
-// the bits of a non-negative double (ordered like the values). *emax starts at 0.
+// The digits of one temperature: sigma, the clouds' exponents and the bits b.
+struct TcScale {
+  double sigma;
+  int ex, ey, bits;
+  __device__ __forceinline__ int a() const { return ex + ey - 2 * (bits - 30); }  // x' . y' = 2^a G
+};
+__device__ __forceinline__ TcScale tc_scale(const TcArgs& ta, double gamma, double sC) {
+  TcScale s;
+  s.sigma = tc_sigma(gamma, sC);
+  s.ex = cloud_exp(ta.emax[0], s.sigma);
+  s.ey = cloud_exp(ta.emax[2], s.sigma);
+  // the largest points' sums of |x'_k| 2^-E: with b bits sum |d_0| <= 2^(b-30) that + 33
+  const double sum = s.sigma * (ldexp(__longlong_as_double((long long)ta.emax[1]), -s.ex) +
+                                ldexp(__longlong_as_double((long long)ta.emax[3]), -s.ey));
+  s.bits = kMaxBits;
+  while (s.bits > kMinBits && !(ldexp(sum, s.bits - 30) + 66.0 <= 32768.0)) --s.bits;
+  return s;
+}
+
+// max_{i,k} |x_ik - c_k| and max_i sum_k |x_ik - c_k| of one cloud (FP64, exact
+// differences; one warp per point) into emax[0] and emax[1] as the bits of non-negative
+// doubles (ordered like the values), which start at 0.
 static __global__ void tc_extent_kernel(const float* X, int64_t n, int d, const float* centre,
                                         unsigned long long* emax) {
   pdl_wait();
-  double mx = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * d;
-       i += (int64_t)gridDim.x * blockDim.x)
-    mx = fmax(mx, fabs((double)X[i] - (double)centre[i % d]));
+  const int lane = threadIdx.x & 31;
+  const double c0 = lane < d ? (double)centre[lane] : 0.0, c1 = lane + 32 < d ? (double)centre[lane + 32] : 0.0;
+  double mx = 0.0, ms = 0.0;
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < n;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const double a = lane < d ? fabs((double)X[i * d + lane] - c0) : 0.0;
+    const double b = lane + 32 < d ? fabs((double)X[i * d + lane + 32] - c1) : 0.0;
+    mx = fmax(mx, fmax(a, b));
+    double s = a + b;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    ms = fmax(ms, s);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0 && mx > 0.0) atomicMax(emax, (unsigned long long)__double_as_longlong(mx));
+  if (lane == 0 && mx > 0.0) {
+    atomicMax(emax, (unsigned long long)__double_as_longlong(mx));
+    atomicMax(emax + 1, (unsigned long long)__double_as_longlong(ms));
+  }
 }
 
 // One warp per point of either cloud (rows >= n and coordinates >= d are zero): the
@@ -190,13 +234,13 @@ static __global__ void tc_prep_kernel(SweepArgs<float> a, TcArgs ta) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
   const float g = a.gamma_dev ? (float)*a.gamma_dev : a.gamma;
-  const double sigma = tc_sigma((double)g, a.sC);
-  const int e = cloud_exp(ta.emax[isx ? 0 : 1], sigma);
+  const TcScale sc = tc_scale(ta, (double)g, a.sC);
+  const int e = isx ? sc.ex : sc.ey;
   if (lane == 0) const_cast<double*>(sd.nx)[row] = q;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const int k = lane + 32 * c;
-    long long Q = (long long)rint(ldexp(xv[c] * sigma, kCoordBits - e));  // |Q| <= 2^37
+    long long Q = (long long)rint(ldexp(xv[c] * sc.sigma, sc.bits - e));  // |Q| <= 2^b
     const int64_t idx = row * 64 + (((k >> 3) ^ (int)(row & 7)) << 3) + (k & 7);
 #pragma unroll
     for (int s = kSlices - 1; s > 0; --s) {  // balanced digits from the lowest up
@@ -204,11 +248,11 @@ static __global__ void tc_prep_kernel(SweepArgs<float> a, TcArgs ta) {
       sl[(int64_t)s * npad * 64 + idx] = __float2half_rn((float)dig);
       Q = (Q - dig) >> 10;
     }
-    sl[idx] = __float2half_rn((float)Q);  // |Q| <= 128
+    sl[idx] = __float2half_rn((float)Q);  // |Q| <= 2^(b - 30)
   }
 }
 
-// Before each sweep: 2^a, the other side's records (all npad of them; padded
+// Before each sweep: 2^a and the choice of pairs, the other side's records (all npad of them; padded
 // points get Qh = -2^23 and weights 0, so no tile needs a mask) and the own
 // side's P split. The same gamma as the sweep: (float) of the device value.
 template <int NR, int SQM, bool ROWS>
@@ -222,8 +266,10 @@ __global__ void tc_sweep_prep_kernel(SweepArgs<float> a, TcArgs ta) {
   const double K = (double)g * a.sC;
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i == 0) {
-    const double sg = tc_sigma((double)g, a.sC);
-    ta.kappa[0] = (float)ldexp(1.0, cloud_exp(ta.emax[0], sg) + cloud_exp(ta.emax[1], sg) - 14);
+    const double k0 = ldexp(1.0, tc_scale(ta, (double)g, a.sC).a());
+    ta.kappa[0] = (float)k0;
+    // 2^-23.6 sqrt(3 d) 2^a > 2^-27
+    ta.kappa[1] = k0 * k0 * (3.0 * a.d) > 0x1p-7 ? 1.f : 0.f;
   }
   if (i < sq.npad) {
     constexpr int RW = rec_floats(NR);
@@ -286,6 +332,9 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* e
   if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, err, kStatTimeout, kTcWaitNs, kEpiSleepNs) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
+
+template <int V>
+using I = std::integral_constant<int, V>;
 
 template <int NR, bool LSE, int SQM, bool ROWS, class Epi>
 __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float> a, TcArgs ta, Epi epi) {
@@ -394,8 +443,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
     // queue stays fed while the epilogue warps compete for issue slots (one issuer
     // loses ~25 % of the MMA rate to them). Per tile each waits for the slices, then
     // for the epilogue to have loaded levels {0,1} and {2,3} of the previous tile,
-    // issues and commits its level of either pair, and commits its use of the slice
-    // buffer (sfree[buffer][issuer]).
+    // issues and commits its level of either pair (A, where they are needed, the three
+    // pairs of level 4 before level 3), and commits its use of the slice buffer
+    // (sfree[buffer][issuer]).
     if (lane == 0) {
       const int who = warp == 0 ? 0 : 1;
       const int ksteps = (a.d + 15) / 16;
@@ -405,7 +455,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
       // every MMA adds a compile-time offset (all unrolled)
       const uint32_t acol = tbase + kOwnCol;
       const uint64_t bdesc0 = desc_sw128(smem_u32(sm + kOffOth));
-      auto level = [&](uint64_t bdesc, int L) {
+      const uint32_t four = ta.kappa[1] != 0.f ? 1u : 0u;
+      auto level = [&](uint64_t bdesc, auto Lc) {
+        constexpr int L = Lc.value;
 #pragma unroll
         for (int k4 = 0; k4 < 4; ++k4) {
           if (k4 >= ksteps) break;  // coordinates beyond d are zero
@@ -413,10 +465,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
           for (int s = 0; s < kSlices; ++s) {
             const int t = L - s;
             if (t < 0 || t >= kSlices) continue;
-            mma_f16(tbase + (uint32_t)(L * kN), acol + (uint32_t)(s * 32 + k4 * 8),
-                     bdesc + (uint64_t)((t * kOthSlice + k4 * 32) >> 4), kIdesc,
-                     (k4 == 0 && s == 0) ? 0u : 1u);
+            const uint32_t at = tbase + (uint32_t)(L * kN), am = acol + (uint32_t)(s * 32 + k4 * 8);
+            const uint64_t bm = bdesc + (uint64_t)((t * kOthSlice + k4 * 32) >> 4);
+            if (L == 3 && k4 == 0 && s == 0) mma_f16_scaled10(at, am, bm, kIdesc, four);
+            else mma_f16(at, am, bm, kIdesc, (k4 == 0 && s == 0) ? 0u : 1u);
           }
+        }
+      };
+      // the pairs s + t = 4 into level 3's accumulator (which then starts from 2^-10 of it);
+      // rolled: the loop over the tiles stays short where they are not needed
+      auto level4 = [&](uint64_t bdesc) {
+#pragma unroll 1
+        for (int k4 = 0; k4 < ksteps; ++k4) {
+#pragma unroll
+          for (int s = 1; s < kSlices; ++s)
+            mma_f16(tbase + (uint32_t)(3 * kN), acol + (uint32_t)(s * 32 + k4 * 8),
+                    bdesc + (uint64_t)(((4 - s) * kOthSlice + k4 * 32) >> 4), kIdesc, (k4 == 0 && s == 1) ? 0u : 1u);
         }
       };
       int committed = 0;
@@ -431,15 +495,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
           ok = false;
         } else {
           tc_fence_after();
-          if (who == 0) level(bdesc, 0);
-          else level(bdesc, 1);
+          if (who == 0) level(bdesc, I<0>());
+          else level(bdesc, I<1>());
           mma_commit(&lvl[0]);
           if (tt >= 1 && !mbar_wait(&lfree[1], ppar, ta.err, kStatTimeout)) {
             ok = false;
           } else {
             tc_fence_after();
-            if (who == 0) level(bdesc, 3);
-            else level(bdesc, 2);
+            if (who == 0) {
+              if (four) level4(bdesc);
+              level(bdesc, I<3>());
+            } else {
+              level(bdesc, I<2>());
+            }
             mma_commit(&lvl[1]);
           }
         }
@@ -569,9 +637,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sweep_kernel(SweepArgs<float
         }
       } else {
         // G = S_0 + 2^-10 S_1 + ... as an FP32 pair (gh, gl) in (u0, u1). S_0 is an
-        // integer up to 2^20 and 2^-10 S_1 a multiple of 2^-10 up to 2^13: where
+        // integer up to 2^24 and 2^-10 S_1 a multiple of 2^-10 up to 2^14: where
         // |S_0| >= |2^-10 S_1| Fast2Sum is exact, and otherwise the sum stays within
-        // 2^14 on the 2^-10 grid and is exact already (z = 2^-10 S_1, error 0).
+        // 2^15 and h - S_0 is a multiple of 2^-9 or 2^-10 that FP32 holds, so z and the
+        // error are exact as well.
 #pragma unroll
         for (int c = 0; c < kPartCols; ++c) {
           const float s0 = __uint_as_float(u0[c]), s1 = __uint_as_float(u1[c]);

@@ -40,8 +40,10 @@ def balanced(C, gamma):
         u, v = u * f, v * f
 
 
-@pytest.mark.parametrize("e", [8])
-@pytest.mark.parametrize("kind,d,shift", [("corners", 64, 0.0), ("corners", 32, 0.0)])
+@pytest.mark.parametrize("e", [8, 10, 12, 14, 16, 18])
+@pytest.mark.parametrize("kind,d,shift", [("uniform", 17, 0.0), ("uniform", 64, 0.0), ("gaussians", 33, 0.0),
+                                          ("gaussians", 64, 0.0), ("uniform", 20, 5.0), ("gaussians", 64, 20.0),
+                                          ("corners", 64, 0.0), ("corners", 32, 0.0)])
 def test_marginals_and_products(H, e, kind, d, shift, monkeypatch):
     """The two LSE sweeps and the two weighted sweeps (Hessian-vector product) against 64
     bits. L1 errors relative to the sum of absolute terms: at most 1.5 times the general
