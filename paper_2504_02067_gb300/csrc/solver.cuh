@@ -46,14 +46,16 @@ inline PtsGeo pts_geo_of(eot_handle h, int64_t n_own, int64_t n_oth, int d) {
 // tensor-core sweeps: own blocks of 128 points x S chunks of the other side
 // (multiples of 96), one CTA per SM. A CTA pays a fixed cost besides its tiles
 // (its own slices and first tile before the first MMA, the last tile's
-// arithmetic, the partials and the finishing CTA's combine), about two tiles'
-// time: at n = m = 16384 a CG sweep took 0.392, 0.363, 0.404 and 0.397 ms with
-// 13, 7, 4 and 1 chunks, which that cost fits. S minimises
-// waves x (that cost + tiles per CTA).
+// arithmetic, the partials and the finishing CTA's combine), about three tiles'
+// time: at n = m = 16384, d = 64 a CG column sweep took 0.295, 0.263, 0.284 and 0.274 ms
+// with 13, 7, 4 and 1 chunks, which that cost and 1.58 us per tile fit within 3 %. S
+// minimises waves x (that cost + tiles per CTA). (With two tiles' time the choice at
+// 10000, 20000 and 32768 points is 7, 11 and 7 chunks: 0.121, 0.414 and 0.948 ms; with
+// three 5, 7 and 4: 0.120, 0.405 and 0.940 ms.)
 struct TcGeo {
   int64_t B, S, chunk;
 };
-constexpr int64_t kTcCtaOverheadTiles = 2;
+constexpr int64_t kTcCtaOverheadTiles = 3;
 inline TcGeo tc_geo_of(eot_handle h, int64_t n_own, int64_t n_oth) {
   TcGeo g;
   g.B = (n_own + tc::kM - 1) / tc::kM;
