@@ -165,6 +165,8 @@ struct CgStage {
   double colfac[kCgMaxStrip];     // colfac and c(P) of the strip (read by the finisher)
   double cP[kCgMaxStrip];
   double iters, rzprev;           // SC_ITERS, SC_RZPREV
+  double beta;                    // prepare_warp's results
+  int first;
 };
 __device__ __forceinline__ CgStage& cg_stage_smem() {
   __shared__ __align__(16) CgStage st;
@@ -172,13 +174,13 @@ __device__ __forceinline__ CgStage& cg_stage_smem() {
 }
 
 // Column half: w_j = (P^T (rowfac z))_j + beta w_prev_j; zf_j = colfac_j^2 w_j / c(P)_j,
-// with beta = <res, z> / <res, z>_prev (0 on the first iteration). begin(): warp 0
-// starts asynchronous copies of what the strip's epilogue needs (the update
+// with beta = <res, z> / <res, z>_prev (0 on the first iteration). begin(): the last
+// warp starts asynchronous copies of what the strip's epilogue needs (the update
 // kernel's partials, w_prev, colfac and c(P) of the strip's columns, two
-// scalars) into shared
-// memory, where they land while the CTA sweeps; drain(): warp 0 waits for them;
-// prepare() (the CTAs that finish a strip): beta and the stop test ||res||_1 <=
-// tol or the iteration cap, published by the finisher of strip 0. When the test
+// scalars) into shared memory, where they land while the CTA sweeps; drain(): it
+// waits for them; prepare_warp() (that warp, of the CTAs that finish columns): beta and
+// the stop test ||res||_1 <= tol or the iteration cap, published by one finisher of
+// strip 0; take(): every thread reads them after a barrier. When the test
 // stops CG this sweep's results are not used: the row half and the update see
 // the cleared flag and return.
 template <class T>
@@ -199,12 +201,13 @@ struct CgColFusedEpi {
   int acol;            // slot of the stop decision: the row half reads it, the update kernel commits it
   __device__ void begin(int64_t strip0, int sw, int64_t m) {
     j0 = strip0;
-    if (threadIdx.x < 32) {
+    if (threadIdx.x >= kThreads - 32) {
+      const int lane = threadIdx.x & 31;
       CgStage& s = cg_stage_smem();
-      for (int k = threadIdx.x; k < nparts; k += 32) cp_async16(s.part + 2 * k, part + 2 * k);
+      for (int k = lane; k < nparts; k += 32) cp_async16(s.part + 2 * k, part + 2 * k);
       // w_prev of the strip (pairs of columns: the strip start is a multiple of 32 V >= 32)
       const int w = (int)min((int64_t)sw, m - strip0);
-      for (int k = 2 * threadIdx.x; k < w; k += 64) {
+      for (int k = 2 * lane; k < w; k += 64) {
         if (k + 1 < w) {
           cp_async16(s.wprev + k, wprev + strip0 + k);
           cp_async16(s.colfac + k, colfac + strip0 + k);
@@ -215,7 +218,7 @@ struct CgColFusedEpi {
           cp_async8(s.cP + k, cP + strip0 + k);
         }
       }
-      if (threadIdx.x == 0) {
+      if (lane == 0) {
         cp_async8(&s.iters, sc + SC_ITERS);
         cp_async8(&s.rzprev, sc + SC_RZPREV);
       }
@@ -223,39 +226,46 @@ struct CgColFusedEpi {
     }
   }
   __device__ void drain() {
-    if (threadIdx.x < 32) asm volatile("cp.async.wait_all;" ::: "memory");
+    if (threadIdx.x >= kThreads - 32) asm volatile("cp.async.wait_all;" ::: "memory");
   }
-  __device__ void prepare(bool publish) {
-    __shared__ double sbeta;
-    __shared__ int sfirst;
+  // the last warp, whose copies these are; take() by every thread after a barrier
+  __device__ void prepare_warp(bool publish) {
     CgStage& st = cg_stage_smem();
-    __syncthreads();  // the copies warp 0 waited for are visible to every thread
-    if (threadIdx.x < 32) {
-      double rz, r1;
-      sum_cg_partials(st.part, nparts, rz, r1);
-      if (threadIdx.x == 0) {
-        const double it = st.iters;
-        const bool f = it == 0.0;
-        const double b = f ? 0.0 : rz / st.rzprev;
-        sbeta = b;
-        sfirst = f ? 1 : 0;
-        if (publish) {
-          const bool fin = isfinite(rz) && isfinite(r1) && isfinite(b);
-          const bool go = fin && r1 > sc[SC_TOL] && it < sc[SC_MAXIT] && it < 1.0e6;
-          sc[SC_RZ] = rz;
-          sc[SC_RESL1] = r1;
-          sc[SC_BETA] = b;
-          if (!fin) atomicOr(status, kStatCgNan);
-          if (!go) {
-            sc[acol] = 0.0;  // not SC_ACTIVE: the other CTAs of this launch may still read it
-            if (cond) cudaGraphSetConditional(cond, 0);
-          }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    double rz, r1;
+    sum_cg_partials(st.part, nparts, rz, r1);
+    if ((threadIdx.x & 31) == 0) {
+      const double it = st.iters;
+      const bool f = it == 0.0;
+      const double b = f ? 0.0 : rz / st.rzprev;
+      st.beta = b;
+      st.first = f ? 1 : 0;
+      if (publish) {
+        const bool fin = isfinite(rz) && isfinite(r1) && isfinite(b);
+        const bool go = fin && r1 > sc[SC_TOL] && it < sc[SC_MAXIT] && it < 1.0e6;
+        sc[SC_RZ] = rz;
+        sc[SC_RESL1] = r1;
+        sc[SC_BETA] = b;
+        if (!fin) atomicOr(status, kStatCgNan);
+        if (!go) {
+          sc[acol] = 0.0;  // not SC_ACTIVE: the other CTAs of this launch may still read it
+          if (cond) cudaGraphSetConditional(cond, 0);
         }
       }
     }
+  }
+  __device__ void take() {
+    const CgStage& st = cg_stage_smem();
+    beta = st.beta;
+    first = st.first != 0;
+  }
+  // a CTA that finishes a strip of the ticketed sweep (all threads)
+  __device__ void prepare(bool publish) {
     __syncthreads();
-    beta = sbeta;
-    first = sfirst != 0;
+    if (threadIdx.x >= kThreads - 32) prepare_warp(publish);
+    __syncthreads();
+    take();
   }
   __device__ void col(int64_t j, const double* s, double* d) {
     const CgStage& st = cg_stage_smem();

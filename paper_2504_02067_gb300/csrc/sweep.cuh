@@ -827,21 +827,28 @@ __global__ void __launch_bounds__(kThreads, kColCtasPerSm) col_sweep_kernel(Swee
   if constexpr (CL) {
     // ---- the strip's CTAs combine through distributed shared memory ----
     const uint32_t rank = cluster_rank();
-    if constexpr (HasPrefetch<Epi>::value) {  // (before the barrier: it needs no column sums)
-      epi.drain();
-      epi.prepare(strip == 0 && rank == 0);
+    if constexpr (HasPrefetch<Epi>::value) {  // by the last warp, while the first ones combine the column sums
+      if (warp == kWarps - 1) epi.prepare_warp(strip == 0 && rank == 0);
     }
-    cluster_sync();  // every CTA's column sums are visible to the cluster
+    cluster_sync();  // every CTA's column sums (and beta) are visible to the cluster
+    if constexpr (HasPrefetch<Epi>::value) epi.take();
     const int per = (SW + R - 1) / R;  // columns this CTA finishes
     const int lo = (int)rank * per, hi = min(SW, lo + per);
     for (int cc = lo + threadIdx.x; cc < hi; cc += kThreads) {
       const int64_t jj = strip * SW + cc;
       if (jj >= a.m) continue;
       float s0 = 0.f, c0 = 0.f;
-      for (int r = 0; r < R; ++r) {  // in rank order, as the ticketed combine adds row blocks
-        const float2 q = ld_cluster_f2(&ccol[cc], (uint32_t)r);
-        kadd(s0, c0, q.x);
-        c0 += q.y;
+      for (int r0 = 0; r0 < R; r0 += kColClusterMax) {  // in rank order, as the ticketed combine adds row blocks
+        float2 q[kColClusterMax];  // one round trip of remote reads
+#pragma unroll
+        for (int r = 0; r < kColClusterMax; ++r)
+          if (r0 + r < R) q[r] = ld_cluster_f2(&ccol[cc], (uint32_t)(r0 + r));
+#pragma unroll
+        for (int r = 0; r < kColClusterMax; ++r) {
+          if (r0 + r >= R) continue;
+          kadd(s0, c0, q[r].x);
+          c0 += q[r].y;
+        }
       }
       double s[1] = {(double)s0 + (double)c0};
       double d[1];
