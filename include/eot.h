@@ -253,7 +253,7 @@ eot_status eot_solve(eot_handle h, const eot_problem* prob, const eot_params* pa
  * probe sweeps of the actual batch (once per batch shape and kind of sweep, cached
  * in the handle; EOT_BATCH_CFG="G,k" in the environment forces G in {1,2,4,8} and
  * k in {1,2,4}; of k, the sweeps from split coordinates use at most 2, with three
- * parts per coordinate 1).
+ * parts per coordinate and d > 2 1).
  * probs: host array [nprob]; every problem EOT_COST_SQEUCLID_POINTS with
  *   1 <= d <= 4, 1 <= n, m <= 32768, all MIXED or all FP64; r, c, X, Y device.
  *   cost_scale <= 0: s_C = 1 / max |x_i - y_j|^2 computed per problem.

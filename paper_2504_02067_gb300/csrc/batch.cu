@@ -337,7 +337,7 @@ struct Dev {
     __syncthreads();
   }
 
-  // A = x + alpha y - z split into h (1/8 grid, exact in T) + l (FP64), as split_kernel
+  // A = x + alpha y - z split into h (1/8 grid, exact in T) + l (FP64), as split_pair_kernel
   __device__ void split(int64_t len, const double* xa, const double* ya, double alpha, const double* za,
                         T* h, double* l, T* ew, double* fac, const double* fshift) {
     for (int64_t i = gp.gt; i < len; i += gp.GT) {
@@ -637,9 +637,12 @@ struct Dev {
         if (ro == 1) return sweep_split<4, 1, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
         return sweep_split<4, 2, 2, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
       }
-      // (three parts: one own element per thread, again for less code)
+      // (three parts above the plane: one own element per thread, again for less code)
       if (split_parts == 3) {
-        if (d <= 2) return sweep_split<2, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+        if (d <= 2) {
+          if (ro == 1) return sweep_split<2, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+          return sweep_split<2, 2, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
+        }
         return sweep_split<4, 1, 3, NR, LSE, SQM, ROWS>(w0, w1, w2, epi);
       }
     }
