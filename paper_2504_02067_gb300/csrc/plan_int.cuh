@@ -212,8 +212,9 @@ __device__ __forceinline__ bool support_bounds(const Screen& sc, float V, double
 // into a shared tile by the CTA (shared by its rows); a lane streams its part of
 // the row in batches of 16 entries (4 x 16 bytes when the rows are aligned), the
 // next batch's loads in flight while one is tested. Bound by the read of C:
-// n = m = 4096, FP32 (67 MB), argmax and support together: 349 -> 56 us; with
-// three CTAs per SM (512 CTAs, the second wave nearly empty) 78 us.
+// n = m = 4096, FP32 (67 MB), argmax and support together: 349 -> 56 us on one GB300 (60
+// to 86 us on others); with three CTAs per SM (512 CTAs, the second wave nearly empty) 78
+// us where it took 56.
 constexpr int kScreenTile = 4096;
 template <class T, int V, int MODE>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && V > 1 ? 4 : 2) plan_screen_dense_kernel(int64_t n, int64_t m, const T* C, int64_t ldc,

@@ -226,7 +226,7 @@ struct Solver {
     pg_grad = pg_parts > 0;
     pg_on = pg_grad && d <= pg::kMaxD;
   }
-  // A bound on max |x_i - y_j|^2 from two passes over the points (pg::extent_kernel).
+  // A bound on max |x_i - y_j|^2 from one or two passes over the points (pg::extent_kernel).
   double extent_bound() {
     uint32_t* ext = (uint32_t*)h->maxbuf;
     static_assert(pg::kExtents * sizeof(uint32_t) <= SC_TOTAL * sizeof(double), "pinned buffer");
@@ -245,8 +245,9 @@ struct Solver {
       return (double)f;
     };
     const double r = std::sqrt(value(0)) + std::sqrt(value(1));
+    if (d > pg::kBoxD) return r * r;
     double diag = 0.0;
-    for (int k = 0; k < d; ++k) diag += std::pow(value(2 + k) + value(66 + k), 2);
+    for (int k = 0; k < d; ++k) diag += std::pow(value(2 + k) + value(2 + pg::kBoxD + k), 2);
     return std::min(r * r, diag);
   }
   template <int D, int RO, int NR, bool LSE, int SQM, bool ROWS, bool GRAD, int P, class Epi>

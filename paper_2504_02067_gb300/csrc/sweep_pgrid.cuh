@@ -761,13 +761,14 @@ inline Geo grad_geo(int sms, int64_t n_own, int64_t n_oth, int per_sm) {
 
 // Two bounds on max |x_i - y_j|^2 for a caller's s_C. ext[0], ext[1]: max |x - x_0|^2 and
 // max |y - x_0|^2 (FP32, rounded up by a part in 10^5), since |x_i - y_j| <= |x_i - x_0| +
-// |y_j - x_0|; ext[2 + k], ext[66 + k]: the largest x_k and -x_k of either cloud, the box
-// whose squared diagonal bounds it too (the tighter one in few dimensions). All of them
-// as ordered integers, zeroed before; a NaN makes them infinite. The grid's threads are a
-// multiple of d in the second loop, so that each stays with one coordinate.
+// |y_j - x_0|; up to kBoxD dimensions, where it is the tighter one, ext[2 + k] and
+// ext[2 + kBoxD + k]: the largest x_k and -x_k of either cloud, the box whose squared
+// diagonal bounds it too. All of them as ordered integers, zeroed before; a NaN makes them
+// infinite. The grid's threads are a multiple of d in the second loop, so that each stays
+// with one coordinate.
 __host__ __device__ inline uint32_t ordered_bits(uint32_t b) { return b >> 31 ? ~b : b | 0x80000000u; }
 __host__ __device__ inline uint32_t unordered_bits(uint32_t b) { return b >> 31 ? b & 0x7fffffffu : ~b; }
-constexpr int kExtents = 2 + 2 * 64;
+constexpr int kBoxD = 8, kExtents = 2 + 2 * kBoxD;
 static __global__ void __launch_bounds__(kThreads) extent_kernel(const float* X, const float* Y, int64_t n, int64_t m,
                                                                  int d, uint32_t* ext) {
   __shared__ uint32_t box[kExtents];
@@ -780,6 +781,7 @@ static __global__ void __launch_bounds__(kThreads) extent_kernel(const float* X,
   for (int64_t q = t; q < n + m; q += T) {
     const float* p = q < n ? X + q * d : Y + (q - n) * d;
     float s = 0.f;
+#pragma unroll 8
     for (int k = 0; k < d; ++k) {
       const float e = __ldg(p + k) - __ldg(X + k);
       s = fmaf(e, e, s);
@@ -793,7 +795,7 @@ static __global__ void __launch_bounds__(kThreads) extent_kernel(const float* X,
     if ((threadIdx.x & 31) == 0) atomicMax(&box[c], up(w));
   }
   const int64_t Td = T / d * d;
-  if (t < Td) {
+  if (d <= kBoxD && t < Td) {
     float hi = -INFINITY, lo = -INFINITY;
     for (int64_t q = t; q < (n + m) * d; q += Td) {
       const float x = __ldg(q < n * d ? X + q : Y + (q - n * d));
@@ -802,7 +804,7 @@ static __global__ void __launch_bounds__(kThreads) extent_kernel(const float* X,
     }
     const int k = (int)(t % d);
     atomicMax(&box[2 + k], up(hi));
-    atomicMax(&box[66 + k], up(lo));
+    atomicMax(&box[2 + kBoxD + k], up(lo));
   }
   __syncthreads();
   for (int q = threadIdx.x; q < kExtents; q += kThreads)

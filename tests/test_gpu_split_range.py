@@ -98,7 +98,7 @@ def test_solve_across_the_range(H, n, m, d, gamma_f):
             assert O.marginal_l1_error(a.cpu().numpy(), b.cpu().numpy(), gamma_f, C, r, c) <= 1e-6
 
 
-@pytest.mark.parametrize("d", [1, 2, 3, 8, 16, 33])
+@pytest.mark.parametrize("d", [1, 2, 3, 8, 16, 17, 33, 64])
 @pytest.mark.parametrize("shift", [0.0, 5.0])
 @pytest.mark.parametrize("gamma", [1400.0, 2600.0, 16384.0, 22000.0])
 @pytest.mark.parametrize("given", [False, True])
