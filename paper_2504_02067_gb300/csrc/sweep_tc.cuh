@@ -182,30 +182,40 @@ __device__ __forceinline__ TcScale tc_scale(const TcArgs& ta, double gamma, doub
   return s;
 }
 
-// max_{i,k} |x_ik - c_k| and max_i sum_k |x_ik - c_k| of one cloud (FP64, exact
-// differences; one warp per point) into emax[0] and emax[1] as the bits of non-negative
-// doubles (ordered like the values), which start at 0.
+// max_{i,k} |x_ik - c_k| (FP64, exact differences) and a bound on max_i sum_k |x_ik - c_k|
+// (FP32, rounded up) of one cloud, one warp per point, into emax[0] and emax[1] as the bits
+// of non-negative doubles (ordered like the values: compared as integers, off the FP64
+// pipe), which start at 0.
 static __global__ void tc_extent_kernel(const float* X, int64_t n, int d, const float* centre,
                                         unsigned long long* emax) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
-  const double c0 = lane < d ? (double)centre[lane] : 0.0, c1 = lane + 32 < d ? (double)centre[lane + 32] : 0.0;
-  double mx = 0.0, ms = 0.0;
+  const float c0 = lane < d ? centre[lane] : 0.f, c1 = lane + 32 < d ? centre[lane + 32] : 0.f;
+  const double w0 = widen(c0), w1 = widen(c1);
+  unsigned long long mx = 0ull;
+  float ms = 0.f;
+  auto far = [&](float x, double w) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(widen(x) - w) & 0x7fffffffffffffffull;
+    mx = mx > b ? mx : b;
+  };
   for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < n;
        i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const double a = lane < d ? fabs((double)X[i * d + lane] - c0) : 0.0;
-    const double b = lane + 32 < d ? fabs((double)X[i * d + lane + 32] - c1) : 0.0;
-    mx = fmax(mx, fmax(a, b));
-    double s = a + b;
+    const float a = lane < d ? X[i * d + lane] : c0, b = lane + 32 < d ? X[i * d + lane + 32] : c1;
+    far(a, w0);
+    far(b, w1);
+    float s = fabsf(a - c0) + fabsf(b - c1);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    ms = fmax(ms, s);
+    ms = fmaxf(ms, s == s ? s : INFINITY);
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0 && mx > 0.0) {
-    atomicMax(emax, (unsigned long long)__double_as_longlong(mx));
-    atomicMax(emax + 1, (unsigned long long)__double_as_longlong(ms));
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long b = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = mx > b ? mx : b;
+  }
+  if (lane == 0 && mx > 0ull) {
+    atomicMax(emax, mx);
+    atomicMax(emax + 1, (unsigned long long)__double_as_longlong((double)ms * 1.00001));
   }
 }
 
@@ -215,7 +225,10 @@ static __global__ void tc_extent_kernel(const float* X, int64_t n, int d, const 
 // so the expansion |x|^2 + |y|^2 - 2 x.y keeps its accuracy however far the clouds lie
 // from the origin. gamma_dev (nullable): gamma is read on the device.
 static __global__ void tc_prep_kernel(SweepArgs<float> a, TcArgs ta) {
+  __shared__ TcScale scale;  // (its FP64 operations once per CTA)
   pdl_wait();
+  if (threadIdx.x == 0) scale = tc_scale(ta, (double)(a.gamma_dev ? (float)*a.gamma_dev : a.gamma), a.sC);
+  __syncthreads();
   const int64_t grow = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31, d = a.d;
   const bool isx = grow < ta.X.npad;
@@ -233,8 +246,7 @@ static __global__ void tc_prep_kernel(SweepArgs<float> a, TcArgs ta) {
   double q = xv[0] * xv[0] + xv[1] * xv[1];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-  const float g = a.gamma_dev ? (float)*a.gamma_dev : a.gamma;
-  const TcScale sc = tc_scale(ta, (double)g, a.sC);
+  const TcScale sc = scale;
   const int e = isx ? sc.ex : sc.ey;
   if (lane == 0) const_cast<double*>(sd.nx)[row] = q;
 #pragma unroll
